@@ -129,8 +129,8 @@ size_t rl_workspace_size(int64_t max_rows, int64_t V, int64_t D);
 size_t rl_fused_head_workspace_size(int64_t T, int64_t V, int64_t D, int64_t group_tokens);
 
 /* Zero the workspace's 256-byte header: the status word and the finished-block
- * counters of the policy and value losses (which each launch leaves at zero
- * again). Call once after allocating a workspace, and again to clear a reported
+ * counters of the policy and value losses and the statistics summary (which each
+ * launch leaves at zero again). Call once after allocating a workspace, and again to clear a reported
  * device error. */
 rl_status rl_workspace_init(void* ws, size_t ws_bytes, rl_stream_t stream);
 
@@ -308,9 +308,10 @@ rl_status rl_fused_head_loss_fwd_bwd(const void* hidden, const void* weight, int
  *   rows, token_stats  float [rows x 5]
  *   mask, token_traj, n_traj, coef   as for rl_policy_loss_fwd_bwd
  *   summary_accum      double [5] on the device
- *   ws, ws_bytes       rl_workspace_size(0, 0, 0) bytes suffice (status word)
- * One launch of one 8-CTA cluster, a fixed assignment of rows to threads and a fixed order of
- * the partial sums, in double precision: deterministic.
+ *   ws, ws_bytes       rl_workspace_size(0, 0, 0) bytes suffice (the header: status word, a
+ *                      finished-cluster counter and the clusters' totals)
+ * One launch of one to five 16-CTA clusters, a fixed assignment of rows to threads and a fixed
+ * order of the partial sums, in double precision: deterministic.
  */
 rl_status rl_token_stats_summary(int64_t rows, const float* token_stats, const uint8_t* mask,
                                  const int32_t* token_traj, int32_t n_traj, const float* coef,

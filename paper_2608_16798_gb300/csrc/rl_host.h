@@ -26,6 +26,10 @@ constexpr size_t kWsDoneOffset = 16;
 constexpr size_t kWsValueDoneOffset = 20;
 // Work-item counter of the fused head's backward products (zeroed before each launch).
 constexpr size_t kWsHeadCounterOffset = 24;
+// The statistics summary's finished clusters, and its clusters' totals (5 doubles each, to the
+// header's end).
+constexpr size_t kWsSummaryDoneOffset = 28;
+constexpr size_t kWsSummaryOffset = 32;
 
 rl_status set_error(rl_status st, const std::string& msg);
 rl_status cuda_error(cudaError_t e, const char* what);
