@@ -105,16 +105,25 @@ def _check(fn, st):
 
 
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
+
+
+# The library's stream argument: the raw handle of torch's current stream on the current device
+# (no Stream object is built for it).
+_current_device = torch._C._cuda_getDevice if hasattr(torch._C, "_cuda_getDevice") else None
+_current_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _stream(stream):
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    if _current_stream is None or _current_device is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _current_stream(_current_device())
 
 
-def _need(t, name, dtype, numel=None, device=None):
+def _refuse(t, name, dtype, numel, index):
+    """The reason why _need did not take `t`."""
     if t is None:
         raise ValueError(f"{name} is required")
     if not t.is_cuda:
@@ -123,15 +132,23 @@ def _need(t, name, dtype, numel=None, device=None):
         raise ValueError(f"{name} must be {dtype}, got {t.dtype}")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
-    if numel is not None and t.numel() < numel:
+    if t.numel() < numel:
         raise ValueError(f"{name} has {t.numel()} elements, needs {numel}")
-    if device is not None and t.device != device:
-        raise ValueError(f"{name} is on {t.device}, expected {device}")
-    return t
+    raise ValueError(f"{name} is on {t.device}, expected {'cpu' if index < 0 else f'cuda:{index}'}")
 
 
-def _opt(t, name, dtype, numel=None, device=None):
-    return None if t is None else _need(t, name, dtype, numel, device)
+def _need(t, name, dtype, numel=0, index=None):
+    """Device pointer of a contiguous CUDA tensor of this type, of at least `numel` elements, on
+    device `index` (any, if None). A call checks about ten tensors, so the checks are one
+    expression on the cheapest queries; the reason for a refusal is worked out afterwards."""
+    if t is not None and t.dtype is dtype and t.is_cuda and t.numel() >= numel and t.is_contiguous() and \
+            (index is None or t.get_device() == index):
+        return t.data_ptr()
+    return _refuse(t, name, dtype, numel, index)
+
+
+def _opt(t, name, dtype, numel=0, index=None):
+    return None if t is None else _need(t, name, dtype, numel, index)
 
 
 def _logits_dtype(t):
@@ -168,17 +185,17 @@ def rl_fused_head_workspace_size(T: int, V: int, D: int, group_tokens: int) -> i
 
 
 def rl_workspace_init(ws: torch.Tensor, stream=None):
-    _need(ws, "ws", torch.uint8)
-    _check("rl_workspace_init", lib().rl_workspace_init(_ptr(ws), ws.numel(), _stream(stream)))
+    p_ws = _need(ws, "ws", torch.uint8)
+    _check("rl_workspace_init", lib().rl_workspace_init(p_ws, ws.numel(), _stream(stream)))
 
 
 def rl_selftest_bounded_wait(ws: torch.Tensor, limit_ns: int, waited_ns: torch.Tensor | None = None, stream=None):
     """Run one bounded wait that runs out (the failure path of every kernel wait); afterwards
     rl_query_status reports RL_ERR_TIMEOUT. waited_ns: optional int64 [1] on the device."""
-    _need(ws, "ws", torch.uint8)
-    _opt(waited_ns, "waited_ns", torch.int64, 1, device=ws.device)
+    p_ws = _need(ws, "ws", torch.uint8)
+    p_waited_ns = _opt(waited_ns, "waited_ns", torch.int64, 1, index=ws.get_device())
     _check("rl_selftest_bounded_wait",
-           lib().rl_selftest_bounded_wait(_ptr(ws), ws.numel(), int(limit_ns), _ptr(waited_ns), _stream(stream)))
+           lib().rl_selftest_bounded_wait(p_ws, ws.numel(), int(limit_ns), p_waited_ns, _stream(stream)))
 
 
 def new_workspace(max_rows: int, V: int, D: int = 0, device=None, stream=None, group_tokens: int = 0) -> torch.Tensor:
@@ -205,27 +222,28 @@ def rl_group_advantages(group_offsets, rewards, traj_offsets, mask, params: rl_l
                         want_token_traj=True, stream=None):
     """Advantages A_i, coefficients c_i, counts L_i (and token owners) for a packed batch."""
     dev = rewards.device
+    ix = rewards.get_device()
     n_traj = rewards.numel()
     n_groups = group_offsets.numel() - 1
     n_tokens = mask.numel()
-    _need(rewards, "rewards", torch.float32, device=dev)
-    _need(group_offsets, "group_offsets", torch.int32, device=dev)
-    _need(traj_offsets, "traj_offsets", torch.int64, n_traj + 1, device=dev)
-    _need(mask, "mask", torch.uint8, device=dev)
-    _opt(traj_valid, "traj_valid", torch.uint8, n_traj, device=dev)
+    p_rewards = _need(rewards, "rewards", torch.float32, index=ix)
+    p_group_offsets = _need(group_offsets, "group_offsets", torch.int32, index=ix)
+    p_traj_offsets = _need(traj_offsets, "traj_offsets", torch.int64, n_traj + 1, index=ix)
+    p_mask = _need(mask, "mask", torch.uint8, index=ix)
+    p_traj_valid = _opt(traj_valid, "traj_valid", torch.uint8, n_traj, index=ix)
     adv_out = torch.empty(n_traj, dtype=torch.float32, device=dev) if adv_out is None else adv_out
     coef_out = torch.empty(n_traj, dtype=torch.float32, device=dev) if coef_out is None else coef_out
     n_tok_out = torch.empty(n_traj, dtype=torch.int32, device=dev) if n_tok_out is None else n_tok_out
     if want_token_traj and token_traj_out is None:
         token_traj_out = torch.empty(n_tokens, dtype=torch.int32, device=dev)
-    _need(adv_out, "adv_out", torch.float32, n_traj, device=dev)
-    _need(coef_out, "coef_out", torch.float32, n_traj, device=dev)
-    _need(n_tok_out, "n_tok_out", torch.int32, n_traj, device=dev)
-    _opt(token_traj_out, "token_traj_out", torch.int32, n_tokens, device=dev)
-    _need(ws, "ws", torch.uint8, device=dev)
-    st = lib().rl_group_advantages(n_traj, n_groups, _ptr(group_offsets), _ptr(rewards), _ptr(traj_valid),
-                                   n_tokens, _ptr(traj_offsets), _ptr(mask), ctypes.byref(params), _ptr(adv_out),
-                                   _ptr(coef_out), _ptr(n_tok_out), _ptr(token_traj_out), _ptr(ws), ws.numel(),
+    p_adv_out = _need(adv_out, "adv_out", torch.float32, n_traj, index=ix)
+    p_coef_out = _need(coef_out, "coef_out", torch.float32, n_traj, index=ix)
+    p_n_tok_out = _need(n_tok_out, "n_tok_out", torch.int32, n_traj, index=ix)
+    p_token_traj_out = _opt(token_traj_out, "token_traj_out", torch.int32, n_tokens, index=ix)
+    p_ws = _need(ws, "ws", torch.uint8, index=ix)
+    st = lib().rl_group_advantages(n_traj, n_groups, p_group_offsets, p_rewards, p_traj_valid,
+                                   n_tokens, p_traj_offsets, p_mask, ctypes.byref(params), p_adv_out,
+                                   p_coef_out, p_n_tok_out, p_token_traj_out, p_ws, ws.numel(),
                                    _stream(stream))
     _check("rl_group_advantages", st)
     return adv_out, coef_out, n_tok_out, token_traj_out
@@ -237,18 +255,19 @@ def rl_token_logprobs(logits, token_ids, ws, logp_out=None, entropy_out=None, ls
     rows, V, ld = _rows_view(logits)
     dt = _logits_dtype(logits)
     dev = logits.device
-    _need(token_ids, "token_ids", torch.int32, rows, device=dev)
+    ix = logits.get_device()
+    p_token_ids = _need(token_ids, "token_ids", torch.int32, rows, index=ix)
     logp_out = torch.empty(rows, dtype=torch.float32, device=dev) if logp_out is None else logp_out
     if want_entropy and entropy_out is None:
         entropy_out = torch.empty(rows, dtype=torch.float32, device=dev)
     if want_lse and lse_out is None:
         lse_out = torch.empty(rows, dtype=torch.float32, device=dev)
-    _need(logp_out, "logp_out", torch.float32, rows, device=dev)
-    _opt(entropy_out, "entropy_out", torch.float32, rows, device=dev)
-    _opt(lse_out, "lse_out", torch.float32, rows, device=dev)
-    _need(ws, "ws", torch.uint8, device=dev)
-    st = lib().rl_token_logprobs(_ptr(logits), dt, rows, V, ld, _ptr(token_ids), _ptr(logp_out), _ptr(entropy_out),
-                                 _ptr(lse_out), _ptr(ws), ws.numel(), _stream(stream))
+    p_logp_out = _need(logp_out, "logp_out", torch.float32, rows, index=ix)
+    p_entropy_out = _opt(entropy_out, "entropy_out", torch.float32, rows, index=ix)
+    p_lse_out = _opt(lse_out, "lse_out", torch.float32, rows, index=ix)
+    p_ws = _need(ws, "ws", torch.uint8, index=ix)
+    st = lib().rl_token_logprobs(_ptr(logits), dt, rows, V, ld, p_token_ids, p_logp_out, p_entropy_out,
+                                 p_lse_out, p_ws, ws.numel(), _stream(stream))
     _check("rl_token_logprobs", st)
     return logp_out, entropy_out, lse_out
 
@@ -264,26 +283,27 @@ def rl_policy_loss_fwd_bwd(logits, token_ids, mask, token_traj, adv, coef, old_l
     rows, V, ld = _rows_view(logits)
     dt = _logits_dtype(logits)
     dev = logits.device
+    ix = logits.get_device()
     n_traj = coef.numel()
-    _need(token_ids, "token_ids", torch.int32, rows, device=dev)
-    _need(mask, "mask", torch.uint8, rows, device=dev)
-    _need(token_traj, "token_traj", torch.int32, rows, device=dev)
-    _need(coef, "coef", torch.float32, n_traj, device=dev)
-    _need(adv, "adv", torch.float32, rows if params.token_level_adv else n_traj, device=dev)
-    _need(old_logp, "old_logp", torch.float32, rows, device=dev)
-    _opt(ref_logp, "ref_logp", torch.float32, rows, device=dev)
-    _opt(rollout_logp, "rollout_logp", torch.float32, rows, device=dev)
-    _need(loss_accum, "loss_accum", torch.float64, 1, device=dev)
-    _opt(token_stats, "token_stats", torch.float32, rows * 5, device=dev)
+    p_token_ids = _need(token_ids, "token_ids", torch.int32, rows, index=ix)
+    p_mask = _need(mask, "mask", torch.uint8, rows, index=ix)
+    p_token_traj = _need(token_traj, "token_traj", torch.int32, rows, index=ix)
+    p_coef = _need(coef, "coef", torch.float32, n_traj, index=ix)
+    p_adv = _need(adv, "adv", torch.float32, rows if params.token_level_adv else n_traj, index=ix)
+    p_old_logp = _need(old_logp, "old_logp", torch.float32, rows, index=ix)
+    p_ref_logp = _opt(ref_logp, "ref_logp", torch.float32, rows, index=ix)
+    p_rollout_logp = _opt(rollout_logp, "rollout_logp", torch.float32, rows, index=ix)
+    p_loss_accum = _need(loss_accum, "loss_accum", torch.float64, 1, index=ix)
+    p_token_stats = _opt(token_stats, "token_stats", torch.float32, rows * 5, index=ix)
     if grad_out is None:
         grad_out = torch.empty_strided(logits.shape, logits.stride(), dtype=logits.dtype, device=dev)
     if grad_out.dtype != logits.dtype or grad_out.shape != logits.shape or grad_out.stride() != logits.stride():
         raise ValueError("grad_out must match logits in dtype, shape and strides")
-    _need(ws, "ws", torch.uint8, device=dev)
-    st = lib().rl_policy_loss_fwd_bwd(_ptr(logits), dt, rows, V, ld, _ptr(token_ids), _ptr(mask), _ptr(token_traj),
-                                      n_traj, _ptr(adv), _ptr(coef), _ptr(old_logp), _ptr(ref_logp),
-                                      _ptr(rollout_logp), ctypes.byref(params), _ptr(grad_out), _ptr(loss_accum),
-                                      _ptr(token_stats), _ptr(ws), ws.numel(), _stream(stream))
+    p_ws = _need(ws, "ws", torch.uint8, index=ix)
+    st = lib().rl_policy_loss_fwd_bwd(_ptr(logits), dt, rows, V, ld, p_token_ids, p_mask, p_token_traj,
+                                      n_traj, p_adv, p_coef, p_old_logp, p_ref_logp,
+                                      p_rollout_logp, ctypes.byref(params), _ptr(grad_out), p_loss_accum,
+                                      p_token_stats, p_ws, ws.numel(), _stream(stream))
     _check("rl_policy_loss_fwd_bwd", st)
     return grad_out
 
@@ -299,26 +319,27 @@ def rl_policy_loss_fwd_bwd_noalloc(logits, token_ids, mask, token_traj, adv, coe
     rows, V, ld = _rows_view(logits)
     dt = _logits_dtype(logits)
     dev = logits.device
+    ix = logits.get_device()
     n_traj = coef.numel()
-    _need(token_ids, "token_ids", torch.int32, rows, device=dev)
-    _need(mask, "mask", torch.uint8, rows, device=dev)
-    _need(token_traj, "token_traj", torch.int32, rows, device=dev)
-    _need(coef, "coef", torch.float32, n_traj, device=dev)
-    _need(adv, "adv", torch.float32, rows if params.token_level_adv else n_traj, device=dev)
-    _need(old_logp, "old_logp", torch.float32, rows, device=dev)
-    _opt(ref_logp, "ref_logp", torch.float32, rows, device=dev)
-    _opt(rollout_logp, "rollout_logp", torch.float32, rows, device=dev)
-    _need(loss_accum, "loss_accum", torch.float64, 1, device=dev)
-    _opt(token_stats, "token_stats", torch.float32, rows * 5, device=dev)
-    _opt(device_status, "device_status", torch.int32, 1, device=dev)
+    p_token_ids = _need(token_ids, "token_ids", torch.int32, rows, index=ix)
+    p_mask = _need(mask, "mask", torch.uint8, rows, index=ix)
+    p_token_traj = _need(token_traj, "token_traj", torch.int32, rows, index=ix)
+    p_coef = _need(coef, "coef", torch.float32, n_traj, index=ix)
+    p_adv = _need(adv, "adv", torch.float32, rows if params.token_level_adv else n_traj, index=ix)
+    p_old_logp = _need(old_logp, "old_logp", torch.float32, rows, index=ix)
+    p_ref_logp = _opt(ref_logp, "ref_logp", torch.float32, rows, index=ix)
+    p_rollout_logp = _opt(rollout_logp, "rollout_logp", torch.float32, rows, index=ix)
+    p_loss_accum = _need(loss_accum, "loss_accum", torch.float64, 1, index=ix)
+    p_token_stats = _opt(token_stats, "token_stats", torch.float32, rows * 5, index=ix)
+    p_device_status = _opt(device_status, "device_status", torch.int32, 1, index=ix)
     if grad_out is None or grad_out.dtype != logits.dtype or grad_out.shape != logits.shape or \
             grad_out.stride() != logits.stride():
         raise ValueError("grad_out must be given and match logits in dtype, shape and strides")
-    st = lib().rl_policy_loss_fwd_bwd_noalloc(_ptr(logits), dt, rows, V, ld, _ptr(token_ids), _ptr(mask),
-                                              _ptr(token_traj), n_traj, _ptr(adv), _ptr(coef), _ptr(old_logp),
-                                              _ptr(ref_logp), _ptr(rollout_logp), ctypes.byref(params),
-                                              _ptr(grad_out), _ptr(loss_accum), _ptr(token_stats),
-                                              _ptr(device_status), _stream(stream))
+    st = lib().rl_policy_loss_fwd_bwd_noalloc(_ptr(logits), dt, rows, V, ld, p_token_ids, p_mask,
+                                              p_token_traj, n_traj, p_adv, p_coef, p_old_logp,
+                                              p_ref_logp, p_rollout_logp, ctypes.byref(params),
+                                              _ptr(grad_out), p_loss_accum, p_token_stats,
+                                              p_device_status, _stream(stream))
     _check("rl_policy_loss_fwd_bwd_noalloc", st)
     return grad_out
 
@@ -334,29 +355,30 @@ def rl_fused_head_loss_fwd_bwd(hidden, weight, token_ids, mask, token_traj, adv,
     T, D = hidden.shape
     V = weight.shape[0]
     dev = hidden.device
+    ix = hidden.get_device()
     n_traj = coef.numel()
-    _need(hidden, "hidden", torch.bfloat16, device=dev)
-    _need(weight, "weight", torch.bfloat16, device=dev)
-    _need(token_ids, "token_ids", torch.int32, T, device=dev)
-    _need(mask, "mask", torch.uint8, T, device=dev)
-    _need(token_traj, "token_traj", torch.int32, T, device=dev)
-    _need(coef, "coef", torch.float32, n_traj, device=dev)
-    _need(adv, "adv", torch.float32, T if params.token_level_adv else n_traj, device=dev)
-    _need(old_logp, "old_logp", torch.float32, T, device=dev)
-    _opt(ref_logp, "ref_logp", torch.float32, T, device=dev)
-    _opt(rollout_logp, "rollout_logp", torch.float32, T, device=dev)
-    _need(loss_accum, "loss_accum", torch.float64, 1, device=dev)
-    _opt(token_stats, "token_stats", torch.float32, T * 5, device=dev)
-    _need(d_weight, "d_weight", torch.float32, V * D, device=dev)
+    p_hidden = _need(hidden, "hidden", torch.bfloat16, index=ix)
+    p_weight = _need(weight, "weight", torch.bfloat16, index=ix)
+    p_token_ids = _need(token_ids, "token_ids", torch.int32, T, index=ix)
+    p_mask = _need(mask, "mask", torch.uint8, T, index=ix)
+    p_token_traj = _need(token_traj, "token_traj", torch.int32, T, index=ix)
+    p_coef = _need(coef, "coef", torch.float32, n_traj, index=ix)
+    p_adv = _need(adv, "adv", torch.float32, T if params.token_level_adv else n_traj, index=ix)
+    p_old_logp = _need(old_logp, "old_logp", torch.float32, T, index=ix)
+    p_ref_logp = _opt(ref_logp, "ref_logp", torch.float32, T, index=ix)
+    p_rollout_logp = _opt(rollout_logp, "rollout_logp", torch.float32, T, index=ix)
+    p_loss_accum = _need(loss_accum, "loss_accum", torch.float64, 1, index=ix)
+    p_token_stats = _opt(token_stats, "token_stats", torch.float32, T * 5, index=ix)
+    p_d_weight = _need(d_weight, "d_weight", torch.float32, V * D, index=ix)
     if d_hidden is None:
         d_hidden = torch.empty((T, D), dtype=d_hidden_dtype, device=dev)
-    _need(d_hidden, "d_hidden", d_hidden.dtype, T * D, device=dev)
+    p_d_hidden = _need(d_hidden, "d_hidden", d_hidden.dtype, T * D, index=ix)
     dt = _logits_dtype(d_hidden)
-    _need(ws, "ws", torch.uint8, device=dev)
-    st = lib().rl_fused_head_loss_fwd_bwd(_ptr(hidden), _ptr(weight), T, D, V, _ptr(token_ids), _ptr(mask),
-                                          _ptr(token_traj), n_traj, _ptr(adv), _ptr(coef), _ptr(old_logp),
-                                          _ptr(ref_logp), _ptr(rollout_logp), ctypes.byref(params), _ptr(d_hidden),
-                                          dt, _ptr(d_weight), _ptr(loss_accum), _ptr(token_stats), _ptr(ws),
+    p_ws = _need(ws, "ws", torch.uint8, index=ix)
+    st = lib().rl_fused_head_loss_fwd_bwd(p_hidden, p_weight, T, D, V, p_token_ids, p_mask,
+                                          p_token_traj, n_traj, p_adv, p_coef, p_old_logp,
+                                          p_ref_logp, p_rollout_logp, ctypes.byref(params), p_d_hidden,
+                                          dt, p_d_weight, p_loss_accum, p_token_stats, p_ws,
                                           ws.numel(), _stream(stream))
     _check("rl_fused_head_loss_fwd_bwd", st)
     return d_hidden
@@ -371,20 +393,21 @@ def rl_fused_head_token_logprobs(hidden, weight, token_ids, ws, logp_out=None, e
     T, D = hidden.shape
     V = weight.shape[0]
     dev = hidden.device
-    _need(hidden, "hidden", torch.bfloat16, device=dev)
-    _need(weight, "weight", torch.bfloat16, device=dev)
-    _need(token_ids, "token_ids", torch.int32, T, device=dev)
+    ix = hidden.get_device()
+    p_hidden = _need(hidden, "hidden", torch.bfloat16, index=ix)
+    p_weight = _need(weight, "weight", torch.bfloat16, index=ix)
+    p_token_ids = _need(token_ids, "token_ids", torch.int32, T, index=ix)
     logp_out = torch.empty(T, dtype=torch.float32, device=dev) if logp_out is None else logp_out
     if want_entropy and entropy_out is None:
         entropy_out = torch.empty(T, dtype=torch.float32, device=dev)
     if want_lse and lse_out is None:
         lse_out = torch.empty(T, dtype=torch.float32, device=dev)
-    _need(logp_out, "logp_out", torch.float32, T, device=dev)
-    _opt(entropy_out, "entropy_out", torch.float32, T, device=dev)
-    _opt(lse_out, "lse_out", torch.float32, T, device=dev)
-    _need(ws, "ws", torch.uint8, device=dev)
-    st = lib().rl_fused_head_token_logprobs(_ptr(hidden), _ptr(weight), T, D, V, _ptr(token_ids), _ptr(logp_out),
-                                            _ptr(entropy_out), _ptr(lse_out), _ptr(ws), ws.numel(), _stream(stream))
+    p_logp_out = _need(logp_out, "logp_out", torch.float32, T, index=ix)
+    p_entropy_out = _opt(entropy_out, "entropy_out", torch.float32, T, index=ix)
+    p_lse_out = _opt(lse_out, "lse_out", torch.float32, T, index=ix)
+    p_ws = _need(ws, "ws", torch.uint8, index=ix)
+    st = lib().rl_fused_head_token_logprobs(p_hidden, p_weight, T, D, V, p_token_ids, p_logp_out,
+                                            p_entropy_out, p_lse_out, p_ws, ws.numel(), _stream(stream))
     _check("rl_fused_head_token_logprobs", st)
     return logp_out, entropy_out, lse_out
 
@@ -396,20 +419,21 @@ def rl_masked_gae(traj_offsets, mask, values, ws, gamma=1.0, gae_lambda=1.0, ski
     n_traj = traj_offsets.numel() - 1
     T = mask.numel()
     dev = mask.device
-    _need(traj_offsets, "traj_offsets", torch.int64, n_traj + 1, device=dev)
-    _need(mask, "mask", torch.uint8, T, device=dev)
-    _need(values, "values", torch.float32, T, device=dev)
-    _opt(token_rewards, "token_rewards", torch.float32, T, device=dev)
-    _opt(traj_rewards, "traj_rewards", torch.float32, n_traj, device=dev)
+    ix = mask.get_device()
+    p_traj_offsets = _need(traj_offsets, "traj_offsets", torch.int64, n_traj + 1, index=ix)
+    p_mask = _need(mask, "mask", torch.uint8, T, index=ix)
+    p_values = _need(values, "values", torch.float32, T, index=ix)
+    p_token_rewards = _opt(token_rewards, "token_rewards", torch.float32, T, index=ix)
+    p_traj_rewards = _opt(traj_rewards, "traj_rewards", torch.float32, n_traj, index=ix)
     adv_out = torch.empty(T, dtype=torch.float32, device=dev) if adv_out is None else adv_out
     if want_returns and returns_out is None:
         returns_out = torch.empty(T, dtype=torch.float32, device=dev)
-    _need(adv_out, "adv_out", torch.float32, T, device=dev)
-    _opt(returns_out, "returns_out", torch.float32, T, device=dev)
-    _need(ws, "ws", torch.uint8, device=dev)
-    st = lib().rl_masked_gae(n_traj, _ptr(traj_offsets), T, _ptr(mask), _ptr(values), _ptr(token_rewards),
-                             _ptr(traj_rewards), float(gamma), float(gae_lambda), 1 if skip_masked else 0,
-                             _ptr(adv_out), _ptr(returns_out), _ptr(ws), ws.numel(), _stream(stream))
+    p_adv_out = _need(adv_out, "adv_out", torch.float32, T, index=ix)
+    p_returns_out = _opt(returns_out, "returns_out", torch.float32, T, index=ix)
+    p_ws = _need(ws, "ws", torch.uint8, index=ix)
+    st = lib().rl_masked_gae(n_traj, p_traj_offsets, T, p_mask, p_values, p_token_rewards,
+                             p_traj_rewards, float(gamma), float(gae_lambda), 1 if skip_masked else 0,
+                             p_adv_out, p_returns_out, p_ws, ws.numel(), _stream(stream))
     _check("rl_masked_gae", st)
     return adv_out, returns_out
 
@@ -418,18 +442,19 @@ def rl_value_loss_fwd_bwd(values, returns, mask, token_traj, coef, ws, loss_accu
     """Adds sum_t c M (V - G)^2 to ``loss_accum`` (float64 [1]); returns d loss / d values (float32)."""
     rows = values.numel()
     dev = values.device
+    ix = values.get_device()
     n_traj = coef.numel()
-    _need(values, "values", torch.float32, rows, device=dev)
-    _need(returns, "returns", torch.float32, rows, device=dev)
-    _need(mask, "mask", torch.uint8, rows, device=dev)
-    _need(token_traj, "token_traj", torch.int32, rows, device=dev)
-    _need(coef, "coef", torch.float32, n_traj, device=dev)
-    _need(loss_accum, "loss_accum", torch.float64, 1, device=dev)
+    p_values = _need(values, "values", torch.float32, rows, index=ix)
+    p_returns = _need(returns, "returns", torch.float32, rows, index=ix)
+    p_mask = _need(mask, "mask", torch.uint8, rows, index=ix)
+    p_token_traj = _need(token_traj, "token_traj", torch.int32, rows, index=ix)
+    p_coef = _need(coef, "coef", torch.float32, n_traj, index=ix)
+    p_loss_accum = _need(loss_accum, "loss_accum", torch.float64, 1, index=ix)
     d_values = torch.empty(rows, dtype=torch.float32, device=dev) if d_values is None else d_values
-    _need(d_values, "d_values", torch.float32, rows, device=dev)
-    _need(ws, "ws", torch.uint8, device=dev)
-    st = lib().rl_value_loss_fwd_bwd(rows, _ptr(values), _ptr(returns), _ptr(mask), _ptr(token_traj), n_traj,
-                                     _ptr(coef), _ptr(d_values), _ptr(loss_accum), _ptr(ws), ws.numel(),
+    p_d_values = _need(d_values, "d_values", torch.float32, rows, index=ix)
+    p_ws = _need(ws, "ws", torch.uint8, index=ix)
+    st = lib().rl_value_loss_fwd_bwd(rows, p_values, p_returns, p_mask, p_token_traj, n_traj,
+                                     p_coef, p_d_values, p_loss_accum, p_ws, ws.numel(),
                                      _stream(stream))
     _check("rl_value_loss_fwd_bwd", st)
     return d_values
@@ -443,21 +468,22 @@ def rl_sequence_is_weights(token_traj, mask, old_logp, rollout_logp, n_traj, ws,
     (weight, log_ratio)."""
     T = mask.numel()
     dev = mask.device
-    _need(token_traj, "token_traj", torch.int32, T, device=dev)
-    _need(mask, "mask", torch.uint8, T, device=dev)
-    _need(old_logp, "old_logp", torch.float32, T, device=dev)
-    _need(rollout_logp, "rollout_logp", torch.float32, T, device=dev)
+    ix = mask.get_device()
+    p_token_traj = _need(token_traj, "token_traj", torch.int32, T, index=ix)
+    p_mask = _need(mask, "mask", torch.uint8, T, index=ix)
+    p_old_logp = _need(old_logp, "old_logp", torch.float32, T, index=ix)
+    p_rollout_logp = _need(rollout_logp, "rollout_logp", torch.float32, T, index=ix)
     weight_out = torch.empty(n_traj, dtype=torch.float32, device=dev) if weight_out is None else weight_out
     if want_log_ratio and log_ratio_out is None:
         log_ratio_out = torch.empty(n_traj, dtype=torch.float32, device=dev)
-    _need(weight_out, "weight_out", torch.float32, n_traj, device=dev)
-    _opt(log_ratio_out, "log_ratio_out", torch.float32, n_traj, device=dev)
-    _opt(traj_adv_inout, "traj_adv_inout", torch.float32, n_traj, device=dev)
-    _opt(token_adv_inout, "token_adv_inout", torch.float32, T, device=dev)
-    _need(ws, "ws", torch.uint8, device=dev)
-    st = lib().rl_sequence_is_weights(n_traj, T, _ptr(token_traj), _ptr(mask), _ptr(old_logp), _ptr(rollout_logp),
-                                      float(cap), _ptr(weight_out), _ptr(log_ratio_out), _ptr(traj_adv_inout),
-                                      _ptr(token_adv_inout), _ptr(ws), ws.numel(), _stream(stream))
+    p_weight_out = _need(weight_out, "weight_out", torch.float32, n_traj, index=ix)
+    p_log_ratio_out = _opt(log_ratio_out, "log_ratio_out", torch.float32, n_traj, index=ix)
+    p_traj_adv_inout = _opt(traj_adv_inout, "traj_adv_inout", torch.float32, n_traj, index=ix)
+    p_token_adv_inout = _opt(token_adv_inout, "token_adv_inout", torch.float32, T, index=ix)
+    p_ws = _need(ws, "ws", torch.uint8, index=ix)
+    st = lib().rl_sequence_is_weights(n_traj, T, p_token_traj, p_mask, p_old_logp, p_rollout_logp,
+                                      float(cap), p_weight_out, p_log_ratio_out, p_traj_adv_inout,
+                                      p_token_adv_inout, p_ws, ws.numel(), _stream(stream))
     _check("rl_sequence_is_weights", st)
     return weight_out, log_ratio_out
 
@@ -533,21 +559,22 @@ def rl_group_advantages_by_owner(group_offsets, rewards, token_traj, mask, param
     n_groups = group_offsets.numel() - 1
     T = mask.numel()
     dev = rewards.device
-    _need(group_offsets, "group_offsets", torch.int32, n_groups + 1, device=dev)
-    _need(rewards, "rewards", torch.float32, n_traj, device=dev)
-    _opt(traj_valid, "traj_valid", torch.uint8, n_traj, device=dev)
-    _need(token_traj, "token_traj", torch.int32, T, device=dev)
-    _need(mask, "mask", torch.uint8, T, device=dev)
+    ix = rewards.get_device()
+    p_group_offsets = _need(group_offsets, "group_offsets", torch.int32, n_groups + 1, index=ix)
+    p_rewards = _need(rewards, "rewards", torch.float32, n_traj, index=ix)
+    p_traj_valid = _opt(traj_valid, "traj_valid", torch.uint8, n_traj, index=ix)
+    p_token_traj = _need(token_traj, "token_traj", torch.int32, T, index=ix)
+    p_mask = _need(mask, "mask", torch.uint8, T, index=ix)
     adv_out = torch.empty(n_traj, dtype=torch.float32, device=dev) if adv_out is None else adv_out
     coef_out = torch.empty(n_traj, dtype=torch.float32, device=dev) if coef_out is None else coef_out
     n_tok_out = torch.empty(n_traj, dtype=torch.int32, device=dev) if n_tok_out is None else n_tok_out
-    _need(adv_out, "adv_out", torch.float32, n_traj, device=dev)
-    _need(coef_out, "coef_out", torch.float32, n_traj, device=dev)
-    _need(n_tok_out, "n_tok_out", torch.int32, n_traj, device=dev)
-    _need(ws, "ws", torch.uint8, device=dev)
-    st = lib().rl_group_advantages_by_owner(n_traj, n_groups, _ptr(group_offsets), _ptr(rewards), _ptr(traj_valid), T,
-                                            _ptr(token_traj), _ptr(mask), ctypes.byref(params), _ptr(adv_out),
-                                            _ptr(coef_out), _ptr(n_tok_out), _ptr(ws), ws.numel(), _stream(stream))
+    p_adv_out = _need(adv_out, "adv_out", torch.float32, n_traj, index=ix)
+    p_coef_out = _need(coef_out, "coef_out", torch.float32, n_traj, index=ix)
+    p_n_tok_out = _need(n_tok_out, "n_tok_out", torch.int32, n_traj, index=ix)
+    p_ws = _need(ws, "ws", torch.uint8, index=ix)
+    st = lib().rl_group_advantages_by_owner(n_traj, n_groups, p_group_offsets, p_rewards, p_traj_valid, T,
+                                            p_token_traj, p_mask, ctypes.byref(params), p_adv_out,
+                                            p_coef_out, p_n_tok_out, p_ws, ws.numel(), _stream(stream))
     _check("rl_group_advantages_by_owner", st)
     return adv_out, coef_out, n_tok_out
 
@@ -558,18 +585,19 @@ def rl_rollout_value_advantages(token_traj, mask, values, rewards, ws, adv_out=N
     T = mask.numel()
     n_traj = rewards.numel()
     dev = mask.device
-    _need(token_traj, "token_traj", torch.int32, T, device=dev)
-    _need(mask, "mask", torch.uint8, T, device=dev)
-    _need(values, "values", torch.float32, T, device=dev)
-    _need(rewards, "rewards", torch.float32, n_traj, device=dev)
+    ix = mask.get_device()
+    p_token_traj = _need(token_traj, "token_traj", torch.int32, T, index=ix)
+    p_mask = _need(mask, "mask", torch.uint8, T, index=ix)
+    p_values = _need(values, "values", torch.float32, T, index=ix)
+    p_rewards = _need(rewards, "rewards", torch.float32, n_traj, index=ix)
     adv_out = torch.empty(T, dtype=torch.float32, device=dev) if adv_out is None else adv_out
     if want_returns and returns_out is None:
         returns_out = torch.empty(T, dtype=torch.float32, device=dev)
-    _need(adv_out, "adv_out", torch.float32, T, device=dev)
-    _opt(returns_out, "returns_out", torch.float32, T, device=dev)
-    _need(ws, "ws", torch.uint8, device=dev)
-    st = lib().rl_rollout_value_advantages(T, _ptr(token_traj), _ptr(mask), _ptr(values), _ptr(rewards), n_traj,
-                                           _ptr(adv_out), _ptr(returns_out), _ptr(ws), ws.numel(), _stream(stream))
+    p_adv_out = _need(adv_out, "adv_out", torch.float32, T, index=ix)
+    p_returns_out = _opt(returns_out, "returns_out", torch.float32, T, index=ix)
+    p_ws = _need(ws, "ws", torch.uint8, index=ix)
+    st = lib().rl_rollout_value_advantages(T, p_token_traj, p_mask, p_values, p_rewards, n_traj,
+                                           p_adv_out, p_returns_out, p_ws, ws.numel(), _stream(stream))
     _check("rl_rollout_value_advantages", st)
     return adv_out, returns_out
 
@@ -580,15 +608,16 @@ def rl_token_stats_summary(token_stats, mask, token_traj, coef, ws, summary_accu
     rows = mask.numel()
     n_traj = coef.numel()
     dev = mask.device
-    _need(token_stats, "token_stats", torch.float32, rows * 5, device=dev)
-    _need(mask, "mask", torch.uint8, rows, device=dev)
-    _need(token_traj, "token_traj", torch.int32, rows, device=dev)
-    _need(coef, "coef", torch.float32, n_traj, device=dev)
+    ix = mask.get_device()
+    p_token_stats = _need(token_stats, "token_stats", torch.float32, rows * 5, index=ix)
+    p_mask = _need(mask, "mask", torch.uint8, rows, index=ix)
+    p_token_traj = _need(token_traj, "token_traj", torch.int32, rows, index=ix)
+    p_coef = _need(coef, "coef", torch.float32, n_traj, index=ix)
     if summary_accum is None:
         summary_accum = torch.zeros(5, dtype=torch.float64, device=dev)
-    _need(summary_accum, "summary_accum", torch.float64, 5, device=dev)
-    _need(ws, "ws", torch.uint8, device=dev)
-    st = lib().rl_token_stats_summary(rows, _ptr(token_stats), _ptr(mask), _ptr(token_traj), n_traj, _ptr(coef),
-                                      _ptr(summary_accum), _ptr(ws), ws.numel(), _stream(stream))
+    p_summary_accum = _need(summary_accum, "summary_accum", torch.float64, 5, index=ix)
+    p_ws = _need(ws, "ws", torch.uint8, index=ix)
+    st = lib().rl_token_stats_summary(rows, p_token_stats, p_mask, p_token_traj, n_traj, p_coef,
+                                      p_summary_accum, p_ws, ws.numel(), _stream(stream))
     _check("rl_token_stats_summary", st)
     return summary_accum
