@@ -1,11 +1,12 @@
 // PPO parts of the method (Sec. 2.3.1, Sec. 2.3.4): the masked generalised advantage
 // estimate over packed ragged trajectories and the masked value loss.
 //
-//   gae_kernel         one CTA per trajectory (grid-stride). The estimate is the backward
+//   gae_kernel         a warp per trajectory of up to kWarpTokens tokens, a CTA per longer one.
+//                      The estimate is the backward
 //                      affine recurrence x_t = a_t x_{t+1} + b_t inside the trajectory
 //                      (x past its end = 0), evaluated chunk by chunk from the end: each
-//                      thread composes its 4 tokens' maps, a block-wide suffix scan of the
-//                      composed maps gives every thread its entry value, and the chunk's
+//                      thread composes its 4 tokens' maps, a warp- or block-wide suffix scan of
+//                      the composed maps gives every thread its entry value, and the chunk's
 //                      first value carries into the next chunk down.
 //                        printed reading  a_t = gamma lambda,
 //                                         b_t = M_t (r_t + gamma M_{t+1} V_{t+1} - V_t)
@@ -14,6 +15,8 @@
 //                                         Vn_{t+1} the value of the next trainable token,
 //                                         itself the suffix scan of the selection map
 //                                         x_t = M_t ? V_t : x_{t+1} (exact in fp32)
+//                      R_i is added at the token with M_t = 1 that has no later one: the scan of
+//                      "is there a trainable token above" rides along.
 //   value_loss_kernel  per token: c M (V - G)^2, added per CTA in a fixed order into one
 //                      partial per CTA, and dV = 2 c M (V - G); the last CTA to finish adds
 //                      the partials, in a fixed order, into the caller's accumulator.
@@ -23,6 +26,7 @@
 //
 // Both touch a few bytes per token (mask, values, rewards, outputs) and are latency- or
 // launch-bound next to the logits stream.
+#include <algorithm>
 #include <cstdint>
 
 #include "rl_device.cuh"
@@ -33,7 +37,6 @@ namespace ppo {
 
 constexpr int kThreads = 256;
 constexpr int kPer = 4;                  // consecutive tokens per thread
-constexpr int kChunk = kThreads * kPer;  // tokens per block step
 constexpr int kWarps = kThreads / 32;
 
 // x -> a x + b
@@ -46,34 +49,11 @@ __device__ __forceinline__ Affine compose(Affine outer, Affine inner) {
   return Affine{outer.a * inner.a, fmaf(outer.a, inner.b, outer.b)};
 }
 
-// Every thread passes the composition of its own tokens' maps (`mine`, mapping the value
-// just above its tokens to the value at its first token) and the value above the whole
-// chunk (`top`, the same in every thread). Returns the value just above this thread's
-// tokens. `sh` holds kWarps maps.
-__device__ __forceinline__ float suffix_entry(Affine mine, float top, Affine* sh) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  // inclusive suffix within the warp: S_k = F_k o F_{k+1} o ... o F_31
-  Affine s = mine;
-#pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    const float oa = __shfl_down_sync(0xffffffffu, s.a, off);
-    const float ob = __shfl_down_sync(0xffffffffu, s.b, off);
-    if (lane + off < 32) s = compose(s, Affine{oa, ob});
-  }
-  if (lane == 0) sh[warp] = s;
-  __syncthreads();
-  // value above this warp: the later warps' totals applied to `top`, highest first
-  float above_warp = top;
-  for (int w = kWarps - 1; w > warp; --w) above_warp = fmaf(sh[w].a, above_warp, sh[w].b);
-  __syncthreads();  // sh is reused by the caller's next scan
-  // exclusive suffix within the warp: S_{k+1} applied to the warp's entry value
-  const float na = __shfl_down_sync(0xffffffffu, s.a, 1);
-  const float nb = __shfl_down_sync(0xffffffffu, s.b, 1);
-  return lane == 31 ? above_warp : fmaf(na, above_warp, nb);
-}
+constexpr int kWarpTokens = 512;  // longest trajectory one warp takes
 
 struct GaeArgs {
   int32_t n_traj;
+  int32_t per_cta;  // trajectories of a CTA (at most kWarps)
   const int64_t* offs;
   int64_t T;
   const uint8_t* mask;
@@ -87,100 +67,202 @@ struct GaeArgs {
   int32_t* status;
 };
 
-__global__ void __launch_bounds__(kThreads) gae_kernel(const GaeArgs p) {
-  __shared__ Affine sh[kWarps];
-  __shared__ int64_t sh_pos[kWarps];
-  __shared__ float sh_carry[2];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const float gl = p.gamma * p.lam;
-  for (int32_t i = blockIdx.x; i < p.n_traj; i += gridDim.x) {
-    const int64_t s = p.offs[i], e = p.offs[i + 1];
-    if (s < 0 || e < s || e > p.T) {
-      if (tid == 0) flag_status(p.status, RL_DEV_BAD_OFFSETS);
-      continue;  // uniform across the block
-    }
-    // last trainable token (for R_i), searched chunk by chunk from the end
-    int64_t last = -1;
-    if (p.traj_rewards) {
-      for (int64_t c1 = e; c1 > s && last < 0; c1 -= kChunk) {
-        const int64_t c0 = c1 - kChunk > s ? c1 - kChunk : s;
-        int64_t best = -1;
-        for (int j = 0; j < kPer; ++j) {
-          const int64_t t = c0 + tid * kPer + j;
-          if (t < c1 && p.mask[t] != 0) best = t;
-        }
+// The same scan for one warp (W = 1) or the whole CTA (W = kWarps). Every thread passes the
+// composition of its own tokens' maps (`mine`, mapping the value just above its tokens to the
+// value at its first token) and the value above the whole chunk (`top`, the same in every thread);
+// returns the value just above this thread's tokens, and in `low` (the same in every thread) the
+// value at the chunk's first token. `sh` holds kWarps maps; the caller alternates between two of
+// them, so one barrier per scan suffices.
+template <int W>
+__device__ __forceinline__ float suffix_entry(Affine mine, float top, Affine* sh, float& low) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // inclusive suffix within the warp: S_k = F_k o F_{k+1} o ... o F_31
+  Affine s = mine;
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-          const int64_t o = __shfl_down_sync(0xffffffffu, best, off);
-          best = o > best ? o : best;
-        }
-        if (lane == 0) sh_pos[warp] = best;
-        __syncthreads();
-        for (int w = 0; w < kWarps; ++w) last = sh_pos[w] > last ? sh_pos[w] : last;
-        __syncthreads();
-      }
+  for (int off = 1; off < 32; off <<= 1) {
+    const float oa = __shfl_down_sync(0xffffffffu, s.a, off);
+    const float ob = __shfl_down_sync(0xffffffffu, s.b, off);
+    if (lane + off < 32) s = compose(s, Affine{oa, ob});
+  }
+  // value above this warp: the later warps' totals applied to `top`, highest first
+  float above_warp = top;
+  if (W > 1) {
+    if (lane == 0) sh[warp] = s;
+    __syncthreads();
+    low = top;
+#pragma unroll
+    for (int w = W - 1; w >= 0; --w) {
+      if (w == warp) above_warp = low;
+      low = fmaf(sh[w].a, low, sh[w].b);
     }
-    const float Ri = (p.traj_rewards && last >= 0) ? p.traj_rewards[i] : 0.f;
+  } else {
+    low = fmaf(__shfl_sync(0xffffffffu, s.a, 0), top, __shfl_sync(0xffffffffu, s.b, 0));
+  }
+  // exclusive suffix within the warp: S_{k+1} applied to the warp's entry value
+  const float na = __shfl_down_sync(0xffffffffu, s.a, 1);
+  const float nb = __shfl_down_sync(0xffffffffu, s.b, 1);
+  return lane == 31 ? above_warp : fmaf(na, above_warp, nb);
+}
 
-    float carry_x = 0.f;   // recurrence value at the first position above the chunk
-    float carry_vn = 0.f;  // skip reading: value of the first trainable token above it
-    for (int64_t c1 = e; c1 > s; c1 -= kChunk) {
-      const int64_t c0 = c1 - kChunk > s ? c1 - kChunk : s;
-      const int64_t t0 = c0 + static_cast<int64_t>(tid) * kPer;
-      bool M[kPer];
-      float V[kPer], r[kPer], a[kPer], b[kPer];
+// One chunk's inputs of a thread (kPer consecutive tokens from t0), loaded a chunk ahead.
+struct GaeTokens {
+  bool M[kPer];
+  float V[kPer], r[kPer];
+};
+
+__device__ __forceinline__ GaeTokens load_tokens(const GaeArgs& p, int64_t t0, int64_t c1) {
+  GaeTokens x;
+  uint8_t m[kPer];
 #pragma unroll
-      for (int j = 0; j < kPer; ++j) {
-        const int64_t t = t0 + j;
-        const bool in = t < c1;
-        M[j] = in && p.mask[t] != 0;
-        V[j] = in ? p.values[t] : 0.f;
-        r[j] = (in && p.token_rewards) ? p.token_rewards[t] : 0.f;
-        if (t == last) r[j] += Ri;
-      }
-      if (p.skip) {
-        // Vn above each token: suffix scan of the selection maps
-        Affine f{1.f, 0.f};
+  for (int j = 0; j < kPer; ++j) {
+    const int64_t t = t0 + j;
+    const bool in = t < c1;
+    m[j] = in ? p.mask[t] : 0;
+    x.V[j] = in ? p.values[t] : 0.f;
+    x.r[j] = (in && p.token_rewards) ? p.token_rewards[t] : 0.f;
+  }
 #pragma unroll
-        for (int j = kPer - 1; j >= 0; --j) f = compose(M[j] ? Affine{0.f, V[j]} : Affine{1.f, 0.f}, f);
-        float vn = suffix_entry(f, carry_vn, sh);
+  for (int j = 0; j < kPer; ++j) x.M[j] = m[j] != 0;
+  return x;
+}
+
+// Trajectory [s, e) by one warp (W = 1) or the whole CTA (W = kWarps). Two barriers per chunk of
+// the CTA form (one per scan).
+template <int W>
+__device__ __forceinline__ void gae_trajectory(const GaeArgs& p, int32_t i, int64_t s, int64_t e, Affine (*sh)[kWarps],
+                                               uint32_t* sh_any) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int tid = W > 1 ? static_cast<int>(threadIdx.x) : lane;
+  constexpr int kStep = W * 32 * kPer;
+  const float gl = p.gamma * p.lam;
+  const float Ri = p.traj_rewards ? p.traj_rewards[i] : 0.f;
+  float carry_x = 0.f;    // recurrence value at the first position above the chunk
+  float carry_vn = 0.f;   // value of the first trainable token above it (skip reading) ...
+  float edge_vn = 0.f;    // ... or M V of the first token above it (printed reading)
+  bool seen = false;      // a trainable token lies above the chunk
+  GaeTokens cur = load_tokens(p, (e - kStep > s ? e - kStep : s) + static_cast<int64_t>(tid) * kPer, e), nxt;
+  for (int64_t c1 = e; c1 > s; c1 -= kStep) {
+    const int64_t c0 = c1 - kStep > s ? c1 - kStep : s;
+    const int64_t t0 = c0 + static_cast<int64_t>(tid) * kPer;
+    const int64_t n1 = c1 - kStep, n0 = n1 - kStep > s ? n1 - kStep : s;  // the next chunk down
+    nxt = cur;
+    if (n1 > s) nxt = load_tokens(p, n0 + static_cast<int64_t>(tid) * kPer, n1);
+    const GaeTokens& x = cur;
+    float a[kPer], b[kPer], r[kPer];
+    // ---- where R_i goes: the last trainable token of the trajectory, in the first chunk from
+    // the end that has one
+    bool any = false;
 #pragma unroll
-        for (int j = kPer - 1; j >= 0; --j) {
-          a[j] = M[j] ? gl : 1.f;
-          b[j] = M[j] ? (r[j] + fmaf(p.gamma, vn, -V[j])) : 0.f;
-          if (M[j]) vn = V[j];
-        }
-        if (tid == 0) sh_carry[1] = vn;  // the chunk's lowest token's selection value
-      } else {
+    for (int j = 0; j < kPer; ++j) any |= x.M[j];
+    const unsigned in_warp = __ballot_sync(0xffffffffu, any);
+    if (W > 1 && lane == 0) sh_any[warp] = in_warp;  // read after the next barrier
+    bool above = (in_warp >> lane) > 1u;             // a later lane of this warp has one
 #pragma unroll
-        for (int j = 0; j < kPer; ++j) {
-          const int64_t t = t0 + j;
-          float boot = 0.f;
-          if (t + 1 < e && p.mask[t + 1] != 0) boot = p.values[t + 1];
-          a[j] = gl;
-          b[j] = M[j] ? (r[j] + fmaf(p.gamma, boot, -V[j])) : 0.f;
-          if (t >= c1) { a[j] = 1.f; b[j] = 0.f; }  // past the chunk: identity
-        }
-      }
+    for (int j = 0; j < kPer; ++j) r[j] = x.r[j];
+    float vn = 0.f, low;
+    if (p.skip) {
+      // Vn above each token: suffix scan of the selection maps
       Affine f{1.f, 0.f};
 #pragma unroll
-      for (int j = kPer - 1; j >= 0; --j) f = compose(Affine{a[j], b[j]}, f);
-      float x = suffix_entry(f, carry_x, sh);
-#pragma unroll
-      for (int j = kPer - 1; j >= 0; --j) {
-        x = fmaf(a[j], x, b[j]);
-        const int64_t t = t0 + j;
-        if (t < c1) {
-          p.adv[t] = M[j] ? x : 0.f;
-          if (p.ret) p.ret[t] = M[j] ? x + V[j] : 0.f;
-        }
+      for (int j = kPer - 1; j >= 0; --j) f = compose(x.M[j] ? Affine{0.f, x.V[j]} : Affine{1.f, 0.f}, f);
+      vn = suffix_entry<W>(f, carry_vn, sh[0], low);
+      carry_vn = low;
+    } else {
+      // M V of the token above this thread's last one: the next lane's or warp's first, or, for the
+      // thread that holds the chunk's last token, the first of the chunk above
+      const float first = x.M[0] ? x.V[0] : 0.f;
+      const float edge = edge_vn;
+      vn = __shfl_down_sync(0xffffffffu, first, 1);
+      if (W > 1) {
+        if (lane == 0) sh[0][warp] = Affine{first, 0.f};
+        __syncthreads();
+        if (lane == 31 && warp + 1 < W) vn = sh[0][warp + 1].a;
+        edge_vn = sh[0][0].a;
+      } else {
+        edge_vn = __shfl_sync(0xffffffffu, first, 0);
       }
-      if (tid == 0) sh_carry[0] = x;
-      __syncthreads();
-      carry_x = sh_carry[0];
-      if (p.skip) carry_vn = sh_carry[1];
-      __syncthreads();
+      if (t0 + kPer >= c1) vn = edge;
     }
+    bool any_chunk = in_warp != 0u;
+    if (W > 1) {
+      any_chunk = false;
+#pragma unroll
+      for (int w = 0; w < W; ++w) {
+        const bool h = sh_any[w] != 0u;
+        any_chunk |= h;
+        above |= h && w > warp;
+      }
+    }
+    if (any && !above && !seen) {
+      bool put = false;
+#pragma unroll
+      for (int j = kPer - 1; j >= 0; --j)
+        if (x.M[j] && !put) {
+          r[j] += Ri;
+          put = true;
+        }
+    }
+    seen |= any_chunk;
+#pragma unroll
+    for (int j = kPer - 1; j >= 0; --j) {
+      if (p.skip) {
+        a[j] = x.M[j] ? gl : 1.f;
+        b[j] = x.M[j] ? (r[j] + fmaf(p.gamma, vn, -x.V[j])) : 0.f;
+        if (x.M[j]) vn = x.V[j];
+      } else {
+        const bool in = t0 + j < c1;  // past the chunk: identity
+        a[j] = in ? gl : 1.f;
+        b[j] = x.M[j] ? (r[j] + fmaf(p.gamma, vn, -x.V[j])) : 0.f;
+        if (in) vn = x.M[j] ? x.V[j] : 0.f;
+      }
+    }
+    Affine f{1.f, 0.f};
+#pragma unroll
+    for (int j = kPer - 1; j >= 0; --j) f = compose(Affine{a[j], b[j]}, f);
+    float y = suffix_entry<W>(f, carry_x, sh[1], low);
+    carry_x = low;
+#pragma unroll
+    for (int j = kPer - 1; j >= 0; --j) {
+      y = fmaf(a[j], y, b[j]);
+      const int64_t t = t0 + j;
+      if (t < c1) {
+        p.adv[t] = x.M[j] ? y : 0.f;
+        if (p.ret) p.ret[t] = x.M[j] ? y + x.V[j] : 0.f;
+      }
+    }
+    cur = nxt;
+  }
+}
+
+// Latency-bound: a chunk is a trip to memory (hidden behind the chunk before it) and two scans.
+// 16,384 trajectories of 8 tokens: 89 us with a CTA each, 13.7 us; 512 of 512 to 8,192: 23.8, 20.4.
+// A CTA takes p.per_cta neighbouring trajectories, each of at most kWarpTokens tokens by a warp of
+// its own, which meets no barrier; the longer ones are taken by the whole CTA afterwards.
+__global__ void __launch_bounds__(kThreads) gae_kernel(const GaeArgs p) {
+  __shared__ Affine sh[2][kWarps];
+  __shared__ uint32_t sh_any[kWarps];
+  __shared__ int64_t span[kWarps][2];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int64_t base = static_cast<int64_t>(blockIdx.x) * p.per_cta; base < p.n_traj;
+       base += static_cast<int64_t>(gridDim.x) * p.per_cta) {
+    const int here = static_cast<int>(min(static_cast<int64_t>(p.per_cta), p.n_traj - base));
+    if (warp < here) {
+      const int32_t i = static_cast<int32_t>(base) + warp;
+      const int64_t s = p.offs[i], e = p.offs[i + 1];
+      const bool bad = s < 0 || e < s || e > p.T;
+      if (bad && lane == 0) flag_status(p.status, RL_DEV_BAD_OFFSETS);
+      const bool longer = !bad && e - s > kWarpTokens;
+      if (lane == 0) {
+        span[warp][0] = s;
+        span[warp][1] = longer ? e : s;
+      }
+      if (!bad && !longer) gae_trajectory<1>(p, i, s, e, nullptr, nullptr);
+    }
+    __syncthreads();
+    for (int w = 0; w < here; ++w)
+      if (span[w][1] > span[w][0])
+        gae_trajectory<kWarps>(p, static_cast<int32_t>(base) + w, span[w][0], span[w][1], sh, sh_any);
+    __syncthreads();  // span is rewritten for the next trajectories
   }
 }
 
@@ -310,7 +392,10 @@ extern "C" rl_status rl_masked_gae(int32_t n_traj, const int64_t* traj_offsets, 
   a.ret = returns_out;
   a.status = reinterpret_cast<int32_t*>(ws);
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  ppo::gae_kernel<<<ppo::grid_for(n_traj, 1, 152 * 8), ppo::kThreads, 0, s>>>(a);
+  // a CTA (8 fit on an SM) per trajectory while they last, then up to a warp per trajectory
+  const int grid = ppo::grid_for(n_traj, 1, 152 * 8);
+  a.per_cta = std::min<int>(ppo::kWarps, (n_traj + grid - 1) / grid);
+  ppo::gae_kernel<<<ppo::grid_for(n_traj, a.per_cta, 152 * 8), ppo::kThreads, 0, s>>>(a);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_error(e, "gae_kernel launch");
   return RL_OK;
