@@ -1,14 +1,14 @@
 // Group-relative advantages and loss coefficients over ragged trajectories.
 //
 //   count_adv_kernel    one launch, two kinds of CTA: the first count L_i, the
-//                       trainable tokens of each trajectory (one warp per
-//                       trajectory span, writing token_traj[t] = i; or, by owner,
+//                       trainable tokens of each trajectory (a CTA or a warp
+//                       per trajectory span, writing token_traj[t] = i; or, by owner,
 //                       a grid-stride pass over tokens in any order), the 1 /
 //                       sum_t M_{i,t} normaliser of the masked GRPO objective
 //                       (Sec. 2.3.2); the others form A_i = (R_i - mu_g) /
-//                       (sigma_g + eps) per group (one warp per group: mean and
-//                       population standard deviation of the valid members'
-//                       rewards in double precision; Sec. 2.3.2 GRPO advantage,
+//                       (sigma_g + eps) per group (a segment of a warp per group:
+//                       mean and population standard deviation of the valid
+//                       members' rewards in double precision; Sec. 2.3.2 GRPO advantage,
 //                       Sec. 3.2.3; discarded rollouts leave the statistics and
 //                       get A = 0, Sec. 3.4). Counts and advantages do not depend
 //                       on each other.
@@ -31,26 +31,39 @@ namespace rl {
 constexpr int kAdvThreads = 256;
 constexpr int kAdvWarps = kAdvThreads / 32;
 
-// L_i over trajectory i's span [traj_offsets[i], traj_offsets[i + 1]) and the owner of each of
-// its tokens (one warp)
-__device__ __forceinline__ void count_span(int64_t i, int lane, int64_t n_tokens, const int64_t* traj_offsets,
-                                           const uint8_t* mask, int32_t* n_tok_out, int32_t* token_traj_out,
-                                           int32_t* status) {
-  const int64_t s = traj_offsets[i], e = traj_offsets[i + 1];
-  if (s < 0 || e < s || e > n_tokens) {
-    if (lane == 0) {
-      flag_status(status, RL_DEV_BAD_OFFSETS);
-      n_tok_out[i] = 0;
-    }
-    return;
-  }
+// Trainable tokens of [s, e) and the owner i of each token of it, by the `n` threads of which this
+// is thread k: 16 mask bytes a load and four owners a store over the part of the span whose
+// addresses are 16-byte aligned (a warp per span with one byte and one owner at a time took 14 us
+// for 512 spans of 512 to 8,192 tokens, a chain of 256 trips of the longest one), one token at a
+// time over the rest.
+__device__ __forceinline__ int32_t count_span(int64_t i, int k, int n, int64_t s, int64_t e, const uint8_t* mask,
+                                              int32_t* token_traj_out) {
   int32_t cnt = 0;
-  for (int64_t t = s + lane; t < e; t += 32) {
-    cnt += mask[t] != 0;
-    if (token_traj_out) token_traj_out[t] = static_cast<int32_t>(i);
+  int64_t v0 = e, v1 = e;  // vector part
+  if (e - s >= 64) {
+    v0 = s + ((16 - (reinterpret_cast<uintptr_t>(mask + s) & 15)) & 15);
+    if (token_traj_out && (reinterpret_cast<uintptr_t>(token_traj_out + v0) & 15) != 0) v0 = e;
+    v1 = v0 + (e - v0) / 16 * 16;
   }
-  cnt = warp_sum(cnt);
-  if (lane == 0) n_tok_out[i] = cnt;
+  const int32_t who = static_cast<int32_t>(i);
+#pragma unroll 4
+  for (int64_t t = v0 + static_cast<int64_t>(k) * 16; t < v1; t += static_cast<int64_t>(n) * 16) {
+    const uint4 w = *reinterpret_cast<const uint4*>(mask + t);
+    cnt += __popc(__vsetne4(w.x, 0u)) + __popc(__vsetne4(w.y, 0u)) + __popc(__vsetne4(w.z, 0u)) +
+           __popc(__vsetne4(w.w, 0u));
+  }
+  if (token_traj_out)
+    for (int64_t t = v0 + static_cast<int64_t>(k) * 4; t < v1; t += static_cast<int64_t>(n) * 4)
+      *reinterpret_cast<int4*>(token_traj_out + t) = make_int4(who, who, who, who);
+  auto one = [&](int64_t t) {
+    cnt += mask[t] != 0;
+    if (token_traj_out) token_traj_out[t] = who;
+  };
+  const int64_t h1 = v0 < v1 ? v0 : e;  // tokens before the vector part, or all of them
+  for (int64_t t = s + k; t < h1; t += n) one(t);
+  if (v0 < v1)
+    for (int64_t t = v1 + k; t < e; t += n) one(t);
+  return cnt;
 }
 
 // L_i by owner, for tokens in any order (tree-packed batches, Sec. 3.2.3: each shared prefix
@@ -122,10 +135,74 @@ __device__ __forceinline__ void group_advantage(int64_t g, int lane, int32_t n_t
   }
 }
 
+// A_i for 32 / W neighbouring groups by one warp, a segment of W lanes each (W a power of two, at
+// least the batch's mean group size): the FP64 pipe bounds this (two lanes per clock and SM, the
+// same for one active lane of a warp as for 32), so a warp per group of 4 spent an eighth of it;
+// 4,096 groups of 4 took 27 us with the counts. Sums go over the same lanes in the same butterfly
+// order as in group_advantage (whose higher lanes add zeros), so a group of at most W members
+// gets the same bits. Groups of more than 8 W members are left to the whole warp.
+__device__ __forceinline__ void group_advantages(int64_t g0, int W, int lane, int32_t n_traj, int32_t n_groups,
+                                                 const int32_t* group_offsets, const float* rewards,
+                                                 const uint8_t* traj_valid, double adv_eps, float* adv_out,
+                                                 int32_t* status) {
+  const int64_t g = g0 + lane / W;
+  const int sl = lane % W;
+  int b = 0, e = 0;
+  if (g < n_groups) {
+    b = group_offsets[g];
+    e = group_offsets[g + 1];
+    if (b < 0 || e < b || e > n_traj) {
+      if (sl == 0) flag_status(status, RL_DEV_BAD_OFFSETS);
+      b = e = 0;
+    }
+  }
+  unsigned big = __ballot_sync(0xffffffffu, sl == 0 && e - b > 8 * W);
+  if (e - b > 8 * W) e = b;
+  int k = 0;
+  double sum = 0.0;
+  float lo = __int_as_float(0x7f800000), hi = -__int_as_float(0x7f800000);
+  for (int i = b + sl; i < e; i += W) {
+    if (traj_valid && traj_valid[i] == 0) continue;
+    const float r = rewards[i];
+    ++k;
+    sum += static_cast<double>(r);
+    lo = fminf(lo, r);
+    hi = fmaxf(hi, r);
+  }
+  __syncwarp();
+  for (int o = W / 2; o > 0; o >>= 1) {
+    k += __shfl_xor_sync(0xffffffffu, k, o);
+    sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+    hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+  }
+  const bool zero = k == 0 || lo == hi;  // nothing valid, or all valid rewards equal: A = 0
+  const double mu = sum / (k > 0 ? k : 1);
+  double sq = 0.0;
+  for (int i = b + sl; i < e && !zero; i += W) {
+    if (traj_valid && traj_valid[i] == 0) continue;
+    const double d = static_cast<double>(rewards[i]) - mu;
+    sq += d * d;
+  }
+  __syncwarp();
+  for (int o = W / 2; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+  const double denom = sqrt(sq / (k > 0 ? k : 1)) + adv_eps;
+  for (int i = b + sl; i < e; i += W) {
+    const bool valid = !zero && (!traj_valid || traj_valid[i] != 0);
+    adv_out[i] = valid ? static_cast<float>((static_cast<double>(rewards[i]) - mu) / denom) : 0.f;
+  }
+  __syncwarp();
+  for (; big; big &= big - 1)
+    group_advantage(g0 + (__ffs(big) - 1) / W, lane, n_traj, group_offsets, rewards, traj_valid, adv_eps, adv_out,
+                    status);
+}
+
 struct CountAdvArgs {
   int32_t n_traj, n_groups;
   int64_t n_tokens;
   int64_t count_blocks;            // CTAs [0, count_blocks) count, the rest form advantages
+  int32_t span_threads;            // threads that count a span: a warp, or the whole CTA
+  int32_t seg;                     // lanes per group
   const int64_t* traj_offsets;     // spans (rl_group_advantages)
   const int32_t* token_traj;       // owners (rl_group_advantages_by_owner)
   const uint8_t* mask;
@@ -142,19 +219,36 @@ struct CountAdvArgs {
 
 template <bool BY_OWNER>
 __global__ void __launch_bounds__(kAdvThreads) count_adv_kernel(const CountAdvArgs a) {
+  __shared__ int32_t part[kAdvWarps];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (blockIdx.x < a.count_blocks) {
-    const int64_t w = static_cast<int64_t>(blockIdx.x) * kAdvWarps + warp;
     if (BY_OWNER) {
-      count_owners(w, a.count_blocks * kAdvWarps, lane, a.n_tokens, a.token_traj, a.mask, a.n_traj, a.n_tok_out,
-                   a.status);
-    } else if (w < a.n_traj) {
-      count_span(w, lane, a.n_tokens, a.traj_offsets, a.mask, a.n_tok_out, a.token_traj_out, a.status);
+      count_owners(static_cast<int64_t>(blockIdx.x) * kAdvWarps + warp, a.count_blocks * kAdvWarps, lane, a.n_tokens,
+                   a.token_traj, a.mask, a.n_traj, a.n_tok_out, a.status);
+      return;
     }
+    const bool whole = a.span_threads > 32;  // the CTA takes one span, else a warp does
+    const int64_t i = whole ? blockIdx.x : static_cast<int64_t>(blockIdx.x) * kAdvWarps + warp;
+    if (i >= a.n_traj) return;
+    const int64_t s = a.traj_offsets[i], e = a.traj_offsets[i + 1];
+    const bool bad = s < 0 || e < s || e > a.n_tokens;
+    const int k = whole ? static_cast<int>(threadIdx.x) : lane;
+    if (bad && k == 0) flag_status(a.status, RL_DEV_BAD_OFFSETS);
+    int32_t cnt = bad ? 0 : count_span(i, k, a.span_threads, s, e, a.mask, a.token_traj_out);
+    cnt = __reduce_add_sync(0xffffffffu, cnt);
+    if (whole) {
+      if (lane == 0) part[warp] = cnt;
+      __syncthreads();
+      cnt = 0;
+      for (int w = 0; w < kAdvWarps; ++w) cnt += part[w];
+    }
+    if (k == 0) a.n_tok_out[i] = cnt;
   } else {
-    const int64_t g = (static_cast<int64_t>(blockIdx.x) - a.count_blocks) * kAdvWarps + warp;
-    if (g < a.n_groups)
-      group_advantage(g, lane, a.n_traj, a.group_offsets, a.rewards, a.traj_valid, a.adv_eps, a.adv_out, a.status);
+    const int per = 32 / a.seg;  // groups of a warp
+    const int64_t g0 = ((static_cast<int64_t>(blockIdx.x) - a.count_blocks) * kAdvWarps + warp) * per;
+    if (g0 < a.n_groups)
+      group_advantages(g0, a.seg, lane, a.n_traj, a.n_groups, a.group_offsets, a.rewards, a.traj_valid, a.adv_eps,
+                       a.adv_out, a.status);
   }
 }
 
@@ -169,7 +263,8 @@ __global__ void __launch_bounds__(kAdvThreads) coef_kernel(int32_t n_traj, int32
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   __shared__ long long red_n[kAdvWarps], red_s[kAdvWarps];
   long long cnt = 0, tok = 0;
-#pragma unroll 4
+  // 16 loads in flight: at 16,384 trajectories a thread's 64 counts are 4 trips to L2, not 16
+#pragma unroll 16
   for (int i = tid; i < n_traj; i += kAdvThreads) {
     const int32_t L = n_tok[i];
     const bool counted = (!traj_valid || traj_valid[i] != 0) && L > 0;
@@ -217,7 +312,12 @@ template <bool BY_OWNER>
 static rl_status launch_advantages(CountAdvArgs a, int64_t count_blocks, const rl_loss_params* params, const char* fn,
                                    cudaStream_t s) {
   a.count_blocks = count_blocks;
-  const int64_t adv_blocks = (static_cast<int64_t>(a.n_groups) + kAdvWarps - 1) / kAdvWarps;
+  // lanes per group: the power of two at or above the mean group size
+  const int64_t mean = a.n_groups > 0 ? (static_cast<int64_t>(a.n_traj) + a.n_groups - 1) / a.n_groups : 32;
+  a.seg = 2;
+  while (a.seg < mean && a.seg < 32) a.seg *= 2;
+  const int64_t per_cta = static_cast<int64_t>(kAdvWarps) * (32 / a.seg);
+  const int64_t adv_blocks = (a.n_groups + per_cta - 1) / per_cta;
   const int64_t blocks = count_blocks + adv_blocks;
   if (blocks > 0) {
     count_adv_kernel<BY_OWNER><<<static_cast<unsigned>(blocks), kAdvThreads, 0, s>>>(a);
@@ -274,7 +374,10 @@ extern "C" rl_status rl_group_advantages(int32_t n_traj, int32_t n_groups, const
   a.n_tok_out = n_tok_out;
   a.token_traj_out = token_traj_out;
   a.status = reinterpret_cast<int32_t*>(ws);
-  const int64_t count_blocks = (static_cast<int64_t>(n_traj) + kAdvWarps - 1) / kAdvWarps;  // a warp per span
+  // a CTA per span while one wave of the GPU (8 CTAs per SM) holds them, else a warp per span
+  a.span_threads = n_traj <= 152 * 8 ? kAdvThreads : 32;
+  const int64_t count_blocks =
+      a.span_threads > 32 ? n_traj : (static_cast<int64_t>(n_traj) + kAdvWarps - 1) / kAdvWarps;
   return launch_advantages<false>(a, count_blocks, params, "rl_group_advantages",
                                   reinterpret_cast<cudaStream_t>(stream));
 }
