@@ -38,6 +38,15 @@ __device__ __forceinline__ uint16_t f32_to_bf16(float x) {
   return r;
 }
 
+// Exact float -> double without the FP64 pipe for normal numbers (the exponent rebiased by
+// 1023 - 127); zeros, subnormals, infinities and NaN take the conversion instruction.
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t b = __float_as_uint(x), e = (b >> 23) & 0xFFu;
+  if (e == 0u || e == 255u) return (b << 1) == 0u ? __hiloint2double(static_cast<int>(b), 0) : static_cast<double>(x);
+  const uint32_t hi = (b & 0x80000000u) | (((b & 0x7FFFFFFFu) >> 3) + (896u << 20));
+  return __hiloint2double(static_cast<int>(hi), static_cast<int>(b << 29));
+}
+
 __device__ __forceinline__ uint64_t global_timer_ns() {
   uint64_t t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));

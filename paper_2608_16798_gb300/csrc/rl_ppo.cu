@@ -28,6 +28,7 @@
 // launch-bound next to the logits stream.
 #include <algorithm>
 #include <cstdint>
+#include <type_traits>
 
 #include "rl_device.cuh"
 #include "rl_host.h"
@@ -284,22 +285,56 @@ struct ValueArgs {
 // Each CTA adds its rows' terms in a fixed order (thread-strided, then warp and CTA) and leaves
 // one partial per CTA in row_loss[blockIdx.x]; the last CTA to finish (a counter in the
 // workspace header, which it resets) adds the partials in a fixed order into loss_accum.
+//
+// The FP64 pipe (16 clocks per warp instruction and SM) and the chain mask -> owner -> coefficient
+// bound it, not the 21 bytes per row: so the floats are widened by integer instructions (one DFMA
+// per row of four FP64 instructions), the grid is at most 4 CTAs per SM (the per-CTA sums are
+// FP64 too), and VEC = 4 (every array on 16-byte boundaries, the mask on 4) takes four rows per
+// thread and load.
+template <int VEC>
 __global__ void __launch_bounds__(256) value_loss_kernel(const ValueArgs p) {
   __shared__ double part[8];
   __shared__ uint32_t last;
   double acc = 0.0;
-  for (int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; t < p.rows;
-       t += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    float c = 0.f;
-    if (p.mask[t] != 0) {
-      const int32_t i = p.token_traj[t];
-      if (i < 0 || i >= p.n_traj) flag_status(p.status, RL_DEV_BAD_TRAJ);
-      else c = p.coef[i];
+  // the value-loss terms of N rows whose inputs are in registers; the gradient goes to g
+  auto terms = [&](auto n, const uint8_t* m, const int32_t* who, const float* v, const float* ret, float* g) {
+    constexpr int N = decltype(n)::value;
+    float c[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      const bool in = who[k] >= 0 && who[k] < p.n_traj;
+      if (m[k] != 0 && !in) flag_status(p.status, RL_DEV_BAD_TRAJ);
+      c[k] = (m[k] != 0 && in) ? p.coef[who[k]] : 0.f;
     }
-    const float d = p.values[t] - p.returns[t];
-    const float cd = c * d;
-    p.d_values[t] = c != 0.f ? 2.f * cd : 0.f;
-    if (c != 0.f) acc += static_cast<double>(cd) * static_cast<double>(d);
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      const float d = v[k] - ret[k];
+      const float cd = c[k] * d;
+      g[k] = c[k] != 0.f ? 2.f * cd : 0.f;
+      if (c[k] != 0.f) acc = fma(widen(cd), widen(d), acc);
+    }
+  };
+  const int64_t first = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+  const int64_t vecs = VEC == 4 ? p.rows / 4 : 0;
+  for (int64_t k = first; k < vecs; k += stride) {
+    const uchar4 m = reinterpret_cast<const uchar4*>(p.mask)[k];
+    const int4 w = reinterpret_cast<const int4*>(p.token_traj)[k];
+    const float4 v = reinterpret_cast<const float4*>(p.values)[k], r = reinterpret_cast<const float4*>(p.returns)[k];
+    const uint8_t ms[4] = {m.x, m.y, m.z, m.w};
+    const int32_t who[4] = {w.x, w.y, w.z, w.w};
+    const float vs[4] = {v.x, v.y, v.z, v.w}, rs[4] = {r.x, r.y, r.z, r.w};
+    float g[4];
+    terms(std::integral_constant<int, 4>{}, ms, who, vs, rs, g);
+    reinterpret_cast<float4*>(p.d_values)[k] = make_float4(g[0], g[1], g[2], g[3]);
+  }
+  for (int64_t t = vecs * 4 + first; t < p.rows; t += stride) {
+    const uint8_t m = p.mask[t];
+    const int32_t who = p.token_traj[t];
+    const float v = p.values[t], r = p.returns[t];
+    float g;
+    terms(std::integral_constant<int, 1>{}, &m, &who, &v, &r, &g);
+    p.d_values[t] = g;
   }
   acc = warp_sum(acc);
   if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = acc;
@@ -430,8 +465,12 @@ extern "C" rl_status rl_value_loss_fwd_bwd(int64_t rows, const float* values, co
   a.done = reinterpret_cast<uint32_t*>(static_cast<char*>(ws) + kWsValueDoneOffset);
   a.status = reinterpret_cast<int32_t*>(ws);
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  const int blocks = ppo::grid_for(rows, 256, 152 * 16);  // <= rows: one partial per CTA fits
-  ppo::value_loss_kernel<<<blocks, 256, 0, s>>>(a);
+  auto on = [](const void* q, uintptr_t n) { return reinterpret_cast<uintptr_t>(q) % n == 0; };
+  const bool vec = on(values, 16) && on(returns, 16) && on(token_traj, 16) && on(d_values, 16) && on(mask, 4);
+  // at least one row per CTA, so that one partial per CTA fits the workspace
+  const int blocks = ppo::grid_for(rows, vec ? 1024 : 256, 152 * 4);
+  if (vec) ppo::value_loss_kernel<4><<<blocks, 256, 0, s>>>(a);
+  else ppo::value_loss_kernel<1><<<blocks, 256, 0, s>>>(a);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_error(e, "value_loss_kernel launch");
   return RL_OK;  // the kernel's last CTA has added the loss into loss_accum

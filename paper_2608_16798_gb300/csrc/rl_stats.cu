@@ -72,15 +72,6 @@ __device__ __forceinline__ void st_cluster_f64(uint32_t addr, double v) {
   asm volatile("st.shared::cluster.f64 [%0], %1;" :: "r"(addr), "d"(v) : "memory");
 }
 
-// Exact float -> double without the FP64 pipe for normal numbers (the exponent rebiased by
-// 1023 - 127); zeros, subnormals, infinities and NaN take the conversion instruction.
-__device__ __forceinline__ double widen(float x) {
-  const uint32_t b = __float_as_uint(x), e = (b >> 23) & 0xFFu;
-  if (e == 0u || e == 255u) return (b << 1) == 0u ? __hiloint2double(static_cast<int>(b), 0) : static_cast<double>(x);
-  const uint32_t hi = (b & 0x80000000u) | (((b & 0x7FFFFFFFu) >> 3) + (896u << 20));
-  return __hiloint2double(static_cast<int>(hi), static_cast<int>(b << 29));
-}
-
 __global__ void __launch_bounds__(kSumThreads)
     stats_summary_kernel(int64_t rows, const float* __restrict__ st, const uint8_t* __restrict__ mask,
                          const int32_t* __restrict__ token_traj, int32_t n_traj, const float* __restrict__ coef,
