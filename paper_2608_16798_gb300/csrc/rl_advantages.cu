@@ -32,7 +32,7 @@ constexpr int kAdvThreads = 256;
 constexpr int kAdvWarps = kAdvThreads / 32;
 
 // Trainable tokens of [s, e) and the owner i of each token of it, by the `n` threads of which this
-// is thread k: 16 mask bytes a load and four owners a store over the part of the span whose
+// is thread k (a few lanes, a warp or a CTA): 16 mask bytes a load and four owners a store over the part of the span whose
 // addresses are 16-byte aligned (a warp per span with one byte and one owner at a time took 14 us
 // for 512 spans of 512 to 8,192 tokens, a chain of 256 trips of the longest one), one token at a
 // time over the rest.
@@ -200,8 +200,8 @@ __device__ __forceinline__ void group_advantages(int64_t g0, int W, int lane, in
 struct CountAdvArgs {
   int32_t n_traj, n_groups;
   int64_t n_tokens;
-  int64_t count_blocks;            // CTAs [0, count_blocks) count, the rest form advantages
-  int32_t span_threads;            // threads that count a span: a warp, or the whole CTA
+  int64_t count_blocks, adv_blocks;  // CTAs [0, adv_blocks) form advantages, the rest count
+  int32_t span_threads;              // threads that count a span: 8 lanes, a warp, or the whole CTA
   int32_t seg;                     // lanes per group
   const int64_t* traj_offsets;     // spans (rl_group_advantages)
   const int32_t* token_traj;       // owners (rl_group_advantages_by_owner)
@@ -221,31 +221,37 @@ template <bool BY_OWNER>
 __global__ void __launch_bounds__(kAdvThreads) count_adv_kernel(const CountAdvArgs a) {
   __shared__ int32_t part[kAdvWarps];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (blockIdx.x < a.count_blocks) {
+  // the advantages first: theirs is the longer chain (two trips to memory, then FP64 divisions and
+  // a square root)
+  const int64_t block = static_cast<int64_t>(blockIdx.x) - a.adv_blocks;
+  if (block >= 0) {
     if (BY_OWNER) {
-      count_owners(static_cast<int64_t>(blockIdx.x) * kAdvWarps + warp, a.count_blocks * kAdvWarps, lane, a.n_tokens,
-                   a.token_traj, a.mask, a.n_traj, a.n_tok_out, a.status);
+      count_owners(block * kAdvWarps + warp, a.count_blocks * kAdvWarps, lane, a.n_tokens, a.token_traj, a.mask,
+                   a.n_traj, a.n_tok_out, a.status);
       return;
     }
-    const bool whole = a.span_threads > 32;  // the CTA takes one span, else a warp does
-    const int64_t i = whole ? blockIdx.x : static_cast<int64_t>(blockIdx.x) * kAdvWarps + warp;
-    if (i >= a.n_traj) return;
-    const int64_t s = a.traj_offsets[i], e = a.traj_offsets[i + 1];
-    const bool bad = s < 0 || e < s || e > a.n_tokens;
-    const int k = whole ? static_cast<int>(threadIdx.x) : lane;
-    if (bad && k == 0) flag_status(a.status, RL_DEV_BAD_OFFSETS);
-    int32_t cnt = bad ? 0 : count_span(i, k, a.span_threads, s, e, a.mask, a.token_traj_out);
-    cnt = __reduce_add_sync(0xffffffffu, cnt);
-    if (whole) {
+    const int n = a.span_threads;
+    const int k = static_cast<int>(threadIdx.x) % n;  // this thread within its span's threads
+    const int64_t i = block * (kAdvThreads / n) + threadIdx.x / n;
+    int32_t cnt = 0;
+    if (i < a.n_traj) {
+      const int64_t s = a.traj_offsets[i], e = a.traj_offsets[i + 1];
+      const bool bad = s < 0 || e < s || e > a.n_tokens;
+      if (bad && k == 0) flag_status(a.status, RL_DEV_BAD_OFFSETS);
+      if (!bad) cnt = count_span(i, k, n, s, e, a.mask, a.token_traj_out);
+    }
+    __syncwarp();
+    for (int o = (n < 32 ? n : 32) / 2; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
+    if (n > 32) {
       if (lane == 0) part[warp] = cnt;
       __syncthreads();
       cnt = 0;
       for (int w = 0; w < kAdvWarps; ++w) cnt += part[w];
     }
-    if (k == 0) a.n_tok_out[i] = cnt;
+    if (k == 0 && i < a.n_traj) a.n_tok_out[i] = cnt;
   } else {
     const int per = 32 / a.seg;  // groups of a warp
-    const int64_t g0 = ((static_cast<int64_t>(blockIdx.x) - a.count_blocks) * kAdvWarps + warp) * per;
+    const int64_t g0 = (static_cast<int64_t>(blockIdx.x) * kAdvWarps + warp) * per;
     if (g0 < a.n_groups)
       group_advantages(g0, a.seg, lane, a.n_traj, a.n_groups, a.group_offsets, a.rewards, a.traj_valid, a.adv_eps,
                        a.adv_out, a.status);
@@ -317,8 +323,8 @@ static rl_status launch_advantages(CountAdvArgs a, int64_t count_blocks, const r
   a.seg = 2;
   while (a.seg < mean && a.seg < 32) a.seg *= 2;
   const int64_t per_cta = static_cast<int64_t>(kAdvWarps) * (32 / a.seg);
-  const int64_t adv_blocks = (a.n_groups + per_cta - 1) / per_cta;
-  const int64_t blocks = count_blocks + adv_blocks;
+  a.adv_blocks = (a.n_groups + per_cta - 1) / per_cta;
+  const int64_t blocks = count_blocks + a.adv_blocks;
   if (blocks > 0) {
     count_adv_kernel<BY_OWNER><<<static_cast<unsigned>(blocks), kAdvThreads, 0, s>>>(a);
     cudaError_t e = cudaGetLastError();
@@ -374,10 +380,11 @@ extern "C" rl_status rl_group_advantages(int32_t n_traj, int32_t n_groups, const
   a.n_tok_out = n_tok_out;
   a.token_traj_out = token_traj_out;
   a.status = reinterpret_cast<int32_t*>(ws);
-  // a CTA per span while one wave of the GPU (8 CTAs per SM) holds them, else a warp per span
-  a.span_threads = n_traj <= 152 * 8 ? kAdvThreads : 32;
-  const int64_t count_blocks =
-      a.span_threads > 32 ? n_traj : (static_cast<int64_t>(n_traj) + kAdvWarps - 1) / kAdvWarps;
+  // a CTA per span while one wave of the GPU (8 CTAs per SM) holds them, else a warp per span, or 8
+  // lanes where the mean span is below 64 tokens (16,384 spans of 8 tokens were 1.7 waves of warps)
+  a.span_threads = n_traj <= 152 * 8 ? kAdvThreads : n_tokens >= 64 * static_cast<int64_t>(n_traj) ? 32 : 8;
+  const int64_t per_cta = kAdvThreads / a.span_threads;
+  const int64_t count_blocks = (n_traj + per_cta - 1) / per_cta;
   return launch_advantages<false>(a, count_blocks, params, "rl_group_advantages",
                                   reinterpret_cast<cudaStream_t>(stream));
 }
