@@ -251,7 +251,31 @@ __device__ __forceinline__ SoftmaxPartial merge(SoftmaxPartial a, SoftmaxPartial
   return r;
 }
 
+// The largest of the warp's 32 values (NaNs do not count), in every lane.
+__device__ __forceinline__ float redux_max(float v) {
+  float r;
+  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+  return r;
+}
+
+// The 32 lanes' partials merged, the same bits in every lane (WITH_U: u too, else u = 0): the
+// largest reference by one redux, each lane's sums rescaled to it once, then butterfly sums. The
+// chain is one redux, one exponential and five shuffles; merging pairs lane by lane
+// (warp_merge_pairs) is five times three shuffles and two exponentials, and a row of the loss
+// kernel waits for two such chains.
+template <bool WITH_U>
 __device__ __forceinline__ SoftmaxPartial warp_merge(SoftmaxPartial p) {
+  const bool seen = p.s != 0.f;  // a NaN sum is seen, and poisons the merge
+  const float M = redux_max(seen ? p.m : -__int_as_float(0x7f800000));
+  const float d = p.m - M;
+  const float f = ex2(d * kLog2e);
+  SoftmaxPartial r{M, warp_sum(seen ? p.s * f : 0.f), 0.f};
+  if (WITH_U) r.u = warp_sum(seen ? f * fmaf(d, p.s, p.u) : 0.f);
+  return r;
+}
+
+// The same by pairs: lane 0's merge, broadcast.
+__device__ __forceinline__ SoftmaxPartial warp_merge_pairs(SoftmaxPartial p) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     SoftmaxPartial q;
@@ -260,6 +284,9 @@ __device__ __forceinline__ SoftmaxPartial warp_merge(SoftmaxPartial p) {
     q.u = __shfl_xor_sync(0xffffffffu, p.u, o);
     p = merge(p, q);
   }
+  p.m = __shfl_sync(0xffffffffu, p.m, 0);
+  p.s = __shfl_sync(0xffffffffu, p.s, 0);
+  p.u = __shfl_sync(0xffffffffu, p.u, 0);
   return p;
 }
 

@@ -348,6 +348,33 @@ __device__ __forceinline__ void fold_block(SoftmaxPartial& ps, const uint4 (&x)[
   ps.s = fmaf(se, f, ps.s);
 }
 
+// Log-sum-exp of a row's merged partial as hi + lo. bf16: lo is what the rounding of m + ln S and of
+// the logarithm leave out (the latter from S e^-lnS = 1 + it), so that the ratio exp(logp - old) is
+// off by the error of S alone; fp32 keeps its order of operations: lo = 0.
+struct RowLse {
+  float lnS, hi, lo;
+};
+template <typename T>
+__device__ __forceinline__ RowLse row_lse(const SoftmaxPartial& q) {
+  RowLse l{logf(q.s), 0.f, 0.f};
+  l.hi = q.m + l.lnS;
+  if constexpr (sizeof(T) == 2) {
+    const float b = l.hi - q.m;
+    l.lo = (q.m - (l.hi - b)) + (l.lnS - b) + fmaf(q.s, expf(-l.lnS), -1.f);
+  }
+  return l;
+}
+
+// The warp's 32 partials of a row of the loss kernels. bf16: the short chain. fp32: by pairs, whose
+// order the results of the fp32 path keep to the bit: a near-one-hot row's gradient is c g (1 - p) at
+// the sampled token, so the last bit of a log-sum-exp of 40 (4e-6) shows in it, and the fp32 edge
+// batch, bound by HBM, gains nothing from the shorter chain (1,062-1,092 us before, 1,109 us with it).
+template <typename T, bool ENT>
+__device__ __forceinline__ SoftmaxPartial merge_lanes(SoftmaxPartial p) {
+  if constexpr (sizeof(T) == 2) return warp_merge<ENT>(p);
+  else return warp_merge_pairs(p);
+}
+
 // MINB: CTAs per SM the register budget is sized for (2, or 3 with a smaller zero region).
 template <typename T, int NW, bool ENT, bool BWD, int HOLDV, int MINB>
 __global__ void __launch_bounds__((NW + 1) * 32, MINB) rows_kernel(const RowArgs p) {
@@ -381,8 +408,8 @@ __global__ void __launch_bounds__((NW + 1) * 32, MINB) rows_kernel(const RowArgs
       mbar_init(&full_bar[k], 1);
       mbar_init(&empty_bar[k], NW);
     }
-    mbar_init(&xbar[0], 1);
-    mbar_init(&xbar[1], 1);
+    mbar_init(&xbar[0], C == 1 ? NW : 1);
+    mbar_init(&xbar[1], C == 1 ? NW : 1);
     fence_mbar_init();
   }
   for (int k = tid; k < kZeroBytes / 16; k += blockDim.x) zeros[k] = make_uint4(0, 0, 0, 0);
@@ -571,11 +598,7 @@ __global__ void __launch_bounds__((NW + 1) * 32, MINB) rows_kernel(const RowArgs
           accumulate<ENT>(ps, z, -ps.m * kLog2e);
         }
       }
-      ps = warp_merge(ps);
-      // lane 0's merge is the warp's partial: broadcast it so every copy sent is identical
-      ps.m = __shfl_sync(0xffffffffu, ps.m, 0);
-      ps.s = __shfl_sync(0xffffffffu, ps.s, 0);
-      ps.u = __shfl_sync(0xffffffffu, ps.u, 0);
+      ps = merge_lanes<T, ENT>(ps);  // the same in every lane
       // warp 0 of the CTA holding the sampled token carries z_a; every other partial carries 0
       const float za_part = (warp == 0 && a_ok && rank == owner) ? Vec<T>::to_f(buf[a - s0]) : 0.f;
       if (HOLDV > 0) {  // every read of the stage is done
@@ -583,42 +606,45 @@ __global__ void __launch_bounds__((NW + 1) * 32, MINB) rows_kernel(const RowArgs
         if (lane == 0) mbar_arrive(&empty_bar[b]);
       }
 
-      // ---- exchange: every warp's partial to every CTA of the cluster
+      // ---- exchange: every warp's partial to every CTA of the cluster (a CTA on its own: to its
+      // own mailbox by a plain store and an arrival, without the trip through the cluster's network)
       const int par = it & 1;
-      if (warp == 0 && lane == 0) mbar_arrive_expect_tx(&xbar[par], C * NW * 16u);
-      if (lane < static_cast<int>(C)) {
-        const uint32_t dst = map_to_rank(smem_addr(&mbox[par][rank * NW + warp]), lane);
-        const uint32_t bar = map_to_rank(smem_addr(&xbar[par]), lane);
-        st_async_f4(dst, make_float4(ps.m, ps.s, ps.u, za_part), bar);
+      if (C == 1) {
+        if (lane == 0) {
+          mbox[par][warp] = make_float4(ps.m, ps.s, ps.u, za_part);
+          mbar_arrive(&xbar[par]);
+        }
+      } else {
+        if (warp == 0 && lane == 0) mbar_arrive_expect_tx(&xbar[par], C * NW * 16u);
+        if (lane < static_cast<int>(C)) {
+          const uint32_t dst = map_to_rank(smem_addr(&mbox[par][rank * NW + warp]), lane);
+          const uint32_t bar = map_to_rank(smem_addr(&xbar[par]), lane);
+          st_async_f4(dst, make_float4(ps.m, ps.s, ps.u, za_part), bar);
+        }
       }
       if (!mbar_wait_cluster_bounded(&xbar[par], (it >> 1) & 1)) {
         if (lane == 0) flag_status(p.status, RL_DEV_TIMEOUT);
         break;
       }
       // ---- merge all C * NW partials in a fixed order
+      // (lane l takes partials l, l + 32, ...; those with nothing seen, s = 0, do not count)
       const int total = static_cast<int>(C) * NW;
-      SoftmaxPartial qa{RL_NEG_INF, 0.f, 0.f}, qb{RL_NEG_INF, 0.f, 0.f};
-      float zsum = 0.f;
-      if (lane < total) {
-        const float4 w = mbox[par][lane];
-        qa = SoftmaxPartial{w.x, w.y, w.z};
-        zsum = w.w;
-      }
-      if (lane + 32 < total) {
-        const float4 w = mbox[par][lane + 32];
-        qb = SoftmaxPartial{w.x, w.y, w.z};
-        zsum += w.w;
-      }
-      for (int k = lane + 64; k < total; k += 32) {  // clusters of 16 with more than 4 consumer warps
+      float4 w0 = make_float4(RL_NEG_INF, 0.f, 0.f, 0.f), w1 = w0;
+      if (lane < total) w0 = mbox[par][lane];
+      if (lane + 32 < total) w1 = mbox[par][lane + 32];
+      SoftmaxPartial q{w0.x, w0.y, w0.z};
+      float zsum = w0.w + w1.w;
+      if (total > 32) q = merge(q, SoftmaxPartial{w1.x, w1.y, w1.z});
+      for (int k = lane + 64; k < total; k += 32) {
         const float4 w = mbox[par][k];
-        qb = merge(qb, SoftmaxPartial{w.x, w.y, w.z});
+        q = merge(q, SoftmaxPartial{w.x, w.y, w.z});
         zsum += w.w;
       }
-      SoftmaxPartial q = warp_merge(merge(qa, qb));
-      const float za = __shfl_sync(0xffffffffu, warp_sum(zsum), 0);
-      const float lnS = logf(__shfl_sync(0xffffffffu, q.s, 0));
-      const float lse = __shfl_sync(0xffffffffu, q.m, 0) + lnS;
-      const float H = lnS - __shfl_sync(0xffffffffu, q.u, 0) / __shfl_sync(0xffffffffu, q.s, 0);
+      q = merge_lanes<T, ENT>(q);  // the same in every lane
+      const float za = warp_sum(zsum);
+      const RowLse rl = row_lse<T>(q);
+      const float lnS = rl.lnS, lse = rl.hi;
+      const float H = ENT || sizeof(T) == 4 ? lnS - q.u / q.s : 0.f;  // times 0 without the entropy
 
       if (!BWD) {
         if (rank == 0 && warp == 0 && lane == 0) {
@@ -630,15 +656,15 @@ __global__ void __launch_bounds__((NW + 1) * 32, MINB) rows_kernel(const RowArgs
       } else {
         // per-token scalars (every lane computes the same values)
         const float A = m.A, c = m.c, old = m.old;
-        const float logp = za - lse;
-        const float rho = expf((za - old) - lse);   // large operands differenced first
+        const float logp = (za - lse) - rl.lo;
+        const float rho = expf(((za - old) - lse) - rl.lo);   // large operands differenced first
         const float crho = fminf(fmaxf(rho, p.clip_lo), p.clip_hi);
         const float surr = fminf(rho * A, crho * A);
         const bool cut = (A > 0.f && rho > p.clip_hi) || (A < 0.f && rho < p.clip_lo);
         const float w = (p.tis_cap > 0.f && p.rollout_logp) ? fminf(expf(old - m.roll), p.tis_cap) : 1.f;
         float kl = 0.f, dkl = 0.f;
         if (p.beta != 0.f && p.ref_logp) {
-          const float d = (m.ref - za) + lse;  // r - logp
+          const float d = ((m.ref - za) + lse) + rl.lo;  // r - logp
           const float ed = expf(d);
           kl = ed - d - 1.f;
           dkl = 1.f - ed;
@@ -649,7 +675,7 @@ __global__ void __launch_bounds__((NW + 1) * 32, MINB) rows_kernel(const RowArgs
         // p_v = 2^(z_v log2(e) + nl) with nl = fl(-lse log2(e)); its rounding scales every p_v of
         // the row by 2^errl (errl exact by one fma), folded into the coefficients below
         const float nl = -lse * kLog2e;
-        const float fl = fmaf(fmaf(-lse, kLog2e, -nl), kLn2, 1.f);
+        const float fl = fmaf(fmaf(-lse, kLog2e, -nl), kLn2, 1.f - rl.lo);
         const float Kp = -cg * fl;                      // gradient = Kp p_v (+ cg at v = a)
         const float ca = ca0 * fl;                      // entropy: p_v (ca z_v + Ke)
         const float Ke = (-cg + ca0 * (H - lse)) * fl;
@@ -834,7 +860,7 @@ __global__ void __launch_bounds__(kSmallWarps * 32, 2) small_rows_kernel(const R
       continue;
     }
     const float za = Vec<T>::to_f(row[a]);
-    // ---- pass 1: the lane's partial, then the warp's (lane 0's merge, broadcast)
+    // ---- pass 1: the lane's partial, then the warp's
     SoftmaxPartial ps{RL_NEG_INF, 0.f, 0.f};
     fold_block<T, ENT>(ps, x, reload);
     float tail_z = 0.f;
@@ -847,23 +873,20 @@ __global__ void __launch_bounds__(kSmallWarps * 32, 2) small_rows_kernel(const R
         accumulate<ENT>(ps, z, -ps.m * kLog2e);
       }
     }
-    SoftmaxPartial q = warp_merge(ps);
-    q.m = __shfl_sync(0xffffffffu, q.m, 0);
-    q.s = __shfl_sync(0xffffffffu, q.s, 0);
-    q.u = __shfl_sync(0xffffffffu, q.u, 0);
-    const float lnS = logf(q.s);
-    const float lse = q.m + lnS;
-    const float H = lnS - q.u / q.s;
+    const SoftmaxPartial q = merge_lanes<T, ENT>(ps);  // the same in every lane
+    const RowLse rl = row_lse<T>(q);
+    const float lnS = rl.lnS, lse = rl.hi;
+    const float H = ENT ? lnS - q.u / q.s : 0.f;
     // ---- per-token scalars (every lane computes the same values)
-    const float logp = za - lse;
-    const float rho = expf((za - old) - lse);  // large operands differenced first
+    const float logp = (za - lse) - rl.lo;
+    const float rho = expf(((za - old) - lse) - rl.lo);  // large operands differenced first
     const float crho = fminf(fmaxf(rho, p.clip_lo), p.clip_hi);
     const float surr = fminf(rho * A, crho * A);
     const bool cut = (A > 0.f && rho > p.clip_hi) || (A < 0.f && rho < p.clip_lo);
     const float w = (p.tis_cap > 0.f && p.rollout_logp) ? fminf(expf(old - roll), p.tis_cap) : 1.f;
     float kl = 0.f, dkl = 0.f;
     if (p.beta != 0.f && p.ref_logp) {
-      const float d = (ref - za) + lse;  // r - logp
+      const float d = ((ref - za) + lse) + rl.lo;  // r - logp
       const float ed = expf(d);
       kl = ed - d - 1.f;
       dkl = 1.f - ed;
@@ -874,7 +897,7 @@ __global__ void __launch_bounds__(kSmallWarps * 32, 2) small_rows_kernel(const R
     // p_v = 2^(z_v log2(e) + nl), the rounding of nl folded into the coefficients (as in the
     // cluster kernel)
     const float nl = -lse * kLog2e;
-    const float fl = fmaf(fmaf(-lse, kLog2e, -nl), kLn2, 1.f);
+    const float fl = fmaf(fmaf(-lse, kLog2e, -nl), kLn2, 1.f - rl.lo);
     const float Kp = -cg * fl;
     const float ca = ca0 * fl;
     const float Ke = (-cg + ca0 * (H - lse)) * fl;
@@ -1091,12 +1114,12 @@ __global__ void __launch_bounds__((NW + 1) * 32, 2) stream_logprobs_kernel(const
       if (ci.first + ci.count == V) {
         // ---- end of row ci.r: merge the consumers' partials
         const int par = row_it & 1;
-        ps = warp_merge(ps);
+        ps = warp_merge<ENT>(ps);
         if (lane == 0) red[par][warp] = ps;
         asm volatile("bar.sync 1, %0;" :: "n"(NC) : "memory");
         if (warp == 0) {
           SoftmaxPartial qq = lane < NW ? red[par][lane] : SoftmaxPartial{RL_NEG_INF, 0.f, 0.f};
-          qq = warp_merge(qq);
+          qq = warp_merge<ENT>(qq);
           if (lane == 0) {
             const int64_t r = ci.r;
             const float lnS = logf(qq.s);
