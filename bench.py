@@ -1176,9 +1176,9 @@ def time_head(torch, R, dev, warmup=2, reps=5, oracle_tokens=0):
         with open(p) as f:
             pk = json.load(f)
         burst, sustained, kind = float(pk["bf16_tflops"]), float(pk["bf16_tflops_sustained"]), "measured"
-    flops = 6.0 * hb.T * hb.D * hb.V
+    flops = 6.0 * hb.trained * hb.D * hb.V  # only trained tokens go through the products
     tf = flops / (ms * 1e-3) / 1e12
-    chunks = (hb.T + 4095) // 4096
+    chunks = (hb.trained + 4095) // 4096
     tf_fwd = 2.0 * hb.T * hb.D * hb.V / (ms_fwd * 1e-3) / 1e12
     fwd = {"ms_per_call": ms_fwd, "tokens_per_s": hb.T / (ms_fwd * 1e-3), "achieved": tf_fwd, "frac": tf_fwd / burst,
            "frac_of_sustained": tf_fwd / sustained, "algorithmic_flops_per_call": 2.0 * hb.T * hb.D * hb.V,
@@ -1189,7 +1189,8 @@ def time_head(torch, R, dev, warmup=2, reps=5, oracle_tokens=0):
             "peak": burst, "unit": "TFLOP/s", "frac": tf / burst, "frac_of_sustained": tf / sustained,
             "peak_source": kind, "algorithmic_flops_per_call": flops, "executed_flops_per_call": flops,
             "reps": reps, "chunks_per_call": chunks,
-            "note": "6 T D V (Z once, dH, dW), all on hand-written tcgen05 kernels (head_kernel: logits tiles and "
+            "note": "6 D V per trained token (Z once, dH, dW; the others enter none of the products), all on "
+                    "hand-written tcgen05 kernels (head_kernel: logits tiles and "
                     "softmax partials; head_grad_kernel: dH and dW in one launch), smallest workspace "
                     f"({hb.ws.numel() / 1e9:.2f} GB: one 4,096-token chunk of the logits gradient)",
             "logprobs": fwd}, hs

@@ -115,8 +115,11 @@ const char* rl_last_error_message(void);
  * workspace holds the device status word and per-row loss contributions; with
  * D > 0 it also holds the fused head's buffers, the largest being the bf16
  * gradient of the logits of ONE chunk of min(max_rows, 4096) tokens
- * (min(max_rows, 4096) * ceil(V / 8) * 8 * 2 bytes: 1.24 GB at V = 151,936).
- * This is the smallest workspace of rl_fused_head_loss_fwd_bwd. */
+ * (min(max_rows, 4096) * ceil(V / 8) * 8 * 2 bytes: 1.24 GB at V = 151,936);
+ * others are the packed hidden states of one chunk and, for few tokens, partial
+ * sums of d_hidden. A smaller workspace, without room for the last two, is
+ * accepted by rl_fused_head_loss_fwd_bwd down to what the others take; every
+ * token then goes through the products. */
 size_t rl_workspace_size(int64_t max_rows, int64_t V, int64_t D);
 
 /* Workspace bytes with which rl_fused_head_loss_fwd_bwd on up to T tokens keeps the
@@ -124,8 +127,10 @@ size_t rl_workspace_size(int64_t max_rows, int64_t V, int64_t D);
  * chunks of 4,096 tokens; group_tokens <= 4096 gives rl_workspace_size(T, V, D)).
  * The fused head then runs its dH and dW products once per group instead of once
  * per chunk, which reads and writes the fp32 d_weight fewer times, at the cost of
- * ceil(V / 8) * 8 * 2 bytes per token of the group. Any workspace size between the
- * two works: the group is as many whole chunks as the workspace holds. */
+ * ceil(V / 8) * 8 * 2 bytes per token of the group. Any workspace size works: the
+ * group is as many whole chunks of trained tokens as the workspace holds, each with its
+ * logits gradient and its packed hidden states (4,096 * D * 2 bytes, which this size
+ * counts once: the group can be one chunk smaller than asked for). */
 size_t rl_fused_head_workspace_size(int64_t T, int64_t V, int64_t D, int64_t group_tokens);
 
 /* Zero the workspace's 256-byte header: the status word and the finished-block
@@ -278,15 +283,17 @@ rl_status rl_policy_loss_fwd_bwd(const void* logits, rl_dtype dtype, int64_t row
  *                 among others, the gradient of the logits (bf16) of one chunk of
  *                 4,096 tokens, or of a group of several chunks when ws_bytes allows
  *                 (rl_fused_head_workspace_size), consumed by the dH and dW products
- * Tokens are processed in chunks of 4,096: per chunk, one tensor-core pass forms the
- * logits tile by tile, folds them into softmax partials and keeps exp(z - tile max)
- * in bf16 with the tile maxima; a per-token merge evaluates the objective; an in-place
- * rescale turns the kept values into the logits' gradient. After the last chunk of
- * each group (each chunk, with the smallest workspace), two tensor-core products give
- * the group's dH and add its dW (fp32, one addition per element and group, in chunk
- * order: deterministic). The groups follow ws_bytes, so the rounding of d_weight and
- * d_hidden (not their values up to rounding) depends on the workspace size; calls with
- * the same ws_bytes give the same bits. The logits of all T tokens are never held at once.
+ * Tokens that are not trained on (M_t = 0, c = 0, a bad id or owner) enter none of the
+ * products, whatever their hidden states hold. The others are packed and processed in chunks
+ * of at most 4,096: per chunk, one tensor-core pass forms the logits tile by tile, folds them
+ * into softmax partials and keeps exp(z - tile max) in bf16 with the tile maxima; a per-token
+ * merge evaluates the objective; an in-place rescale turns the kept values into the logits'
+ * gradient. After the last chunk of each group (each chunk, with the smallest workspace), two
+ * tensor-core products give the group's dH and add its dW (fp32, one addition per element and
+ * group, in chunk order: deterministic). The groups follow ws_bytes, and the blocks of the
+ * vocabulary and the parts of dH's contraction follow T, so the rounding of d_weight and
+ * d_hidden (not their values up to rounding) depends on both; calls with the same T and
+ * ws_bytes give the same bits. The logits of all T tokens are never held at once.
  */
 rl_status rl_fused_head_loss_fwd_bwd(const void* hidden, const void* weight, int64_t T, int64_t D, int64_t V,
                                      const int32_t* token_ids, const uint8_t* mask, const int32_t* token_traj,
@@ -459,9 +466,9 @@ rl_status rl_sequence_is_weights(int32_t n_traj, int64_t n_tokens, const int32_t
  *   entropy_out  float [T] or NULL (entropy work is skipped when NULL)
  *   lse_out      float [T] or NULL
  *   ws, ws_bytes workspace; rl_workspace_size(T, V, D) bytes always suffice (the
- *                call uses the status word and 32 * ceil(V / 4096) * min(T, 4096)
- *                bytes of softmax partials after it: two per token and 4,096-entry
- *                vocabulary block)
+ *                call uses the status word and softmax partials after it: two of 16 bytes per
+ *                token and vocabulary block, at least 32 * ceil(V / 4096) * min(T, 4096) bytes;
+ *                more allow smaller blocks, which few tokens need to fill the GPU)
  * One tensor-core pass per chunk of 4,096 tokens, then a per-token merge of the
  * vocabulary blocks' partials in fixed order (deterministic).
  */

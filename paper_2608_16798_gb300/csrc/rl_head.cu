@@ -1,7 +1,9 @@
 // Fused LM head: the policy loss and its gradients with respect to the hidden states
 // and the output projection, with the logits Z = H W^T never written to memory.
 //
-// For each chunk of tokens:
+// Only the tokens that are trained on go through the products: head_select_kernel lists them, and
+// for each chunk of the list:
+//   0. head_gather_kernel   packs the chunk's hidden states.
 //   1. head_kernel<STATS_P> tcgen05 GEMM tiles Z[256 x 256] = H W^T on CTA pairs (2-CTA
 //      clusters, cta_group::2 MMAs; TMA-fed shared-memory stages, fp32 accumulators in TMEM,
 //      two accumulators so the epilogue of one tile overlaps the MMAs of the next; each CTA
@@ -9,7 +11,7 @@
 //      its row maximum m_j, then e = exp(z - m_j), which it stores (bf16) in the chunk's
 //      dZ buffer, with m_j per token and tile, and folds into per-row online-softmax
 //      partials: two per vocabulary block (its even and its odd tiles).
-//   2. head_merge_kernel    one thread per token: merges the partials into lse, entropy and
+//   2. head_merge_kernel    one warp per token: merges the partials into lse, entropy and
 //      logp, evaluates the objective's per-token terms (same readings as the logits path),
 //      writes the row's loss contribution and the coefficients of dZ.
 //   3. head_dz_kernel       rescales the stored e in place into
@@ -21,8 +23,9 @@
 //   4. dH = dZ W and dW += dZ^T H over the group in one persistent launch of
 //      head_grad_kernel (rl_head_grad.cu): CTA-pair tcgen05 MMAs on 256 x 512 tiles with the
 //      operands in their row-major layouts (dZ K-major for dH, MN-major for dW; W and H
-//      MN-major), dH tiles first and dW tiles after them, handed out by a work counter; dH is
-//      stored, dW added in fp32 by TMA reduce-add, once per group.
+//      MN-major), dH tiles first and dW tiles after them, handed out by a work counter; dH rows
+//      are stored at their tokens' places (a short call's in parts of the contraction, which
+//      head_combine_kernel adds), dW added in fp32 by TMA reduce-add, once per group.
 // The forward-only call runs head_wide_kernel<STATS> (256 x 512 tiles, no stores; the same two
 // partials per block) and head_logp_merge_kernel.
 // The objective (Sec. 2.3.2, Sec. 3.2.4) is the same as for rl_policy_loss_fwd_bwd; here
@@ -35,6 +38,7 @@
 #include <string>
 
 #include "rl_device.cuh"
+#include "rl_head_tokens.cuh"
 #include "rl_host.h"
 #include "rl_tc.cuh"
 #include "rl_tmap.h"
@@ -46,10 +50,8 @@ constexpr int BM = 128;            // tokens per tile (TMEM lanes)
 constexpr int BN = 256;            // vocabulary entries per tile (TMEM columns per accumulator)
 constexpr int BK = 64;             // hidden elements per stage (one 128-byte swizzle row)
 constexpr int NS = 4;              // shared-memory stages
-#ifndef RL_HEAD_VB_TILES
-#define RL_HEAD_VB_TILES 16
-#endif
-constexpr int VB_TILES = RL_HEAD_VB_TILES;  // N tiles per work item (16: a vocabulary block of 4,096)
+constexpr int kMaxVb = 16;         // most N tiles per work item (16: a vocabulary block of 4,096)
+constexpr int kPairs = 76;         // CTA pairs of the GPU (152 SMs)
 constexpr uint32_t A_BYTES = BM * BK * 2, B_BYTES = BN * BK * 2, STAGE_BYTES = A_BYTES + B_BYTES;
 constexpr int kThreads = 192;      // warp 0 TMA, warp 1 MMA, warps 2-5 epilogue
 constexpr size_t kSmem = NS * STAGE_BYTES + 1024;
@@ -86,12 +88,13 @@ struct RowCoef {
 };
 
 struct HeadArgs {
-  int64_t t0;  // first token of the chunk
-  int32_t Tc, D, V, n_mt, n_vb, n_nt;
+  Tokens tok;  // the call's tokens
+  int32_t chunk;           // which chunk of them
+  int32_t D, V, vb_tiles, n_vb, n_nt;  // N tiles per work item (even), items and tiles per row tile
   int32_t ent;
   const int32_t* token_ids;
   float4* partials;        // [2 n_vb][Tc] (m, s, u, z_a): a block's even tiles, then its odd tiles
-  uint16_t* dz;            // [Tc x ldz] bf16: e = exp(z - m_j) (STATS_P)
+  uint16_t* dz;            // [G Tc x ldz] bf16: e = exp(z - m_j) (STATS_P), the group's chunks in turn
   int64_t ldz;
   float* tmax;             // [Tc x n_nt]: m_j per token and tile (STATS_P)
   int32_t* status;
@@ -120,9 +123,11 @@ __global__ void __launch_bounds__(kThreads, 1) head_kernel(const __grid_constant
   const int unit = PAIR ? static_cast<int>(blockIdx.x >> 1) : static_cast<int>(blockIdx.x);
   const int n_units = PAIR ? static_cast<int>(gridDim.x >> 1) : static_cast<int>(gridDim.x);
   constexpr int kMStep = PAIR ? 2 * BM : BM;  // tokens per work item
-  const int n_m = (p.Tc + kMStep - 1) / kMStep;
+  const Chunk ch = chunk_of(p.tok, p.chunk);
+  const int n_m = (ch.count + kMStep - 1) / kMStep;
   const int n_items = n_m * p.n_vb;
   const int nkb = p.D / BK;
+  if (n_items == 0) return;  // the whole grid: no token of this chunk is trained on
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kNS; ++s) {
@@ -152,8 +157,8 @@ __global__ void __launch_bounds__(kThreads, 1) head_kernel(const __grid_constant
       bool ok = true;
       for (int item = unit; item < n_items && ok; item += n_units) {
         const int vb = item / n_m, m0 = (item % n_m) * kMStep + static_cast<int>(rank) * BM;
-        const int nt1 = min((vb + 1) * VB_TILES, p.n_nt);
-        for (int nt = vb * VB_TILES; nt < nt1 && ok; ++nt) {
+        const int nt1 = min((vb + 1) * p.vb_tiles, p.n_nt);
+        for (int nt = vb * p.vb_tiles; nt < nt1 && ok; ++nt) {
           for (int kb = 0; kb < nkb; ++kb, ++g) {
             const int s = g % kNS;
             const uint32_t use = g / kNS;
@@ -166,11 +171,11 @@ __global__ void __launch_bounds__(kThreads, 1) head_kernel(const __grid_constant
             if constexpr (PAIR) {
               if (rank == 0) mbar_arrive_expect_tx(&full[s], 2 * kStage);  // both CTAs' bytes
               const uint32_t bar = map_to_rank(smem_addr(&full[s]), 0);
-              tc::tma_load_2d_pair(st, &tmH, kb * BK, m0, bar);
+              tc::tma_load_2d_pair(st, &tmH, kb * BK, ch.row + m0, bar);
               tc::tma_load_2d_pair(st + A_BYTES, &tmW, kb * BK, nt * BN + static_cast<int>(rank) * (BN / 2), bar);
             } else {
               mbar_arrive_expect_tx(&full[s], kStage);
-              tc::tma_load_2d(st, &tmH, kb * BK, m0, &full[s]);
+              tc::tma_load_2d(st, &tmH, kb * BK, ch.row + m0, &full[s]);
               tc::tma_load_2d(st + A_BYTES, &tmW, kb * BK, nt * BN, &full[s]);
             }
           }
@@ -185,8 +190,8 @@ __global__ void __launch_bounds__(kThreads, 1) head_kernel(const __grid_constant
       bool ok = true;
       for (int item = unit; item < n_items && ok; item += n_units) {
         const int vb = item / n_m;
-        const int nt1 = min((vb + 1) * VB_TILES, p.n_nt);
-        for (int nt = vb * VB_TILES; nt < nt1 && ok; ++nt, ++t) {
+        const int nt1 = min((vb + 1) * p.vb_tiles, p.n_nt);
+        for (int nt = vb * p.vb_tiles; nt < nt1 && ok; ++nt, ++t) {
           const int acc = t & 1;
           if (t >= 2) {
             const uint32_t par = ((t >> 1) - 1) & 1;
@@ -237,13 +242,13 @@ __global__ void __launch_bounds__(kThreads, 1) head_kernel(const __grid_constant
     for (int item = unit; item < n_items && ok; item += n_units) {
       const int vb = item / n_m, m0 = (item % n_m) * kMStep + static_cast<int>(rank) * BM;
       const int r = m0 + rl;  // token within the chunk
-      const bool row_ok = r < p.Tc;
-      const int nt1 = min((vb + 1) * VB_TILES, p.n_nt);
+      const bool row_ok = r < ch.count;
+      const int nt1 = min((vb + 1) * p.vb_tiles, p.n_nt);
       // running partials of the block's even and odd tiles (the halves of its 256 x 512 tiles)
       SoftmaxPartial ps0{kNegInf, 0.f, 0.f}, ps1{kNegInf, 0.f, 0.f};
       float za = 0.f;
-      const int32_t a = row_ok ? p.token_ids[p.t0 + r] : -1;
-      for (int nt = vb * VB_TILES; nt < nt1; ++nt, ++t) {
+      const int32_t a = row_ok ? p.token_ids[token_of(p.tok, ch, r)] : -1;
+      for (int nt = vb * p.vb_tiles; nt < nt1; ++nt, ++t) {
         const int acc = t & 1;
         if (!mbar_wait_bounded(&accf[acc], (t >> 1) & 1)) {
           if (lane == 0) flag_status(p.status, RL_DEV_TIMEOUT);
@@ -298,7 +303,7 @@ __global__ void __launch_bounds__(kThreads, 1) head_kernel(const __grid_constant
             w[j / 2] = pack_bf16x2(e2[0], e2[1]);
           }
           if (MODE == STATS_P && row_ok) {
-            uint16_t* out = p.dz + static_cast<int64_t>(r) * p.ldz + col0;
+            uint16_t* out = p.dz + static_cast<int64_t>(ch.row + r) * p.ldz + col0;
             if (nvalid == 32) {
 #pragma unroll
               for (int j = 0; j < 4; ++j)
@@ -322,8 +327,8 @@ __global__ void __launch_bounds__(kThreads, 1) head_kernel(const __grid_constant
         else ps0 = merge(ps0, tile);
       }
       if (ok && row_ok) {
-        p.partials[static_cast<int64_t>(2 * vb) * p.Tc + r] = make_float4(ps0.m, ps0.s, ps0.u, za);
-        p.partials[static_cast<int64_t>(2 * vb + 1) * p.Tc + r] = make_float4(ps1.m, ps1.s, ps1.u, 0.f);
+        p.partials[static_cast<int64_t>(2 * vb) * p.tok.Tc + r] = make_float4(ps0.m, ps0.s, ps0.u, za);
+        p.partials[static_cast<int64_t>(2 * vb + 1) * p.tok.Tc + r] = make_float4(ps1.m, ps1.s, ps1.u, 0.f);
       }
     }
   }
@@ -434,11 +439,13 @@ __global__ void __launch_bounds__(kThreadsW, 1) head_wide_kernel(const __grid_co
   const uint32_t rank = cluster_ctarank();
   const int unit = static_cast<int>(blockIdx.x >> 1);
   const int n_units = static_cast<int>(gridDim.x >> 1);
-  constexpr int VB2 = VB_TILES / 2;  // 512-column tiles per vocabulary block
-  const int n_m = (p.Tc + 2 * BM - 1) / (2 * BM);
+  const int VB2 = p.vb_tiles / 2;  // 512-column tiles per vocabulary block
+  const Chunk ch = chunk_of(p.tok, p.chunk);
+  const int n_m = (ch.count + 2 * BM - 1) / (2 * BM);
   const int n_nt2 = (p.n_nt + 1) / 2;
   const int n_items = n_m * p.n_vb;
   const int nkb = p.D / BK;
+  if (n_items == 0) return;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < NSW; ++s) {
@@ -474,7 +481,7 @@ __global__ void __launch_bounds__(kThreadsW, 1) head_wide_kernel(const __grid_co
             uint8_t* st = sm + s * STAGEW_BYTES;
             if (rank == 0) mbar_arrive_expect_tx(&full[s], 2 * STAGEW_BYTES);  // both CTAs' bytes
             const uint32_t bar = map_to_rank(smem_addr(&full[s]), 0);
-            tc::tma_load_2d_pair(st, &tmH, kb * BK, m0, bar);
+            tc::tma_load_2d_pair(st, &tmH, kb * BK, ch.row + m0, bar);
 #pragma unroll
             for (int h = 0; h < 2; ++h)
               tc::tma_load_2d_pair(st + A_BYTES + h * W_HALF, &tmW, kb * BK,
@@ -532,12 +539,12 @@ __global__ void __launch_bounds__(kThreadsW, 1) head_wide_kernel(const __grid_co
     for (int item = unit; item < n_items && ok; item += n_units) {
       const int vb = item / n_m, m0 = (item % n_m) * 2 * BM + static_cast<int>(rank) * BM;
       const int r = m0 + rl;
-      const bool row_ok = r < p.Tc;
+      const bool row_ok = r < ch.count;
       const int nt1 = min((vb + 1) * VB2, n_nt2);
       SoftmaxPartial ps{kNegInf, 0.f, 0.f};
       float za = 0.f;
-      const int32_t a = row_ok ? p.token_ids[p.t0 + r] : -1;
-      uint16_t* dz_row = (MODE == STATS_P && row_ok) ? p.dz + static_cast<int64_t>(r) * p.ldz : nullptr;
+      const int32_t a = row_ok ? p.token_ids[token_of(p.tok, ch, r)] : -1;
+      uint16_t* dz_row = (MODE == STATS_P && row_ok) ? p.dz + static_cast<int64_t>(ch.row + r) * p.ldz : nullptr;
       for (int nt = vb * VB2; nt < nt1; ++nt, ++t) {
         if (!mbar_wait_sleep_bounded(&accf, t & 1)) {
           if (lane == 0) flag_status(p.status, RL_DEV_TIMEOUT);
@@ -561,7 +568,7 @@ __global__ void __launch_bounds__(kThreadsW, 1) head_wide_kernel(const __grid_co
         }
       }
       if (ok && row_ok)
-        p.partials[static_cast<int64_t>(2 * vb + h) * p.Tc + r] = make_float4(ps.m, ps.s, ps.u, za);
+        p.partials[static_cast<int64_t>(2 * vb + h) * p.tok.Tc + r] = make_float4(ps.m, ps.s, ps.u, za);
     }
   }
   tc::fence_before_sync();
@@ -573,8 +580,9 @@ __global__ void __launch_bounds__(kThreadsW, 1) head_wide_kernel(const __grid_co
 }
 
 struct MergeArgs {
-  int64_t t0;
-  int32_t Tc, V, n_part, n_traj;  // n_part partials per token (two per vocabulary block)
+  Tokens tok;
+  int32_t chunk;
+  int32_t V, n_part, n_traj;  // n_part partials per token (two per vocabulary block)
   const float4* partials;
   const int32_t* token_ids;
   const uint8_t* mask;
@@ -592,34 +600,34 @@ struct MergeArgs {
   int32_t* status;
 };
 
-// Token r's partials merged in index order (the same order in both merge kernels, so that the
-// forward-only call and the loss call agree bit for bit); the loads run 8 ahead of the merges.
+// Token r's partials, merged by a warp: lane l takes partials l, l + 32, ... in order, the lanes
+// are combined by shuffles (the same order in both merge kernels, so that the forward-only call and
+// the loss call agree bit for bit). One trip to memory per 32 partials: a thread per token walking
+// them 8 loads at a time took 16 us for 4,096 tokens and 7 us for 500 of 16 partials each.
 __device__ __forceinline__ void merge_partials(const float4* partials, int64_t Tc, int r, int n_part,
                                                SoftmaxPartial& q, float& za) {
-  constexpr int kAhead = 8;
-  for (int b0 = 0; b0 < n_part; b0 += kAhead) {
-    float4 w[kAhead];
-#pragma unroll
-    for (int k = 0; k < kAhead; ++k)
-      if (b0 + k < n_part) w[k] = partials[static_cast<int64_t>(b0 + k) * Tc + r];
-#pragma unroll
-    for (int k = 0; k < kAhead; ++k)
-      if (b0 + k < n_part) {
-        q = merge(q, SoftmaxPartial{w[k].x, w[k].y, w[k].z});
-        za += w[k].w;  // nonzero in the one partial whose columns hold the sampled id
-      }
+  const int lane = threadIdx.x & 31;
+#pragma unroll 4
+  for (int b = lane; b < n_part; b += 32) {
+    const float4 w = partials[static_cast<int64_t>(b) * Tc + r];
+    q = merge(q, SoftmaxPartial{w.x, w.y, w.z});
+    za += w.w;  // nonzero in the one partial whose columns hold the sampled id
   }
+  q = warp_merge<true>(q);
+  za = warp_sum(za);
 }
 
-// threads per CTA of the merge kernels: small CTAs spread a chunk's tokens over many SMs
-constexpr int kMergeThreads = 64;
+constexpr int kMergeThreads = 128;
+constexpr int kMergeRows = kMergeThreads / 32;
 
-// One thread per token of the chunk: merge the vocabulary blocks' partials (fixed order)
+// One warp per token of the chunk: merge the vocabulary blocks' partials (fixed order)
 // and evaluate the per-token objective terms.
 __global__ void __launch_bounds__(kMergeThreads) head_merge_kernel(const MergeArgs p) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= p.Tc) return;
-  const int64_t t = p.t0 + r;
+  const int r = static_cast<int>(blockIdx.x) * kMergeRows + static_cast<int>(threadIdx.x >> 5);
+  const bool lead = (threadIdx.x & 31) == 0;
+  const Chunk ch = chunk_of(p.tok, p.chunk);
+  if (r >= ch.count) return;
+  const int64_t t = token_of(p.tok, ch, r);
   RowCoef rc = {};
   rc.a = -1;
   bool active = p.mask[t] != 0;
@@ -627,7 +635,7 @@ __global__ void __launch_bounds__(kMergeThreads) head_merge_kernel(const MergeAr
   if (active) {
     i = p.token_traj[t];
     if (i < 0 || i >= p.n_traj) {
-      flag_status(p.status, RL_DEV_BAD_TRAJ);
+      if (lead) flag_status(p.status, RL_DEV_BAD_TRAJ);
       active = false;
     } else if (p.coef[i] == 0.f) {
       active = false;
@@ -635,10 +643,11 @@ __global__ void __launch_bounds__(kMergeThreads) head_merge_kernel(const MergeAr
   }
   const int32_t a = p.token_ids[t];
   if (active && (a < 0 || a >= p.V)) {
-    flag_status(p.status, RL_DEV_BAD_TOKEN);
+    if (lead) flag_status(p.status, RL_DEV_BAD_TOKEN);
     active = false;
   }
   if (!active) {
+    if (!lead) return;
     p.rc[r] = rc;
     p.row_loss[t] = 0.0;
     if (p.token_stats)
@@ -647,7 +656,8 @@ __global__ void __launch_bounds__(kMergeThreads) head_merge_kernel(const MergeAr
   }
   SoftmaxPartial q{-__int_as_float(0x7f800000), 0.f, 0.f};
   float za = 0.f;
-  merge_partials(p.partials, p.Tc, r, p.n_part, q, za);
+  merge_partials(p.partials, p.tok.Tc, r, p.n_part, q, za);
+  if (!lead) return;
   const float lnS = logf(q.s);
   const float lse = q.m + lnS;
   const float H = lnS - q.u / q.s;
@@ -684,7 +694,9 @@ __global__ void __launch_bounds__(kMergeThreads) head_merge_kernel(const MergeAr
 }
 
 struct DzArgs {
-  int32_t Tc, V, n_nt;
+  Tokens tok;
+  int32_t chunk;
+  int32_t V, n_nt;
   int32_t ent;
   const RowCoef* rc;
   uint16_t* dz;       // in: e = exp(z - m_j) (bf16); out: dZ (bf16)
@@ -700,9 +712,11 @@ constexpr int kMaxTilesSmem = 2048;  // V up to 524,288 keeps the row's tile fac
 // z_v = m_j + ln e_v. Rows that are not trained on become zeros. 16-byte loads and stores.
 __global__ void __launch_bounds__(kDzThreads) head_dz_kernel(const DzArgs p) {
   __shared__ float fac[kMaxTilesSmem], zoff[kMaxTilesSmem];
-  for (int r = blockIdx.x; r < p.Tc; r += gridDim.x) {
-    const RowCoef rc = p.rc[r];
-    uint16_t* row = p.dz + static_cast<int64_t>(r) * p.ldz;
+  const Chunk ch = chunk_of(p.tok, p.chunk);
+  for (int r = blockIdx.x; r < ch.padded; r += gridDim.x) {
+    RowCoef rc = {};
+    if (r < ch.count) rc = p.rc[r];  // rows past the chunk's tokens: zeros, like untrained ones
+    uint16_t* row = p.dz + static_cast<int64_t>(ch.row + r) * p.ldz;
     const int nvec = p.V / 8;
     if (!rc.active) {
       for (int k = threadIdx.x; k < nvec; k += kDzThreads) reinterpret_cast<uint4*>(row)[k] = make_uint4(0, 0, 0, 0);
@@ -754,8 +768,9 @@ __global__ void __launch_bounds__(kDzThreads) head_dz_kernel(const DzArgs p) {
 }
 
 struct LogpMergeArgs {
-  int64_t t0;
-  int32_t Tc, V, n_part;  // n_part partials per token (two per vocabulary block)
+  Tokens tok;
+  int32_t chunk;
+  int32_t V, n_part;  // n_part partials per token (two per vocabulary block)
   const float4* partials;
   const int32_t* token_ids;
   float* logp_out;
@@ -764,14 +779,17 @@ struct LogpMergeArgs {
   int32_t* status;
 };
 
-// Forward-only merge: one thread per token of the chunk writes logp, H and lse.
+// Forward-only merge: one warp per token of the chunk writes logp, H and lse.
 __global__ void __launch_bounds__(kMergeThreads) head_logp_merge_kernel(const LogpMergeArgs p) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= p.Tc) return;
-  const int64_t t = p.t0 + r;
+  const int r = static_cast<int>(blockIdx.x) * kMergeRows + static_cast<int>(threadIdx.x >> 5);
+  const bool lead = (threadIdx.x & 31) == 0;
+  const Chunk ch = chunk_of(p.tok, p.chunk);
+  if (r >= ch.count) return;
+  const int64_t t = token_of(p.tok, ch, r);
   SoftmaxPartial q{-__int_as_float(0x7f800000), 0.f, 0.f};
   float za = 0.f;
-  merge_partials(p.partials, p.Tc, r, p.n_part, q, za);
+  merge_partials(p.partials, p.tok.Tc, r, p.n_part, q, za);
+  if (!lead) return;
   const float lnS = logf(q.s);
   const float lse = q.m + lnS;
   const int32_t a = p.token_ids[t];
@@ -782,6 +800,118 @@ __global__ void __launch_bounds__(kMergeThreads) head_logp_merge_kernel(const Lo
   if (p.lse_out) p.lse_out[t] = lse;
 }
 
+// ------------------------------------------------------------------ trained tokens
+//
+// A token that is not trained on (M_t = 0, c = 0, or a bad id or owner, which is flagged) has no
+// loss and a zero gradient, so it needs none of the three products: head_select_kernel lists the
+// trained tokens in their order (and the others from the list's end), head_gather_kernel packs a
+// chunk's hidden states, and everything after it works on packed rows. On the multi-turn batch
+// (62% trained) that is 38% of the call's flops: 6,000 tokens at D = 4,096 and V = 151,936
+// 14.2 -> 11.1 ms (13.9 -> 9.3 to 10.7 ms in other runs: power, and how many tokens are trained).
+struct SelectArgs {
+  int32_t T, V, n_traj;
+  const int32_t* token_ids;
+  const uint8_t* mask;
+  const int32_t* token_traj;
+  const float* coef;
+  int32_t* idx;      // [T]
+  int32_t* n_dev;    // number of trained tokens
+  double* row_loss;  // 0 for the others
+  float* token_stats;
+  int32_t* status;
+};
+
+constexpr int kSelThreads = 1024;
+
+// One CTA per kSelThreads tokens. Each counts the trained tokens before its own by itself (mask,
+// owner and coefficient of every earlier token: 9 bytes each, from L2), which costs less than a
+// second launch until T is in the millions.
+__global__ void __launch_bounds__(kSelThreads) head_select_kernel(const SelectArgs p) {
+  __shared__ int32_t part[kSelThreads / 32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  auto trained = [&](int64_t t, bool flag) {
+    if (p.mask[t] == 0) return false;
+    const int32_t i = p.token_traj[t];
+    if (i < 0 || i >= p.n_traj) {
+      if (flag) flag_status(p.status, RL_DEV_BAD_TRAJ);
+      return false;
+    }
+    if (p.coef[i] == 0.f) return false;
+    const int32_t a = p.token_ids[t];
+    if (a < 0 || a >= p.V) {
+      if (flag) flag_status(p.status, RL_DEV_BAD_TOKEN);
+      return false;
+    }
+    return true;
+  };
+  const int64_t t0 = static_cast<int64_t>(blockIdx.x) * kSelThreads, t = t0 + tid;
+  int32_t before = 0;
+#pragma unroll 4
+  for (int64_t u = tid; u < t0; u += kSelThreads) before += trained(u, false) ? 1 : 0;
+  before = __reduce_add_sync(0xffffffffu, before);
+  if (lane == 0) part[warp] = before;
+  __syncthreads();
+  int32_t base = 0;
+  for (int w = 0; w < kSelThreads / 32; ++w) base += part[w];
+  __syncthreads();
+  const bool on = t < p.T && trained(t, true);
+  const unsigned ballot = __ballot_sync(0xffffffffu, on);
+  if (lane == 0) part[warp] = __popc(ballot);
+  __syncthreads();
+  int32_t rank = base + __popc(ballot & ((1u << lane) - 1u)), all = base;
+  for (int w = 0; w < kSelThreads / 32; ++w) {
+    if (w < warp) rank += part[w];
+    all += part[w];
+  }
+  if (t < p.T) {
+    if (on) {
+      p.idx[rank] = static_cast<int32_t>(t);
+    } else {
+      p.idx[p.T - 1 - (t - rank)] = static_cast<int32_t>(t);  // t - rank untrained tokens before it
+      p.row_loss[t] = 0.0;
+      if (p.token_stats)
+        for (int k = 0; k < 5; ++k) p.token_stats[t * 5 + k] = 0.f;
+    }
+  }
+  if (blockIdx.x == gridDim.x - 1 && tid == 0) *p.n_dev = all;
+}
+
+struct GatherArgs {
+  Tokens tok;
+  int32_t chunk;
+  int32_t D;            // a multiple of 64
+  int32_t dh_bytes;     // bytes per element of d_hidden
+  const uint16_t* hidden;
+  uint16_t* packed;     // [G Tc x D]
+  char* d_hidden;
+};
+
+// Packs the hidden states of the chunk's tokens (zeros up to `padded`, where the product over
+// tokens reads whole blocks of 64); the first chunk's launch also writes the zero d_hidden rows of
+// the tokens that are not trained on. A warp per row, 16 bytes per lane and access.
+__global__ void __launch_bounds__(256) head_gather_kernel(const GatherArgs p) {
+  const int lane = threadIdx.x & 31;
+  const Chunk ch = chunk_of(p.tok, p.chunk);
+  const int64_t warps = static_cast<int64_t>(gridDim.x) * 8;
+  const int vec = p.D / 8;
+  for (int64_t r = static_cast<int64_t>(blockIdx.x) * 8 + (threadIdx.x >> 5); r < ch.padded; r += warps) {
+    uint4* dst = reinterpret_cast<uint4*>(p.packed + (ch.row + r) * p.D);
+    if (r < ch.count) {
+      const uint4* src = reinterpret_cast<const uint4*>(p.hidden + static_cast<int64_t>(token_of(p.tok, ch, r)) * p.D);
+#pragma unroll 8
+      for (int k = lane; k < vec; k += 32) dst[k] = src[k];
+    } else {
+      for (int k = lane; k < vec; k += 32) dst[k] = make_uint4(0u, 0u, 0u, 0u);
+    }
+  }
+  if (p.chunk != 0) return;
+  const int64_t row16 = static_cast<int64_t>(p.D) * p.dh_bytes / 16;
+  for (int64_t k = *p.tok.n_dev + static_cast<int64_t>(blockIdx.x) * 8 + (threadIdx.x >> 5); k < p.tok.T; k += warps) {
+    uint4* row = reinterpret_cast<uint4*>(p.d_hidden) + p.tok.idx[k] * row16;
+    for (int64_t q = lane; q < row16; q += 32) row[q] = make_uint4(0u, 0u, 0u, 0u);
+  }
+}
+
 // ------------------------------------------------------------------ host side
 
 // bf16 matrix [rows x inner] (row stride inner), tiles of box_rows x 64 with the 128-byte swizzle.
@@ -790,23 +920,61 @@ static rl_status make_map(CUtensorMap* m, const void* base, int64_t inner, int64
                  CU_TENSOR_MAP_SWIZZLE_128B);
 }
 
+// N tiles per work item of the statistics pass. Items are 256 tokens x a block of the vocabulary;
+// blocks of 16 tiles leave few partials, but a short chunk then has fewer items than CTA pairs (500
+// tokens x 32,000 entries: 16 items on 76 pairs, 121 us). The largest of 16, 8, 4 and 2 tiles
+// whose longest pair does at most 3% more tiles than the best of them: full chunks keep 16. A
+// function of the call's token count and vocabulary alone, the same for the loss and the
+// forward-only call, so that their statistics agree bit for bit.
+static int64_t vb_tiles(int64_t Tc, int64_t n_nt) {
+  const int64_t n_m = (Tc + 2 * BM - 1) / (2 * BM);
+  auto cost = [&](int64_t vb) { return (n_m * ((n_nt + vb - 1) / vb) + kPairs - 1) / kPairs * vb; };
+  const int64_t best = std::min(std::min(cost(16), cost(8)), std::min(cost(4), cost(2)));
+  for (int64_t vb = kMaxVb; vb > 2; vb /= 2)
+    if (100 * cost(vb) <= 103 * best) return vb;
+  return 2;
+}
+
+// Parts of the contraction over V in dH = dZ W. A dH tile is 256 tokens x 512 columns over the
+// whole vocabulary, by far the longest item of the backward launch: with fewer than half as many
+// of them as CTA pairs they outlast everything else (500 tokens, D = 1,024: 4 tiles, 285 us), so
+// each is cut into parts whose fp32 sums head_combine_kernel adds in order.
+static int64_t dh_parts(int64_t Tc, int64_t V, int64_t D) {
+  const int64_t tiles = (Tc + 2 * BM - 1) / (2 * BM) * ((D + 511) / 512);
+  if (2 * tiles >= kPairs) return 1;
+  const int64_t most = std::max<int64_t>(1, V / 1024);  // at least 16 K blocks of 64 per part
+  return std::min(std::min<int64_t>(16, most), (kPairs + tiles - 1) / tiles);
+}
+
 struct Layout {
   int64_t Tc, G, n_nt, n_vb, ldz;  // G chunks per group
-  size_t off_partials, off_rc, off_tmax, off_dz, total;
+  int64_t vb, parts;               // N tiles per work item; parts of dH's contraction
+  bool pack;                       // the trained tokens are packed
+  size_t off_partials, off_rc, off_tmax, off_idx, off_h, off_parts, off_dz, total;
 };
 
 static size_t al256(size_t x) { return (x + 255) & ~size_t(255); }
 
+// What a workspace has room for: only what every call needs (every token goes through the products,
+// vocabulary blocks of 16 tiles); the packed trained tokens and the finer blocks besides; and the
+// parts of dH besides.
+enum Room { kLeast = 0, kPacked = 1, kAll = 2 };
+
 // Workspace of the loss call for up to max_rows tokens. Its smallest form (ws_bytes = 0)
-// keeps the dZ of one chunk; every further Tc x ldz x 2 bytes the caller passes keep one more
-// chunk's dZ, so that the two products run once per group of G chunks.
-static Layout layout(int64_t max_rows, int64_t V, size_t ws_bytes = 0, int64_t want_G = 0) {
+// keeps the dZ and the packed hidden states of one chunk; a caller that passes more gets as many
+// chunks of both as fit (want_G chunks of dZ, for the size query), so that the two products run
+// once per group of G chunks.
+static Layout layout(int64_t max_rows, int64_t V, int64_t D, size_t ws_bytes = 0, int64_t want_G = 0,
+                     Room room = kAll) {
+  const bool pack = room != kLeast;
   Layout L;
+  L.pack = pack;
   L.Tc = std::max<int64_t>(1, std::min<int64_t>(max_rows, kChunk));
   const int64_t chunks = (std::max<int64_t>(max_rows, 1) + L.Tc - 1) / L.Tc;
   const int64_t n_nt = (V + BN - 1) / BN;
   L.n_nt = n_nt;
-  L.n_vb = (n_nt + VB_TILES - 1) / VB_TILES;
+  L.vb = pack ? vb_tiles(L.Tc, n_nt) : kMaxVb;
+  L.n_vb = (n_nt + L.vb - 1) / L.vb;
   L.ldz = (V + 7) / 8 * 8;
   auto al = al256;
   size_t off = kWsHeader + al(static_cast<size_t>(std::max<int64_t>(max_rows, 0)) * sizeof(double));
@@ -816,14 +984,34 @@ static Layout layout(int64_t max_rows, int64_t V, size_t ws_bytes = 0, int64_t w
   off += al(static_cast<size_t>(L.Tc) * sizeof(RowCoef));
   L.off_tmax = off;
   off += al(static_cast<size_t>(L.Tc * n_nt) * sizeof(float));
-  L.off_dz = off;
+  L.off_idx = off;  // the number of trained tokens (64 words apart from the list), then the list
+  if (pack) off += 256 + al(static_cast<size_t>(std::max<int64_t>(max_rows, 1)) * sizeof(int32_t));
+  L.parts = room == kAll && max_rows <= kChunk ? dh_parts(L.Tc, V, D) : 1;
+  L.off_parts = off;
+  if (L.parts > 1) off += al(static_cast<size_t>(L.parts * L.Tc * D) * sizeof(float));
   const size_t chunk_dz = static_cast<size_t>(L.Tc * L.ldz) * 2;
-  int64_t G = std::max<int64_t>(want_G, 1);
-  if (ws_bytes > off + chunk_dz) G = static_cast<int64_t>((ws_bytes - off) / chunk_dz);
+  const size_t chunk_h = pack ? al(static_cast<size_t>(L.Tc * D) * 2) : 0;
+  int64_t G = 1;
+  if (ws_bytes > off) G = static_cast<int64_t>((ws_bytes - off) / (chunk_dz + chunk_h));
   L.G = std::max<int64_t>(1, std::min<int64_t>(G, chunks));
-  off += al(static_cast<size_t>(L.G) * chunk_dz);
+  L.off_h = off;
+  off += static_cast<size_t>(L.G) * chunk_h;
+  L.off_dz = off;
+  const int64_t dz_chunks = std::max<int64_t>(L.G, std::min<int64_t>(want_G, chunks));
+  off += al(static_cast<size_t>(dz_chunks) * chunk_dz);
   L.total = off;
   return L;
+}
+
+// The layout that a workspace of ws_bytes gives (Layout::total above ws_bytes: too small). The
+// size that rl_workspace_size gives for these T, V and D has room for everything; one made for
+// other sizes may not.
+static Layout layout_in(int64_t T, int64_t V, int64_t D, size_t ws_bytes) {
+  for (Room room : {kAll, kPacked}) {
+    const Layout L = layout(T, V, D, ws_bytes, 0, room);
+    if (L.total <= ws_bytes) return L;
+  }
+  return layout(T, V, D, ws_bytes, 0, kLeast);
 }
 
 // Which passes use the 256 x 512 form: bit 0 the forward-only statistics (STATS), bit 1 the
@@ -879,13 +1067,13 @@ static rl_status launch_head(const CUtensorMap& mh, const CUtensorMap& mw, const
   }
   if constexpr (kPair || kWide) {
     // persistent: one 2-CTA cluster per resident pair, work items of 256 tokens x one vocabulary block
-    const int items = (a.Tc + 2 * BM - 1) / (2 * BM) * a.n_vb;
+    const int items = static_cast<int>((std::min<int64_t>(a.tok.Tc, a.tok.T) + 2 * BM - 1) / (2 * BM)) * a.n_vb;
     const int pairs = std::max(1, std::min(items, max_pairs));
     cfg.gridDim = dim3(2 * pairs);
     e = cudaLaunchKernelEx(&cfg, kern, mh, mw, a);
     if (e != cudaSuccess) return cuda_error(e, "cudaLaunchKernelEx(head_kernel)");
   } else {
-    const int items = a.n_mt * a.n_vb;
+    const int items = static_cast<int>((std::min<int64_t>(a.tok.Tc, a.tok.T) + BM - 1) / BM) * a.n_vb;
     kern<<<std::min(items, sms), kThreads, smem, s>>>(mh, mw, a);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_error(e, "head_kernel launch");
@@ -896,14 +1084,12 @@ static rl_status launch_head(const CUtensorMap& mh, const CUtensorMap& mw, const
 }  // namespace head
 
 size_t head_workspace_bytes(int64_t max_rows, int64_t V, int64_t D) {
-  (void)D;
-  return head::layout(max_rows, V).total;
+  return head::layout(max_rows, V, D).total;
 }
 
 size_t head_workspace_bytes_grouped(int64_t max_rows, int64_t V, int64_t D, int64_t group_tokens) {
   const int64_t g = (std::max<int64_t>(group_tokens, 1) + head::kChunk - 1) / head::kChunk;
-  (void)D;
-  return head::layout(max_rows, V, 0, g).total;
+  return head::layout(max_rows, V, D, 0, g).total;
 }
 
 // The forward-only call needs the status word and one chunk's partials, which sit at the
@@ -913,8 +1099,7 @@ size_t head_workspace_bytes_grouped(int64_t max_rows, int64_t V, int64_t D, int6
 // 151,936: chunks of 4,096 tokens give 24.8 ms per forward-only call (70.9 ms per loss call),
 // 3,072 and 6,144 are within 2%, 8,192 takes 26.7 ms (73.1), and 32,768 takes 31.5 ms: the
 // hidden states (256 MB) then evict W's tiles from the 129 MB L2.
-static size_t head_logp_workspace_bytes(int64_t T, int64_t V) {
-  const head::Layout L = head::layout(T, V);
+static size_t head_logp_workspace_bytes(const head::Layout& L) {
   return kWsHeader + head::al256(static_cast<size_t>(head::kParts * L.n_vb * L.Tc) * sizeof(float4));
 }
 
@@ -941,7 +1126,8 @@ extern "C" rl_status rl_fused_head_loss_fwd_bwd(
     return set_error(RL_ERR_UNSUPPORTED, "rl_fused_head_loss_fwd_bwd: kl_estimator must be 0 or 3");
   if (params->token_level_adv != 0 && params->token_level_adv != 1)
     return set_error(RL_ERR_INVALID_ARG, "rl_fused_head_loss_fwd_bwd: token_level_adv must be 0 or 1");
-  if (ws_bytes < rl_workspace_size(T, V, D))
+  const Layout L = layout_in(T, V, D, ws_bytes);
+  if (ws_bytes < L.total)
     return set_error(RL_ERR_WORKSPACE_TOO_SMALL,
                      "rl_fused_head_loss_fwd_bwd: workspace smaller than rl_workspace_size(T, V, D)");
   if (T == 0) return RL_OK;
@@ -953,7 +1139,6 @@ extern "C" rl_status rl_fused_head_loss_fwd_bwd(
                      "rl_fused_head_loss_fwd_bwd: hidden, weight, d_hidden, d_weight and ws must be 16-byte aligned");
 
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  const Layout L = layout(T, V, ws_bytes);
   char* wsb = static_cast<char*>(ws);
   int32_t* status = reinterpret_cast<int32_t*>(wsb);
   double* row_loss = reinterpret_cast<double*>(wsb + ws_row_loss_offset());
@@ -968,28 +1153,71 @@ extern "C" rl_status rl_fused_head_loss_fwd_bwd(
   CUtensorMap mw;
   st = make_map(&mw, weight, D, V, kWBoxRows);
   if (st != RL_OK) return st;
-  const int n_nt = static_cast<int>((V + BN - 1) / BN);
+  const int n_nt = static_cast<int>(L.n_nt);
   const int64_t group_rows = L.G * L.Tc;
-  for (int64_t t0 = 0; t0 < T; t0 += L.Tc) {
-    const int Tc = static_cast<int>(std::min<int64_t>(L.Tc, T - t0));
-    const int64_t g0 = t0 - t0 % group_rows;  // first token of this chunk's group
-    uint16_t* dz = dz_base + (t0 - g0) * L.ldz;
-    const uint16_t* h0 = static_cast<const uint16_t*>(hidden) + t0 * D;
+  Tokens tok = {};
+  tok.T = static_cast<int32_t>(T);
+  tok.Tc = static_cast<int32_t>(L.Tc);
+  tok.G = static_cast<int32_t>(L.G);
+  uint16_t* packed = reinterpret_cast<uint16_t*>(wsb + L.off_h);
+  cudaError_t e = cudaSuccess;
+  if (L.pack) {
+    SelectArgs sa = {};
+    sa.T = tok.T;
+    sa.V = static_cast<int>(V);
+    sa.n_traj = n_traj;
+    sa.token_ids = token_ids;
+    sa.mask = mask;
+    sa.token_traj = token_traj;
+    sa.coef = coef;
+    sa.n_dev = reinterpret_cast<int32_t*>(wsb + L.off_idx);
+    sa.idx = reinterpret_cast<int32_t*>(wsb + L.off_idx + 256);
+    sa.row_loss = row_loss;
+    sa.token_stats = token_stats;
+    sa.status = status;
+    head_select_kernel<<<static_cast<unsigned>((T + kSelThreads - 1) / kSelThreads), kSelThreads, 0, s>>>(sa);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return cuda_error(e, "head_select_kernel launch");
+    tok.idx = sa.idx;
+    tok.n_dev = sa.n_dev;
+  }
+  // as many chunks as the tokens could need (the trained ones may need fewer: the kernels of a
+  // chunk without tokens return at once)
+  const int n_chunks = static_cast<int>((T + L.Tc - 1) / L.Tc);
+  for (int c = 0; c < n_chunks; ++c) {
+    const int64_t g0 = c / L.G * group_rows;  // first token of this chunk's group
+    const int64_t gn = std::min<int64_t>(group_rows, T - g0);
+    const uint16_t* h_group = L.pack ? packed : static_cast<const uint16_t*>(hidden) + g0 * D;
+    const int64_t h_rows = L.pack ? group_rows : gn;
+    const int Tc = static_cast<int>(std::min<int64_t>(L.Tc, T));
+    if (L.pack) {
+      GatherArgs ga = {};
+      ga.tok = tok;
+      ga.chunk = c;
+      ga.D = static_cast<int>(D);
+      ga.dh_bytes = d_hidden_dtype == RL_BF16 ? 2 : 4;
+      ga.hidden = static_cast<const uint16_t*>(hidden);
+      ga.packed = packed;
+      ga.d_hidden = static_cast<char*>(d_hidden);
+      head_gather_kernel<<<std::min((Tc + 7) / 8, 152 * 8), 256, 0, s>>>(ga);
+      e = cudaGetLastError();
+      if (e != cudaSuccess) return cuda_error(e, "head_gather_kernel launch");
+    }
     CUtensorMap mh;
-    st = make_map(&mh, h0, D, Tc, BM);
+    st = make_map(&mh, h_group, D, h_rows, BM);
     if (st != RL_OK) return st;
     HeadArgs ha = {};
-    ha.t0 = t0;
-    ha.Tc = Tc;
+    ha.tok = tok;
+    ha.chunk = c;
     ha.D = static_cast<int>(D);
     ha.V = static_cast<int>(V);
-    ha.n_mt = (Tc + BM - 1) / BM;
     ha.n_nt = n_nt;
+    ha.vb_tiles = static_cast<int>(L.vb);
     ha.n_vb = static_cast<int>(L.n_vb);
     ha.ent = ent ? 1 : 0;
     ha.token_ids = token_ids;
     ha.partials = partials;
-    ha.dz = dz;
+    ha.dz = dz_base;
     ha.ldz = L.ldz;
     ha.tmax = tmax;
     ha.status = status;
@@ -997,8 +1225,8 @@ extern "C" rl_status rl_fused_head_loss_fwd_bwd(
     if (st != RL_OK) return st;
 
     MergeArgs ma = {};
-    ma.t0 = t0;
-    ma.Tc = Tc;
+    ma.tok = tok;
+    ma.chunk = c;
     ma.V = static_cast<int>(V);
     ma.n_part = ha.n_vb * static_cast<int>(kParts);
     ma.n_traj = n_traj;
@@ -1021,30 +1249,30 @@ extern "C" rl_status rl_fused_head_loss_fwd_bwd(
     ma.row_loss = row_loss;
     ma.token_stats = token_stats;
     ma.status = status;
-    head_merge_kernel<<<(Tc + kMergeThreads - 1) / kMergeThreads, kMergeThreads, 0, s>>>(ma);
-    cudaError_t e = cudaGetLastError();
+    head_merge_kernel<<<(Tc + kMergeRows - 1) / kMergeRows, kMergeThreads, 0, s>>>(ma);
+    e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_error(e, "head_merge_kernel launch");
 
     DzArgs da = {};
-    da.Tc = Tc;
+    da.tok = tok;
+    da.chunk = c;
     da.V = static_cast<int>(V);
     da.n_nt = n_nt;
     da.ent = ent && params->entropy_coef != 0.f ? 1 : 0;
     da.rc = rcs;
-    da.dz = dz;
+    da.dz = dz_base;
     da.ldz = L.ldz;
     da.tmax = tmax;
     head_dz_kernel<<<std::min(Tc, 148 * 16), kDzThreads, 0, s>>>(da);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_error(e, "head_dz_kernel launch");
 
-    // after the group's last chunk, the two products over the group's n = g1 - g0 tokens
-    const int64_t g1 = std::min<int64_t>(g0 + group_rows, T);
-    if (t0 + Tc == g1) {
-      const int64_t n = g1 - g0;
-      void* dh = static_cast<char*>(d_hidden) + g0 * D * (d_hidden_dtype == RL_BF16 ? 2 : 4);
-      st = head_grad(dz_base, L.ldz, n, V, weight, static_cast<const uint16_t*>(hidden) + g0 * D, D, dh,
-                     d_hidden_dtype, d_weight, reinterpret_cast<uint32_t*>(wsb + kWsHeadCounterOffset), status, s);
+    // after the group's last chunk, the two products over the group's tokens
+    if ((c + 1) % L.G == 0 || c + 1 == n_chunks) {
+      float* parts = L.parts > 1 ? reinterpret_cast<float*>(wsb + L.off_parts) : nullptr;
+      st = head_grad(tok, static_cast<int>(c / L.G), h_rows, dz_base, L.ldz, V, weight, h_group, D, d_hidden,
+                     d_hidden_dtype, d_weight, parts, static_cast<int>(L.parts),
+                     reinterpret_cast<uint32_t*>(wsb + kWsHeadCounterOffset), status, s);
       if (st != RL_OK) return st;
     }
   }
@@ -1064,7 +1292,10 @@ extern "C" rl_status rl_fused_head_token_logprobs(const void* hidden, const void
   if (T > INT32_MAX || V > INT32_MAX || D > 65536)
     return set_error(RL_ERR_UNSUPPORTED, "rl_fused_head_token_logprobs: T or V above 2^31 - 1, or D above 65536");
   if (!ws) return set_error(RL_ERR_INVALID_ARG, "rl_fused_head_token_logprobs: NULL workspace");
-  if (ws_bytes < head_logp_workspace_bytes(T, V))
+  // the finer vocabulary blocks where their partials fit, else blocks of 16 tiles
+  Layout L = layout(T, V, D);
+  if (ws_bytes < head_logp_workspace_bytes(L)) L = layout(T, V, D, 0, 0, kLeast);
+  if (ws_bytes < head_logp_workspace_bytes(L))
     return set_error(RL_ERR_WORKSPACE_TOO_SMALL, "rl_fused_head_token_logprobs: workspace too small");
   if (T == 0) return RL_OK;
   if (!hidden || !weight || !token_ids || !logp_out)
@@ -1073,26 +1304,29 @@ extern "C" rl_status rl_fused_head_token_logprobs(const void* hidden, const void
     return set_error(RL_ERR_ALIGNMENT, "rl_fused_head_token_logprobs: hidden, weight and ws must be 16-byte aligned");
 
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  const Layout L = layout(T, V);
   char* wsb = static_cast<char*>(ws);
   int32_t* status = reinterpret_cast<int32_t*>(wsb);
   float4* partials = reinterpret_cast<float4*>(wsb + kWsHeader);
   CUtensorMap mw;
   rl_status st = make_map(&mw, weight, D, V, kWBoxRows);
   if (st != RL_OK) return st;
-  const int n_nt = static_cast<int>((V + BN - 1) / BN);
-  for (int64_t t0 = 0; t0 < T; t0 += L.Tc) {
+  Tokens tok = {};
+  tok.T = static_cast<int32_t>(T);
+  tok.Tc = static_cast<int32_t>(L.Tc);
+  tok.G = 1;
+  for (int c = 0; c * L.Tc < T; ++c) {
+    const int64_t t0 = c * L.Tc;
     const int Tc = static_cast<int>(std::min<int64_t>(L.Tc, T - t0));
     CUtensorMap mh;
     st = make_map(&mh, static_cast<const uint16_t*>(hidden) + t0 * D, D, Tc, BM);
     if (st != RL_OK) return st;
     HeadArgs ha = {};
-    ha.t0 = t0;
-    ha.Tc = Tc;
+    ha.tok = tok;
+    ha.chunk = c;
     ha.D = static_cast<int>(D);
     ha.V = static_cast<int>(V);
-    ha.n_mt = (Tc + BM - 1) / BM;
-    ha.n_nt = n_nt;
+    ha.n_nt = static_cast<int>(L.n_nt);
+    ha.vb_tiles = static_cast<int>(L.vb);
     ha.n_vb = static_cast<int>(L.n_vb);
     ha.ent = entropy_out ? 1 : 0;
     ha.token_ids = token_ids;
@@ -1101,8 +1335,8 @@ extern "C" rl_status rl_fused_head_token_logprobs(const void* hidden, const void
     st = launch_head<STATS>(mh, mw, ha, s);
     if (st != RL_OK) return st;
     LogpMergeArgs ma = {};
-    ma.t0 = t0;
-    ma.Tc = Tc;
+    ma.tok = tok;
+    ma.chunk = c;
     ma.V = static_cast<int>(V);
     ma.n_part = ha.n_vb * static_cast<int>(kParts);
     ma.partials = partials;
@@ -1111,7 +1345,7 @@ extern "C" rl_status rl_fused_head_token_logprobs(const void* hidden, const void
     ma.entropy_out = entropy_out;
     ma.lse_out = lse_out;
     ma.status = status;
-    head_logp_merge_kernel<<<(Tc + kMergeThreads - 1) / kMergeThreads, kMergeThreads, 0, s>>>(ma);
+    head_logp_merge_kernel<<<(Tc + kMergeRows - 1) / kMergeRows, kMergeThreads, 0, s>>>(ma);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_error(e, "head_logp_merge_kernel launch");
   }

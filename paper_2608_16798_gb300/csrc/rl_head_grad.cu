@@ -36,6 +36,7 @@
 #include <utility>
 
 #include "rl_device.cuh"
+#include "rl_head_tokens.cuh"
 #include "rl_host.h"
 #include "rl_tc.cuh"
 #include "rl_tmap.h"
@@ -62,10 +63,15 @@ static_assert(kSmem <= 232448 - 1024, "shared memory of the backward kernel");
 constexpr uint32_t kItemReaders = 10;
 
 struct GradArgs {
-  int32_t n_h;           // dH tiles: row tiles x n_nt
+  Tokens tok;
+  int32_t group;         // which group of tokens
+  int32_t D;
   int32_t n_w;           // dW tiles: row tiles x n_nt
   int32_t n_nt;          // 512-column tiles of D
-  int32_t nkb_h, nkb_w;  // 64-element K blocks: over V (dH), over the tokens (dW)
+  int32_t nkb_h;         // 64-element K blocks over V (dH)
+  int32_t parts;         // parts of that contraction, each an item
+  float* part_sums;      // [parts][Tc x D] with parts > 1 (one chunk per group then)
+  void* d_hidden;        // [T x D]
   uint32_t* counter;     // work-item counter (zero at launch)
   int32_t* status;
 };
@@ -76,8 +82,8 @@ enum HOut { H_F32 = 0, H_BF16 = 1 };
 template <int HO>
 __global__ void __launch_bounds__(kThreads, 1) head_grad_kernel(
     const __grid_constant__ CUtensorMap tmAh, const __grid_constant__ CUtensorMap tmBh,
-    const __grid_constant__ CUtensorMap tmOh, const __grid_constant__ CUtensorMap tmAw,
-    const __grid_constant__ CUtensorMap tmBw, const __grid_constant__ CUtensorMap tmOw, const GradArgs p) {
+    const __grid_constant__ CUtensorMap tmAw, const __grid_constant__ CUtensorMap tmBw,
+    const __grid_constant__ CUtensorMap tmOw, const GradArgs p) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full[NS], empty[NS], accf, acce, ifull[NR], iempty[NR];
   __shared__ int32_t ring[NR];
@@ -86,7 +92,13 @@ __global__ void __launch_bounds__(kThreads, 1) head_grad_kernel(
   uint8_t* slabs = sm + NS * STAGE_BYTES;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
-  const int n_items = p.n_h + p.n_w;
+  // the group's tokens, its dH tiles (row tiles x n_nt) and the dW tiles' K blocks
+  const Chunk grp = group_of(p.tok, p.group);
+  if (grp.count == 0) return;  // the whole grid: nothing to add
+  const int n_h1 = (grp.count + 2 * BM - 1) / (2 * BM) * p.n_nt;
+  const int n_h = n_h1 * p.parts;
+  const int nkb_w = (grp.count + BK - 1) / BK;
+  const int n_items = n_h + p.n_w;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < NS; ++s) {
@@ -107,14 +119,17 @@ __global__ void __launch_bounds__(kThreads, 1) head_grad_kernel(
   tc::fence_after_sync();
   const uint32_t tmem = tbase;
 
-  // item -> (dW?, tile row, tile column, K blocks); columns fastest
-  const int n_h = p.n_h, n_nt = p.n_nt, nkb_h = p.nkb_h, nkb_w = p.nkb_w;
-  auto decode = [n_h, n_nt, nkb_h, nkb_w](int item, bool& w, int& mt, int& nt, int& nkb) {
+  // item -> (dW?, tile row, tile column, first K block, K blocks); columns fastest, then rows, then
+  // the parts of dH's contraction
+  const int n_nt = p.n_nt, nkb_h = p.nkb_h, parts = p.parts;
+  auto decode = [=](int item, bool& w, int& mt, int& nt, int& kb0, int& nkb) {
     w = item >= n_h;
-    const int r = w ? item - n_h : item;
+    const int part = w ? 0 : item / n_h1;
+    const int r = w ? item - n_h : item % n_h1;
     mt = r / n_nt;
     nt = r % n_nt;
-    nkb = w ? nkb_w : nkb_h;
+    kb0 = static_cast<int>(static_cast<int64_t>(part) * nkb_h / parts);
+    nkb = w ? nkb_w : static_cast<int>(static_cast<int64_t>(part + 1) * nkb_h / parts) - kb0;
   };
   // Read the k-th published item (every role but the even CTA's producer): -1 if the wait
   // ran out.
@@ -159,13 +174,14 @@ __global__ void __launch_bounds__(kThreads, 1) head_grad_kernel(
         }
         if (item >= n_items) break;
         bool w;
-        int mt, nt, nkb;
-        decode(item, w, mt, nt, nkb);
+        int mt, nt, kb0, nkb;
+        decode(item, w, mt, nt, kb0, nkb);
         const int m0 = mt * 2 * BM + static_cast<int>(rank) * BM;
         const int n0 = nt * NB + static_cast<int>(rank) * 128;
         const CUtensorMap* mb = w ? &tmBw : &tmBh;
         for (int kb = 0; kb < nkb; ++kb, ++g) {
           const int s = g % NS;
+          const int k0 = (kb0 + kb) * BK;
           const uint32_t use = g / NS;
           if (use > 0 && !mbar_wait_bounded(&empty[s], (use - 1) & 1)) {
             flag_status(p.status, RL_DEV_TIMEOUT);
@@ -176,16 +192,16 @@ __global__ void __launch_bounds__(kThreads, 1) head_grad_kernel(
           if (rank == 0) mbar_arrive_expect_tx(&full[s], 2 * STAGE_BYTES);  // both CTAs' bytes
           const uint32_t bar = map_to_rank(smem_addr(&full[s]), 0);
           if (w) {
-            tc::tma_load_2d_pair(st, &tmAw, m0, kb * BK, bar);
-            tc::tma_load_2d_pair(st + HALF_BYTES, &tmAw, m0 + 64, kb * BK, bar);
+            tc::tma_load_2d_pair(st, &tmAw, m0, k0, bar);
+            tc::tma_load_2d_pair(st + HALF_BYTES, &tmAw, m0 + 64, k0, bar);
           } else {
-            tc::tma_load_2d_pair(st, &tmAh, kb * BK, m0, bar);
+            tc::tma_load_2d_pair(st, &tmAh, k0, m0, bar);
           }
 #pragma unroll
           for (int h = 0; h < NH; ++h) {
             uint8_t* sb = st + A_BYTES + h * 2 * HALF_BYTES;
-            tc::tma_load_2d_pair(sb, mb, n0 + h * 256, kb * BK, bar);
-            tc::tma_load_2d_pair(sb + HALF_BYTES, mb, n0 + h * 256 + 64, kb * BK, bar);
+            tc::tma_load_2d_pair(sb, mb, n0 + h * 256, k0, bar);
+            tc::tma_load_2d_pair(sb + HALF_BYTES, mb, n0 + h * 256 + 64, k0, bar);
           }
         }
       }
@@ -204,8 +220,8 @@ __global__ void __launch_bounds__(kThreads, 1) head_grad_kernel(
         }
         if (item >= n_items) break;
         bool w;
-        int mt, nt, nkb;
-        decode(item, w, mt, nt, nkb);
+        int mt, nt, kb0, nkb;
+        decode(item, w, mt, nt, kb0, nkb);
         if (t > 0 && !mbar_wait_cluster_bounded(&acce, (t - 1) & 1)) {
           flag_status(p.status, RL_DEV_TIMEOUT);
           break;
@@ -254,14 +270,23 @@ __global__ void __launch_bounds__(kThreads, 1) head_grad_kernel(
       }
       if (item >= n_items) break;
       bool w;
-      int mt, nt, nkb;
-      decode(item, w, mt, nt, nkb);
+      int mt, nt, kb0, nkb;
+      decode(item, w, mt, nt, kb0, nkb);
       if (!mbar_wait_sleep_bounded(&accf, t & 1)) {
         if (lane == 0) flag_status(p.status, RL_DEV_TIMEOUT);
         break;
       }
       tc::fence_after_sync();
       const int row0 = mt * 2 * BM + static_cast<int>(rank) * BM + 32 * q;
+      // dH: lane l holds row row0 + l, which goes straight to its token's row of d_hidden, or, as
+      // one of several parts, to its row of the part's sums
+      const int hr = row0 + lane;
+      const bool h_ok = !w && hr < grp.count;
+      const bool in_parts = parts > 1;
+      int64_t h_at = 0;
+      if (h_ok)
+        h_at = (in_parts ? static_cast<int64_t>(item / n_h1) * p.tok.Tc + hr
+                         : static_cast<int64_t>(token_of(p.tok, grp, hr))) * p.D + nt * NB;
 #pragma unroll 1
       for (int c = 0; c < NB / 32; ++c) {
         float v[32];
@@ -275,31 +300,38 @@ __global__ void __launch_bounds__(kThreads, 1) head_grad_kernel(
             else mbar_arrive(&acce);
           }
         }
+        if (!w) {
+          if (h_ok && nt * NB + c * 32 < p.D) {  // neither past the tokens nor past D's last tile
+            if (HO == H_BF16 && !in_parts) {
+              uint16_t* out = static_cast<uint16_t*>(p.d_hidden) + h_at + c * 32;
+#pragma unroll
+              for (int j = 0; j < 4; ++j)
+                *reinterpret_cast<uint4*>(out + 8 * j) =
+                    make_uint4(pack_bf16x2(v[8 * j], v[8 * j + 1]), pack_bf16x2(v[8 * j + 2], v[8 * j + 3]),
+                               pack_bf16x2(v[8 * j + 4], v[8 * j + 5]), pack_bf16x2(v[8 * j + 6], v[8 * j + 7]));
+            } else {
+              float* out = (in_parts ? p.part_sums : static_cast<float*>(p.d_hidden)) + h_at + c * 32;
+#pragma unroll
+              for (int j = 0; j < 8; ++j)
+                *reinterpret_cast<float4*>(out + 4 * j) =
+                    make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+            }
+          }
+          __syncwarp();  // the next TMEM load is the whole warp's
+          continue;
+        }
         uint8_t* sb = my + buf * SLAB_BYTES;
         if (lane == 0) tc::bulk_wait_read_1();  // the slab's previous TMA has read it
         __syncwarp();
-        if (!w && HO == H_BF16) {
-          // 32 rows x 64 bytes, 64-byte swizzle: 16-byte chunk j of row r at chunk j ^ ((r / 2) % 4)
+        // 32 rows x 128 bytes, 128-byte swizzle: 16-byte chunk j of row r at chunk j ^ (r % 8)
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const uint4 u = make_uint4(pack_bf16x2(v[8 * j], v[8 * j + 1]), pack_bf16x2(v[8 * j + 2], v[8 * j + 3]),
-                                       pack_bf16x2(v[8 * j + 4], v[8 * j + 5]),
-                                       pack_bf16x2(v[8 * j + 6], v[8 * j + 7]));
-            *reinterpret_cast<uint4*>(sb + lane * 64 + ((j ^ ((lane >> 1) & 3)) << 4)) = u;
-          }
-        } else {
-          // 32 rows x 128 bytes, 128-byte swizzle: 16-byte chunk j of row r at chunk j ^ (r % 8)
-#pragma unroll
-          for (int j = 0; j < 8; ++j)
-            *reinterpret_cast<float4*>(sb + lane * 128 + ((j ^ (lane & 7)) << 4)) =
-                make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
-        }
+        for (int j = 0; j < 8; ++j)
+          *reinterpret_cast<float4*>(sb + lane * 128 + ((j ^ (lane & 7)) << 4)) =
+              make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
         fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) {
-          const int col = nt * NB + c * 32;
-          if (w) tc::tma_reduce_add_2d(&tmOw, col, row0, sb);
-          else tc::tma_store_2d(&tmOh, col, row0, sb);
+          tc::tma_reduce_add_2d(&tmOw, nt * NB + c * 32, row0, sb);
           bulk_commit();
         }
         buf ^= 1;
@@ -315,35 +347,67 @@ __global__ void __launch_bounds__(kThreads, 1) head_grad_kernel(
   }
 }
 
+// dH from its parts: the fp32 sums of the parts of the contraction over V added in order, into the
+// token's row of d_hidden. Grid-stride over rows, four columns per thread and step.
+template <int HO>
+__global__ void __launch_bounds__(256) head_combine_kernel(const GradArgs p) {
+  const Chunk grp = group_of(p.tok, p.group);
+  const int64_t per_part = static_cast<int64_t>(p.tok.Tc) * p.D;
+  for (int r = blockIdx.x; r < grp.count; r += gridDim.x) {
+    const int64_t to = static_cast<int64_t>(token_of(p.tok, grp, r)) * p.D;
+    for (int c = threadIdx.x * 4; c < p.D; c += 1024) {
+      const float* src = p.part_sums + static_cast<int64_t>(r) * p.D + c;
+      float4 a = *reinterpret_cast<const float4*>(src);
+#pragma unroll 4
+      for (int k = 1; k < p.parts; ++k) {
+        const float4 b = *reinterpret_cast<const float4*>(src + k * per_part);
+        a.x += b.x;
+        a.y += b.y;
+        a.z += b.z;
+        a.w += b.w;
+      }
+      if (HO == H_BF16)
+        *reinterpret_cast<uint2*>(static_cast<uint16_t*>(p.d_hidden) + to + c) =
+            make_uint2(pack_bf16x2(a.x, a.y), pack_bf16x2(a.z, a.w));
+      else
+        *reinterpret_cast<float4*>(static_cast<float*>(p.d_hidden) + to + c) = a;
+    }
+  }
+}
+
 }  // namespace grad
 
-rl_status head_grad(const uint16_t* dz, int64_t ldz, int64_t n, int64_t V, const void* weight, const void* hidden,
-                    int64_t D, void* d_hidden, rl_dtype dh_dtype, float* d_weight, uint32_t* counter,
-                    int32_t* status, cudaStream_t s) {
+rl_status head_grad(const Tokens& tok, int group, int64_t rows, const uint16_t* dz, int64_t ldz, int64_t V,
+                    const void* weight, const void* hidden, int64_t D, void* d_hidden, rl_dtype dh_dtype,
+                    float* d_weight, float* part_sums, int parts, uint32_t* counter, int32_t* status,
+                    cudaStream_t s) {
   using namespace grad;
-  CUtensorMap ah, bh, oh, aw, bw, ow;
+  CUtensorMap ah, bh, aw, bw, ow;
   const bool bf16 = dh_dtype == RL_BF16;
-  rl_status st = tmap_2d(&ah, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, dz, V, n, ldz * 2, BK, BM, CU_TENSOR_MAP_SWIZZLE_128B);
+  rl_status st =
+      tmap_2d(&ah, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, dz, V, rows, ldz * 2, BK, BM, CU_TENSOR_MAP_SWIZZLE_128B);
   if (st == RL_OK)
     st = tmap_2d(&bh, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, weight, D, V, D * 2, 64, BK, CU_TENSOR_MAP_SWIZZLE_128B);
   if (st == RL_OK)
-    st = bf16 ? tmap_2d(&oh, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, d_hidden, D, n, D * 2, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B)
-              : tmap_2d(&oh, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, d_hidden, D, n, D * 4, 32, 32, CU_TENSOR_MAP_SWIZZLE_128B);
+    st = tmap_2d(&aw, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, dz, V, rows, ldz * 2, 64, BK, CU_TENSOR_MAP_SWIZZLE_128B);
   if (st == RL_OK)
-    st = tmap_2d(&aw, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, dz, V, n, ldz * 2, 64, BK, CU_TENSOR_MAP_SWIZZLE_128B);
-  if (st == RL_OK)
-    st = tmap_2d(&bw, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, hidden, D, n, D * 2, 64, BK, CU_TENSOR_MAP_SWIZZLE_128B);
+    st = tmap_2d(&bw, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, hidden, D, rows, D * 2, 64, BK, CU_TENSOR_MAP_SWIZZLE_128B);
   if (st == RL_OK)
     st = tmap_2d(&ow, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, d_weight, D, V, D * 4, 32, 32, CU_TENSOR_MAP_SWIZZLE_128B);
   if (st != RL_OK) return st;
   GradArgs a = {};
+  a.tok = tok;
+  a.group = group;
+  a.D = static_cast<int32_t>(D);
   a.n_nt = static_cast<int32_t>((D + NB - 1) / NB);
-  a.n_h = static_cast<int32_t>((n + 2 * BM - 1) / (2 * BM)) * a.n_nt;
   a.n_w = static_cast<int32_t>((V + 2 * BM - 1) / (2 * BM)) * a.n_nt;
   a.nkb_h = static_cast<int32_t>((V + BK - 1) / BK);
-  a.nkb_w = static_cast<int32_t>((n + BK - 1) / BK);
+  a.parts = parts;
+  a.part_sums = part_sums;
+  a.d_hidden = d_hidden;
   a.counter = counter;
   a.status = status;
+  const int32_t n_h = static_cast<int32_t>((rows + 2 * BM - 1) / (2 * BM)) * a.n_nt * parts;  // at most
 
   cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(uint32_t), s);
   if (e != cudaSuccess) return cuda_error(e, "cudaMemsetAsync(work counter)");
@@ -382,9 +446,15 @@ rl_status head_grad(const uint16_t* dz, int64_t ldz, int64_t n, int64_t V, const
     max_pairs = it->second;
   }
   // persistent: at most as many pairs as fit on the device at once, and no more than items
-  cfg.gridDim = dim3(2 * std::max(1, std::min(a.n_h + a.n_w, max_pairs)));
-  e = cudaLaunchKernelEx(&cfg, kern, ah, bh, oh, aw, bw, ow, a);
+  cfg.gridDim = dim3(2 * std::max(1, std::min(n_h + a.n_w, max_pairs)));
+  e = cudaLaunchKernelEx(&cfg, kern, ah, bh, aw, bw, ow, a);
   if (e != cudaSuccess) return cuda_error(e, "cudaLaunchKernelEx(head_grad_kernel)");
+  if (parts > 1) {
+    auto combine = bf16 ? head_combine_kernel<H_BF16> : head_combine_kernel<H_F32>;
+    combine<<<static_cast<unsigned>(std::min<int64_t>(rows, 152 * 8)), 256, 0, s>>>(a);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return cuda_error(e, "head_combine_kernel launch");
+  }
   return RL_OK;
 }
 

@@ -42,13 +42,19 @@ size_t head_workspace_bytes(int64_t max_rows, int64_t V, int64_t D);
 // The same, keeping the dZ of up to group_tokens tokens (whole chunks) at once.
 size_t head_workspace_bytes_grouped(int64_t max_rows, int64_t V, int64_t D, int64_t group_tokens);
 
-// Backward products of the fused LM head on the tensor cores (rl_head_grad.cu), one launch:
-// d_hidden[n x D] = dZ W (stored, bf16 or fp32) and d_weight[V x D] += dZ^T H[n x D] (fp32),
-// with dz the bf16 gradient of the logits of the n tokens ([n x V], rows ldz elements apart).
-// counter: a workspace word for the work-item counter (zeroed here, on the stream).
-rl_status head_grad(const uint16_t* dz, int64_t ldz, int64_t n, int64_t V, const void* weight, const void* hidden,
-                    int64_t D, void* d_hidden, rl_dtype dh_dtype, float* d_weight, uint32_t* counter,
-                    int32_t* status, cudaStream_t s);
+struct Tokens;  // rl_head_tokens.cuh
+
+// Backward products of the fused LM head on the tensor cores (rl_head_grad.cu), one launch over
+// the n tokens of one group: d_hidden = dZ W (stored in the tokens' rows, bf16 or fp32) and
+// d_weight[V x D] += dZ^T H[n x D] (fp32), with dz the bf16 gradient of the logits of the group's
+// tokens ([rows x V] at most, rows ldz elements apart) and hidden their hidden states in the same
+// order. parts > 1 cuts dH's contraction over V into that many items per tile, whose fp32 sums
+// ([parts][Tc x D] at part_sums) a second launch adds. counter: a workspace word for the work-item
+// counter (zeroed here, on the stream).
+rl_status head_grad(const Tokens& tok, int group, int64_t rows, const uint16_t* dz, int64_t ldz, int64_t V,
+                    const void* weight, const void* hidden, int64_t D, void* d_hidden, rl_dtype dh_dtype,
+                    float* d_weight, float* part_sums, int parts, uint32_t* counter, int32_t* status,
+                    cudaStream_t s);
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
