@@ -310,21 +310,38 @@ __device__ __forceinline__ void fold_block(SoftmaxPartial& ps, const uint4 (&x)[
   ps.s = fmaf(se, f, ps.s);
 }
 
-// Log-sum-exp of a row's merged partial as hi + lo. bf16: lo is what the rounding of m + ln S and of
-// the logarithm leave out (the latter from S e^-lnS = 1 + it), so that the ratio exp(logp - old) is
-// off by the error of S alone; fp32 keeps its order of operations: lo = 0.
+// Log-sum-exp of a row's merged partial as hi + lo. SPLIT: lo is what the rounding of m + ln S and
+// of the logarithm leave out (the latter from S e^-lnS = 1 + it), so that the ratio exp(logp - old) is
+// off by the error of S alone; without it lo = 0 and the order of operations is the plain one.
 struct RowLse {
   float lnS, hi, lo;
 };
-template <typename T>
+template <bool SPLIT>
 __device__ __forceinline__ RowLse row_lse(const SoftmaxPartial& q) {
   RowLse l{logf(q.s), 0.f, 0.f};
   l.hi = q.m + l.lnS;
-  if constexpr (sizeof(T) == 2) {
+  if constexpr (SPLIT) {
     const float b = l.hi - q.m;
     l.lo = (q.m - (l.hi - b)) + (l.lnS - b) + fmaf(q.s, expf(-l.lnS), -1.f);
   }
   return l;
+}
+
+// logp - old: large operands are differenced first. SPLIT: with what the rounding of z_a - old leaves
+// out, which is up to 5e-7 where the log-prob is about -10. With row_lse's lo the loss of 512 rows of
+// 4,096 bf16 entries, a sum that nearly cancels, is off by 1.2e-6 on average over 60 seeds (4.6e-6
+// without either), and the gradient of fp32 rows of 151,936 entries by 1.9e-7 (5.0e-7).
+template <bool SPLIT>
+__device__ __forceinline__ float log_ratio(float za, float old, const RowLse& l) {
+  const float d = za - old;
+  if constexpr (SPLIT) {
+    const float b = d - za;
+    const float rest = (za - (d - b)) - (old + b);
+    const float x = (d - l.hi) + (rest - l.lo);
+    return fabsf(rest) <= 1.f ? x : (d - l.hi) - l.lo;  // infinities leave no rest
+  } else {
+    return (d - l.hi) - l.lo;
+  }
 }
 
 // The warp's 32 partials of a row of the loss kernels. bf16: the short chain. fp32: by pairs, whose
@@ -350,6 +367,7 @@ template <typename T, int NW, bool ENT, int HOLDV, int MINB, bool SHIFT>
 __global__ void __launch_bounds__((NW + 1) * 32, MINB) rows_kernel(const RowArgs p) {
   constexpr bool kBlocks = sizeof(T) == 2;
   static_assert(!(kBlocks && SHIFT), "bf16 rows are cut into blocks");
+  constexpr bool kSplit = kBlocks || NW >= 16;  // not where fp32 keeps its bits (merge_lanes)
   constexpr int kZeroBytes = MINB >= 3 ? 2048 : kZeroBytesMax;
   constexpr int EPV = Vec<T>::N;
   constexpr int NB = RL_STAGES;
@@ -712,7 +730,7 @@ __global__ void __launch_bounds__((NW + 1) * 32, MINB) rows_kernel(const RowArgs
       }
       q = merge_lanes<T, ENT>(q);  // the same in every lane
       const float za = warp_sum(zsum);
-      const RowLse rl = row_lse<T>(q);
+      const RowLse rl = row_lse<kSplit>(q);
       const float lnS = rl.lnS, lse = rl.hi;
       const float H = ENT || sizeof(T) == 4 ? lnS - q.u / q.s : 0.f;  // times 0 without the entropy
 
@@ -720,7 +738,7 @@ __global__ void __launch_bounds__((NW + 1) * 32, MINB) rows_kernel(const RowArgs
         // per-token scalars (every lane computes the same values)
         const float A = m.A, c = m.c, old = m.old;
         const float logp = (za - lse) - rl.lo;
-        const float rho = expf(((za - old) - lse) - rl.lo);   // large operands differenced first
+        const float rho = expf(log_ratio<kSplit>(za, old, rl));
         const float crho = fminf(fmaxf(rho, p.clip_lo), p.clip_hi);
         const float surr = fminf(rho * A, crho * A);
         const bool cut = (A > 0.f && rho > p.clip_hi) || (A < 0.f && rho < p.clip_lo);
@@ -1108,7 +1126,7 @@ __global__ void __launch_bounds__((kF32Warps + 1) * 32, 3) rows_f32_kernel(const
       }
       q = merge_lanes<T, ENT>(q);  // the same in every lane
       const float za = warp_sum(zsum);
-      const RowLse rl = row_lse<T>(q);
+      const RowLse rl = row_lse<false>(q);
       const float lnS = rl.lnS, lse = rl.hi;
       const float H = ENT || sizeof(T) == 4 ? lnS - q.u / q.s : 0.f;  // times 0 without the entropy
 
@@ -1116,7 +1134,7 @@ __global__ void __launch_bounds__((kF32Warps + 1) * 32, 3) rows_f32_kernel(const
         // per-token scalars (every lane computes the same values)
         const float A = m.A, c = m.c, old = m.old;
         const float logp = (za - lse) - rl.lo;
-        const float rho = expf(((za - old) - lse) - rl.lo);   // large operands differenced first
+        const float rho = expf(log_ratio<false>(za, old, rl));
         const float crho = fminf(fmaxf(rho, p.clip_lo), p.clip_hi);
         const float surr = fminf(rho * A, crho * A);
         const bool cut = (A > 0.f && rho > p.clip_hi) || (A < 0.f && rho < p.clip_lo);
@@ -1291,6 +1309,7 @@ struct SmallRow {
 
 template <typename T, bool ENT, int NV>
 __global__ void __launch_bounds__(kSmallWarps * 32, small_ctas<T, NV>(true)) small_rows_kernel(const RowArgs p) {
+  constexpr bool kSplit = sizeof(T) == 2;
   constexpr int EPV = Vec<T>::N;
   __shared__ double warp_loss[kSmallWarps];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1355,13 +1374,13 @@ __global__ void __launch_bounds__(kSmallWarps * 32, small_ctas<T, NV>(true)) sma
     }
     // ---- pass 1
     const SoftmaxPartial q = sr.template fold<ENT>(lane);
-    const RowLse rl = row_lse<T>(q);
+    const RowLse rl = row_lse<kSplit>(q);
     const float lnS = rl.lnS, lse = rl.hi;
     const float H = ENT ? lnS - q.u / q.s : 0.f;
     // ---- per-token scalars (every lane computes the same values)
     const float old = wd.old;
     const float logp = (za - lse) - rl.lo;
-    const float rho = expf(((za - old) - lse) - rl.lo);  // large operands differenced first
+    const float rho = expf(log_ratio<kSplit>(za, old, rl));
     const float crho = fminf(fmaxf(rho, p.clip_lo), p.clip_hi);
     const float surr = fminf(rho * A, crho * A);
     const bool cut = (A > 0.f && rho > p.clip_hi) || (A < 0.f && rho < p.clip_lo);
