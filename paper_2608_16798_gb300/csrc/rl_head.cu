@@ -11,16 +11,15 @@
 //      its row maximum m_j, then e = exp(z - m_j), which it stores (bf16) in the chunk's
 //      dZ buffer, with m_j per token and tile, and folds into per-row online-softmax
 //      partials: two per vocabulary block (its even and its odd tiles).
-//   2. head_merge_kernel    one warp per token: merges the partials into lse, entropy and
-//      logp, evaluates the objective's per-token terms (same readings as the logits path),
-//      writes the row's loss contribution and the coefficients of dZ.
-//   3. head_dz_kernel       rescales the stored e in place into
+//   2. head_dz_kernel       merges each token's partials into lse, entropy and logp (one warp),
+//      evaluates the objective's per-token terms (same readings as the logits path), writes the
+//      token's loss contribution, and rescales the stored e in place into
 //      dZ = c [g (delta_a - p) + alpha p (log p + H)], p = e exp(m_j - lse) (HBM-bound: the
-//      logits are formed once, not twice).
+//      logits are formed once, not twice); the last CTA of the last chunk sums the loss.
 // The dZ of one chunk (4,096 tokens x V in bf16) is the only logits-sized buffer; a caller
 // that passes more workspace lets a group of several chunks keep their dZ side by side.
 // After the group's last chunk (every chunk, with the smallest workspace):
-//   4. dH = dZ W and dW += dZ^T H over the group in one persistent launch of
+//   3. dH = dZ W and dW += dZ^T H over the group in one persistent launch of
 //      head_grad_kernel (rl_head_grad.cu): CTA-pair tcgen05 MMAs on 256 x 512 tiles with the
 //      operands in their row-major layouts (dZ K-major for dH, MN-major for dW; W and H
 //      MN-major), dH tiles first and dW tiles after them, handed out by a work counter; dH rows
@@ -84,7 +83,6 @@ struct RowCoef {
   float Ke;
   int32_t a;
   int32_t active;
-  float pad;
 };
 
 struct HeadArgs {
@@ -579,11 +577,16 @@ __global__ void __launch_bounds__(kThreadsW, 1) head_wide_kernel(const __grid_co
   }
 }
 
-struct MergeArgs {
+struct DzArgs {
   Tokens tok;
   int32_t chunk;
-  int32_t V, n_part, n_traj;  // n_part partials per token (two per vocabulary block)
+  int32_t V, n_nt, n_part, n_traj;  // n_part partials per token (two per vocabulary block)
+  int32_t split;                    // CTAs per row
+  int32_t ent;                      // the entropy term is in the gradient
   const float4* partials;
+  const float* tmax;                // [Tc x n_nt]
+  uint16_t* dz;                     // in: e = exp(z - m_j) (bf16); out: dZ (bf16)
+  int64_t ldz;
   const int32_t* token_ids;
   const uint8_t* mask;
   const int32_t* token_traj;
@@ -594,8 +597,10 @@ struct MergeArgs {
   const float* rollout_logp;
   float clip_lo, clip_hi, beta, alpha, tis_cap;
   int32_t adv_per_row;  // adv holds one A_t per token (else one per trajectory)
-  RowCoef* rc;
-  double* row_loss;
+  double* row_loss;     // [T]
+  double* loss_accum;   // the caller's total in the call's last chunk, else null
+  uint32_t* done;       // finished-CTA count in the workspace header
+  uint32_t* counter;    // the products' work counter, set back here for their next launch
   float* token_stats;
   int32_t* status;
 };
@@ -620,57 +625,58 @@ __device__ __forceinline__ void merge_partials(const float4* partials, int64_t T
 constexpr int kMergeThreads = 128;
 constexpr int kMergeRows = kMergeThreads / 32;
 
-// One warp per token of the chunk: merge the vocabulary blocks' partials (fixed order)
-// and evaluate the per-token objective terms.
-__global__ void __launch_bounds__(kMergeThreads) head_merge_kernel(const MergeArgs p) {
-  const int r = static_cast<int>(blockIdx.x) * kMergeRows + static_cast<int>(threadIdx.x >> 5);
-  const bool lead = (threadIdx.x & 31) == 0;
-  const Chunk ch = chunk_of(p.tok, p.chunk);
-  if (r >= ch.count) return;
+// Row r's coefficients, by one warp (the same in every lane): the vocabulary blocks' partials merged
+// in a fixed order and the per-token objective terms. With `write` lane 0 also writes the token's
+// loss contribution and statistics. The words that need only the token are loaded together.
+__device__ __forceinline__ RowCoef row_coef(const DzArgs& p, const Chunk& ch, int r, bool write) {
   const int64_t t = token_of(p.tok, ch, r);
-  RowCoef rc = {};
-  rc.a = -1;
-  bool active = p.mask[t] != 0;
-  int32_t i = 0;
-  if (active) {
-    i = p.token_traj[t];
-    if (i < 0 || i >= p.n_traj) {
-      if (lead) flag_status(p.status, RL_DEV_BAD_TRAJ);
-      active = false;
-    } else if (p.coef[i] == 0.f) {
-      active = false;
-    }
-  }
-  const int32_t a = p.token_ids[t];
-  if (active && (a < 0 || a >= p.V)) {
-    if (lead) flag_status(p.status, RL_DEV_BAD_TOKEN);
-    active = false;
-  }
-  if (!active) {
-    if (!lead) return;
-    p.rc[r] = rc;
-    p.row_loss[t] = 0.0;
-    if (p.token_stats)
-      for (int k = 0; k < 5; ++k) p.token_stats[t * 5 + k] = 0.f;
-    return;
-  }
+  const uint8_t m = p.mask[t];
+  const int32_t i = p.token_traj[t], a = p.token_ids[t];
+  const float old = p.old_logp[t];
+  const float ref = p.ref_logp ? p.ref_logp[t] : 0.f;
+  const float roll = p.rollout_logp ? p.rollout_logp[t] : 0.f;
   SoftmaxPartial q{-__int_as_float(0x7f800000), 0.f, 0.f};
   float za = 0.f;
   merge_partials(p.partials, p.tok.Tc, r, p.n_part, q, za);
-  if (!lead) return;
+  write = write && (threadIdx.x & 31) == 0;
+  RowCoef rc = {};
+  rc.a = -1;
+  bool active = m != 0;
+  float c = 0.f, A = 0.f;
+  if (active) {
+    if (i < 0 || i >= p.n_traj) {
+      if (write) flag_status(p.status, RL_DEV_BAD_TRAJ);
+      active = false;
+    } else {
+      c = p.coef[i];
+      A = p.adv_per_row ? p.adv[t] : p.adv[i];
+      active = c != 0.f;
+    }
+  }
+  if (active && (a < 0 || a >= p.V)) {
+    if (write) flag_status(p.status, RL_DEV_BAD_TOKEN);
+    active = false;
+  }
+  if (!active) {
+    if (write) {
+      p.row_loss[t] = 0.0;
+      if (p.token_stats)
+        for (int k = 0; k < 5; ++k) p.token_stats[t * 5 + k] = 0.f;
+    }
+    return rc;
+  }
   const float lnS = logf(q.s);
   const float lse = q.m + lnS;
   const float H = lnS - q.u / q.s;
-  const float A = p.adv_per_row ? p.adv[t] : p.adv[i], c = p.coef[i], old = p.old_logp[t];
   const float logp = za - lse;
   const float rho = expf((za - old) - lse);
   const float crho = fminf(fmaxf(rho, p.clip_lo), p.clip_hi);
   const float surr = fminf(rho * A, crho * A);
   const bool cut = (A > 0.f && rho > p.clip_hi) || (A < 0.f && rho < p.clip_lo);
-  const float w = (p.tis_cap > 0.f && p.rollout_logp) ? fminf(expf(old - p.rollout_logp[t]), p.tis_cap) : 1.f;
+  const float w = (p.tis_cap > 0.f && p.rollout_logp) ? fminf(expf(old - roll), p.tis_cap) : 1.f;
   float kl = 0.f, dkl = 0.f;
   if (p.beta != 0.f && p.ref_logp) {
-    const float d = (p.ref_logp[t] - za) + lse;
+    const float d = (ref - za) + lse;
     const float ed = expf(d);
     kl = ed - d - 1.f;
     dkl = 1.f - ed;
@@ -685,85 +691,149 @@ __global__ void __launch_bounds__(kMergeThreads) head_merge_kernel(const MergeAr
   rc.Ke = -cg + ca * (H - lse);
   rc.a = a;
   rc.active = 1;
-  p.rc[r] = rc;
-  p.row_loss[t] = static_cast<double>(c) * static_cast<double>(ell);
-  if (p.token_stats) {
-    float* st = p.token_stats + t * 5;
-    st[0] = logp; st[1] = rho; st[2] = cut ? 1.f : 0.f; st[3] = H; st[4] = kl;
+  if (write) {
+    p.row_loss[t] = static_cast<double>(c) * static_cast<double>(ell);
+    if (p.token_stats) {
+      float* st = p.token_stats + t * 5;
+      st[0] = logp; st[1] = rho; st[2] = cut ? 1.f : 0.f; st[3] = H; st[4] = kl;
+    }
   }
+  return rc;
 }
 
-struct DzArgs {
-  Tokens tok;
-  int32_t chunk;
-  int32_t V, n_nt;
-  int32_t ent;
-  const RowCoef* rc;
-  uint16_t* dz;       // in: e = exp(z - m_j) (bf16); out: dZ (bf16)
-  int64_t ldz;
-  const float* tmax;  // [Tc x n_nt]
-};
-
 constexpr int kDzThreads = 256;
+constexpr int kDzLoads = 4;          // vectors in flight per thread
 constexpr int kMaxTilesSmem = 2048;  // V up to 524,288 keeps the row's tile factors in shared memory
 
-// One CTA per token row of the chunk (grid-stride): p_v = e_v exp(m_j - lse), then
-// dZ_v = Kp p_v (+ cg at v = a), or with the entropy bonus p_v (ca z_v + Ke) (+ cg at v = a),
-// z_v = m_j + ln e_v. Rows that are not trained on become zeros. 16-byte loads and stores.
-__global__ void __launch_bounds__(kDzThreads) head_dz_kernel(const DzArgs p) {
+// p.split CTAs per token row of the chunk (grid-stride): the CTA's first warp merges the row's
+// partials into its coefficients while the others' first loads are on their way, then
+// p_v = e_v exp(m_j - lse) and dZ_v = Kp p_v (+ cg at v = a), or with the entropy bonus
+// p_v (ca z_v + Ke) (+ cg at v = a), z_v = m_j + ln e_v. Rows that are not trained on become zeros.
+// 16-byte loads and stores. In the call's last chunk the last CTA to finish adds all tokens' loss
+// contributions, in a fixed order, into the caller's total.
+//
+// HBM bounds it in a full chunk (2 x 2 B per logit), the chain of trips to memory in a short call: the
+// merge, the rescale, the loss sum and the products' counter were four launches of 7, 14, 8 and 2 us
+// at 500 tokens x 32,000 entries with one CTA and one vector in flight per thread and row.
+__global__ void __launch_bounds__(kDzThreads, 4) head_dz_kernel(const DzArgs p) {
   __shared__ float fac[kMaxTilesSmem], zoff[kMaxTilesSmem];
+  __shared__ RowCoef shared_rc;
+  __shared__ double part_sum[kDzThreads / 32];
+  __shared__ int is_last;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const Chunk ch = chunk_of(p.tok, p.chunk);
-  for (int r = blockIdx.x; r < ch.padded; r += gridDim.x) {
-    RowCoef rc = {};
-    if (r < ch.count) rc = p.rc[r];  // rows past the chunk's tokens: zeros, like untrained ones
+  if (blockIdx.x == 0 && tid == 0) *p.counter = 0u;
+  const int nvec = p.V / 8, split = p.split;
+  for (int item = blockIdx.x; item < ch.padded * split; item += gridDim.x) {
+    const int r = item / split, part = item - r * split;
     uint16_t* row = p.dz + static_cast<int64_t>(ch.row + r) * p.ldz;
-    const int nvec = p.V / 8;
-    if (!rc.active) {
-      for (int k = threadIdx.x; k < nvec; k += kDzThreads) reinterpret_cast<uint4*>(row)[k] = make_uint4(0, 0, 0, 0);
-      for (int v = nvec * 8 + threadIdx.x; v < p.V; v += kDzThreads) row[v] = 0;
+    uint4* vec = reinterpret_cast<uint4*>(row);
+    // the CTA's vectors (and, in the row's last part, the elements after them), and their tiles
+    const int k_lo = static_cast<int>(static_cast<int64_t>(nvec) * part / split);
+    const int k_hi = static_cast<int>(static_cast<int64_t>(nvec) * (part + 1) / split);
+    const int tail = part == split - 1 ? nvec * 8 : p.V;
+    if (r >= ch.count) {  // rows past the chunk's tokens: zeros
+      for (int k = k_lo + tid; k < k_hi; k += kDzThreads) vec[k] = make_uint4(0, 0, 0, 0);
+      for (int v = tail + tid; v < p.V; v += kDzThreads) row[v] = 0;
       continue;
     }
+    const int j_lo = k_lo * 8 / BN, j_hi = part == split - 1 ? p.n_nt : (k_hi * 8 + BN - 1) / BN;
+    uint4 w[kDzLoads];
+    auto load = [&](int k0) {
+#pragma unroll
+      for (int i = 0; i < kDzLoads; ++i) {
+        const int k = k0 + i * kDzThreads;
+        if (k < k_hi) w[i] = vec[k];
+      }
+    };
+    load(k_lo + tid);
+    float m = j_lo + tid < j_hi ? p.tmax[static_cast<int64_t>(r) * p.n_nt + j_lo + tid] : 0.f;
+    if (warp == 0) {
+      const RowCoef c = row_coef(p, ch, r, part == 0);
+      if (lane == 0) shared_rc = c;
+    }
+    __syncthreads();
+    const RowCoef rc = shared_rc;
     // per tile: Kp exp(m_j - lse) (no entropy) or exp(m_j - lse) and m_j (entropy)
-    for (int j = threadIdx.x; j < p.n_nt; j += kDzThreads) {
-      const float m = p.tmax[static_cast<int64_t>(r) * p.n_nt + j];
+    for (int j = j_lo + tid; j < j_hi; j += kDzThreads) {
+      if (j >= j_lo + kDzThreads) m = p.tmax[static_cast<int64_t>(r) * p.n_nt + j];
       const float f = ex2(fmaf(m, kLog2e, rc.nlse2));
       fac[j] = p.ent ? f : rc.Kp * f;
       zoff[j] = fmaf(rc.ca, m, rc.Ke);  // ca m_j + Ke
     }
     __syncthreads();
-    for (int k = threadIdx.x; k < nvec; k += kDzThreads) {
-      uint4 w = reinterpret_cast<const uint4*>(row)[k];
-      const int j = (k * 8) / BN;
-      const float f = fac[j];
-      uint32_t* wp = reinterpret_cast<uint32_t*>(&w);
-#pragma unroll
-      for (int h = 0; h < 4; ++h) {
-        float o[2];
-#pragma unroll
-        for (int b = 0; b < 2; ++b) {
-          const float e = b ? bf16_hi(wp[h]) : bf16_lo(wp[h]);
-          float x;
-          if (p.ent) {
-            // p (ca z + Ke) with z = m_j + ln e; e = 0 contributes 0
-            x = e > 0.f ? f * e * fmaf(rc.ca, __logf(e), zoff[j]) : 0.f;
-          } else {
-            x = f * e;
-          }
-          if (k * 8 + 2 * h + b == rc.a) x += rc.cg;
-          o[b] = x;
-        }
-        wp[h] = pack_bf16x2(o[0], o[1]);
-      }
-      reinterpret_cast<uint4*>(row)[k] = w;
+    if (!rc.active) {
+      for (int k = k_lo + tid; k < k_hi; k += kDzThreads) vec[k] = make_uint4(0, 0, 0, 0);
+      for (int v = tail + tid; v < p.V; v += kDzThreads) row[v] = 0;
+      continue;
     }
-    for (int v = nvec * 8 + threadIdx.x; v < p.V; v += kDzThreads) {
+    for (int k0 = k_lo + tid; k0 < k_hi; k0 += kDzLoads * kDzThreads) {
+      if (k0 != k_lo + tid) load(k0);
+#pragma unroll
+      for (int i = 0; i < kDzLoads; ++i) {
+        const int k = k0 + i * kDzThreads;
+        if (k >= k_hi) break;
+        const int j = (k * 8) / BN;
+        const float f = fac[j];
+        uint32_t wp[4] = {w[i].x, w[i].y, w[i].z, w[i].w};
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+          float o[2];
+#pragma unroll
+          for (int b = 0; b < 2; ++b) {
+            const float e = b ? bf16_hi(wp[h]) : bf16_lo(wp[h]);
+            float x;
+            if (p.ent) {
+              // p (ca z + Ke) with z = m_j + ln e; e = 0 contributes 0
+              x = e > 0.f ? f * e * fmaf(rc.ca, __logf(e), zoff[j]) : 0.f;
+            } else {
+              x = f * e;
+            }
+            if (k * 8 + 2 * h + b == rc.a) x += rc.cg;
+            o[b] = x;
+          }
+          wp[h] = pack_bf16x2(o[0], o[1]);
+        }
+        vec[k] = make_uint4(wp[0], wp[1], wp[2], wp[3]);
+      }
+    }
+    for (int v = tail + tid; v < p.V; v += kDzThreads) {
       const int j = v / BN;
       const float e = bf16_to_f32(row[v]);
       float x = p.ent ? (e > 0.f ? fac[j] * e * fmaf(rc.ca, __logf(e), zoff[j]) : 0.f) : fac[j] * e;
       if (v == rc.a) x += rc.cg;
       row[v] = f32_to_bf16(x);
     }
-    __syncthreads();  // fac / zoff are rewritten for the next row
+    // the next row's shared_rc is written past this row's second barrier, its fac and zoff past the
+    // next row's first: every read of this row's comes before
+  }
+  if (!p.loss_accum) return;
+  // thread 0 wrote this CTA's rows' loss contributions (and earlier launches the others)
+  if (tid == 0) {
+    __threadfence();
+    is_last = atomicAdd(p.done, 1u) == gridDim.x - 1 ? 1 : 0;
+    if (is_last) __threadfence();
+  }
+  __syncthreads();
+  if (!is_last) return;
+  // thread k adds tokens k, k + 256, ... into eight accumulators in turn (eight loads in flight)
+  double acc[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+  int64_t t = tid;
+  for (; t + 7 * kDzThreads < p.tok.T; t += 8 * kDzThreads) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) acc[k] += __ldcg(p.row_loss + t + k * kDzThreads);
+  }
+#pragma unroll
+  for (int k = 0; k < 8; ++k)
+    if (t + k * kDzThreads < p.tok.T) acc[k] += __ldcg(p.row_loss + t + k * kDzThreads);
+  const double sum = warp_sum(((acc[0] + acc[1]) + (acc[2] + acc[3])) + ((acc[4] + acc[5]) + (acc[6] + acc[7])));
+  if (lane == 0) part_sum[warp] = sum;
+  __syncthreads();
+  if (tid == 0) {
+    double total = 0.0;
+    for (int k = 0; k < kDzThreads / 32; ++k) total += part_sum[k];
+    *p.loss_accum += total;
+    *p.done = 0u;
   }
 }
 
@@ -946,11 +1016,18 @@ static int64_t dh_parts(int64_t Tc, int64_t V, int64_t D) {
   return std::min(std::min<int64_t>(16, most), (kPairs + tiles - 1) / tiles);
 }
 
+// CTAs that share a row of the rescale: as many as give every SM eight CTAs, down to 512 vectors
+// (two per thread) each; one where the chunk's rows suffice.
+static int dz_split(int64_t Tc, int64_t V) {
+  const int64_t most = std::max<int64_t>(1, V / 8 / 512);
+  return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(most, 152 * 8 / Tc)));
+}
+
 struct Layout {
   int64_t Tc, G, n_nt, n_vb, ldz;  // G chunks per group
   int64_t vb, parts;               // N tiles per work item; parts of dH's contraction
   bool pack;                       // the trained tokens are packed
-  size_t off_partials, off_rc, off_tmax, off_idx, off_h, off_parts, off_dz, total;
+  size_t off_partials, off_tmax, off_idx, off_h, off_parts, off_dz, total;
 };
 
 static size_t al256(size_t x) { return (x + 255) & ~size_t(255); }
@@ -980,8 +1057,9 @@ static Layout layout(int64_t max_rows, int64_t V, int64_t D, size_t ws_bytes = 0
   size_t off = kWsHeader + al(static_cast<size_t>(std::max<int64_t>(max_rows, 0)) * sizeof(double));
   L.off_partials = off;
   off += al(static_cast<size_t>(kParts * L.n_vb * L.Tc) * sizeof(float4));
-  L.off_rc = off;
-  off += al(static_cast<size_t>(L.Tc) * sizeof(RowCoef));
+  // 32 B per token that nothing uses: the sizes asked for, and so what a given workspace has room
+  // for, stay what callers have laid out
+  off += al(static_cast<size_t>(L.Tc) * 32);
   L.off_tmax = off;
   off += al(static_cast<size_t>(L.Tc * n_nt) * sizeof(float));
   L.off_idx = off;  // the number of trained tokens (64 words apart from the list), then the list
@@ -1143,7 +1221,6 @@ extern "C" rl_status rl_fused_head_loss_fwd_bwd(
   int32_t* status = reinterpret_cast<int32_t*>(wsb);
   double* row_loss = reinterpret_cast<double*>(wsb + ws_row_loss_offset());
   float4* partials = reinterpret_cast<float4*>(wsb + L.off_partials);
-  RowCoef* rcs = reinterpret_cast<RowCoef*>(wsb + L.off_rc);
   float* tmax = reinterpret_cast<float*>(wsb + L.off_tmax);
   uint16_t* dz_base = reinterpret_cast<uint16_t*>(wsb + L.off_dz);
   rl_status st = RL_OK;
@@ -1224,46 +1301,40 @@ extern "C" rl_status rl_fused_head_loss_fwd_bwd(
     st = launch_head<STATS_P>(mh, mw, ha, s);
     if (st != RL_OK) return st;
 
-    MergeArgs ma = {};
-    ma.tok = tok;
-    ma.chunk = c;
-    ma.V = static_cast<int>(V);
-    ma.n_part = ha.n_vb * static_cast<int>(kParts);
-    ma.n_traj = n_traj;
-    ma.partials = partials;
-    ma.token_ids = token_ids;
-    ma.mask = mask;
-    ma.token_traj = token_traj;
-    ma.adv = adv;
-    ma.coef = coef;
-    ma.old_logp = old_logp;
-    ma.ref_logp = kl_on ? ref_logp : nullptr;
-    ma.rollout_logp = rollout_logp;
-    ma.clip_lo = 1.f - params->clip_eps_low;
-    ma.clip_hi = 1.f + params->clip_eps_high;
-    ma.beta = kl_on ? params->kl_coef : 0.f;
-    ma.alpha = params->entropy_coef;
-    ma.tis_cap = rollout_logp ? params->tis_cap : 0.f;
-    ma.adv_per_row = params->token_level_adv;
-    ma.rc = rcs;
-    ma.row_loss = row_loss;
-    ma.token_stats = token_stats;
-    ma.status = status;
-    head_merge_kernel<<<(Tc + kMergeRows - 1) / kMergeRows, kMergeThreads, 0, s>>>(ma);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_error(e, "head_merge_kernel launch");
-
     DzArgs da = {};
     da.tok = tok;
     da.chunk = c;
     da.V = static_cast<int>(V);
     da.n_nt = n_nt;
-    da.ent = ent && params->entropy_coef != 0.f ? 1 : 0;
-    da.rc = rcs;
+    da.n_part = ha.n_vb * static_cast<int>(kParts);
+    da.n_traj = n_traj;
+    da.split = dz_split(Tc, V);
+    da.ent = params->entropy_coef != 0.f ? 1 : 0;
+    da.partials = partials;
+    da.tmax = tmax;
     da.dz = dz_base;
     da.ldz = L.ldz;
-    da.tmax = tmax;
-    head_dz_kernel<<<std::min(Tc, 148 * 16), kDzThreads, 0, s>>>(da);
+    da.token_ids = token_ids;
+    da.mask = mask;
+    da.token_traj = token_traj;
+    da.adv = adv;
+    da.coef = coef;
+    da.old_logp = old_logp;
+    da.ref_logp = kl_on ? ref_logp : nullptr;
+    da.rollout_logp = rollout_logp;
+    da.clip_lo = 1.f - params->clip_eps_low;
+    da.clip_hi = 1.f + params->clip_eps_high;
+    da.beta = kl_on ? params->kl_coef : 0.f;
+    da.alpha = params->entropy_coef;
+    da.tis_cap = rollout_logp ? params->tis_cap : 0.f;
+    da.adv_per_row = params->token_level_adv;
+    da.row_loss = row_loss;
+    da.loss_accum = c + 1 == n_chunks ? loss_accum : nullptr;
+    da.done = reinterpret_cast<uint32_t*>(wsb + kWsDoneOffset);
+    da.counter = reinterpret_cast<uint32_t*>(wsb + kWsHeadCounterOffset);
+    da.token_stats = token_stats;
+    da.status = status;
+    head_dz_kernel<<<std::min(Tc * da.split, 152 * 16), kDzThreads, 0, s>>>(da);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_error(e, "head_dz_kernel launch");
 
@@ -1276,7 +1347,7 @@ extern "C" rl_status rl_fused_head_loss_fwd_bwd(
       if (st != RL_OK) return st;
     }
   }
-  return launch_reduce_loss(row_loss, T, loss_accum, s);
+  return RL_OK;
 }
 
 extern "C" rl_status rl_fused_head_token_logprobs(const void* hidden, const void* weight, int64_t T, int64_t D,

@@ -409,11 +409,9 @@ rl_status head_grad(const Tokens& tok, int group, int64_t rows, const uint16_t* 
   a.status = status;
   const int32_t n_h = static_cast<int32_t>((rows + 2 * BM - 1) / (2 * BM)) * a.n_nt * parts;  // at most
 
-  cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(uint32_t), s);
-  if (e != cudaSuccess) return cuda_error(e, "cudaMemsetAsync(work counter)");
   auto kern = bf16 ? head_grad_kernel<H_BF16> : head_grad_kernel<H_F32>;
   int dev = 0;
-  e = cudaGetDevice(&dev);
+  cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return cuda_error(e, "cudaGetDevice");
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];

@@ -24,7 +24,7 @@ inline size_t ws_row_loss_offset() { return kWsHeader; }
 constexpr size_t kWsDoneOffset = 16;
 // The same for the value loss kernel's finished CTAs.
 constexpr size_t kWsValueDoneOffset = 20;
-// Work-item counter of the fused head's backward products (zeroed before each launch).
+// Work-item counter of the fused head's backward products (set back by the rescale before it).
 constexpr size_t kWsHeadCounterOffset = 24;
 // The statistics summary's finished clusters, and its clusters' totals (5 doubles each, to the
 // header's end).
@@ -35,8 +35,6 @@ rl_status set_error(rl_status st, const std::string& msg);
 rl_status cuda_error(cudaError_t e, const char* what);
 void clear_error();
 
-// Fixed-order sum of `rows` loss contributions into *loss_accum (rl_stats.cu).
-rl_status launch_reduce_loss(const double* row_loss, int64_t rows, double* loss_accum, cudaStream_t s);
 // Smallest workspace of the fused LM head for up to max_rows tokens (rl_head.cu).
 size_t head_workspace_bytes(int64_t max_rows, int64_t V, int64_t D);
 // The same, keeping the dZ of up to group_tokens tokens (whole chunks) at once.
@@ -50,7 +48,7 @@ struct Tokens;  // rl_head_tokens.cuh
 // tokens ([rows x V] at most, rows ldz elements apart) and hidden their hidden states in the same
 // order. parts > 1 cuts dH's contraction over V into that many items per tile, whose fp32 sums
 // ([parts][Tc x D] at part_sums) a second launch adds. counter: a workspace word for the work-item
-// counter (zeroed here, on the stream).
+// counter, zero before the launch (head_dz_kernel sets it back).
 rl_status head_grad(const Tokens& tok, int group, int64_t rows, const uint16_t* dz, int64_t ldz, int64_t V,
                     const void* weight, const void* hidden, int64_t D, void* d_hidden, rl_dtype dh_dtype,
                     float* d_weight, float* part_sums, int parts, uint32_t* counter, int32_t* status,
