@@ -134,7 +134,7 @@ size_t rl_workspace_size(int64_t max_rows, int64_t V, int64_t D);
 size_t rl_fused_head_workspace_size(int64_t T, int64_t V, int64_t D, int64_t group_tokens);
 
 /* Zero the workspace's 256-byte header: the status word and the finished-block
- * counters of the policy, value and fused-head losses and the statistics summary (which each
+ * counters of the policy and value losses and the statistics summary (which each
  * launch leaves at zero again). Call once after allocating a workspace, and again to clear a reported
  * device error. */
 rl_status rl_workspace_init(void* ws, size_t ws_bytes, rl_stream_t stream);

@@ -15,7 +15,7 @@
 //      evaluates the objective's per-token terms (same readings as the logits path), writes the
 //      token's loss contribution, and rescales the stored e in place into
 //      dZ = c [g (delta_a - p) + alpha p (log p + H)], p = e exp(m_j - lse) (HBM-bound: the
-//      logits are formed once, not twice); the last CTA of the last chunk sums the loss.
+//      logits are formed once, not twice).
 // The dZ of one chunk (4,096 tokens x V in bf16) is the only logits-sized buffer; a caller
 // that passes more workspace lets a group of several chunks keep their dZ side by side.
 // After the group's last chunk (every chunk, with the smallest workspace):
@@ -24,7 +24,8 @@
 //      operands in their row-major layouts (dZ K-major for dH, MN-major for dW; W and H
 //      MN-major), dH tiles first and dW tiles after them, handed out by a work counter; dH rows
 //      are stored at their tokens' places (a short call's in parts of the contraction, which
-//      head_combine_kernel adds), dW added in fp32 by TMA reduce-add, once per group.
+//      head_combine_kernel adds), dW added in fp32 by TMA reduce-add, once per group. The last
+//      group's launch also sums the loss.
 // The forward-only call runs head_wide_kernel<STATS> (256 x 512 tiles, no stores; the same two
 // partials per block) and head_logp_merge_kernel.
 // The objective (Sec. 2.3.2, Sec. 3.2.4) is the same as for rl_policy_loss_fwd_bwd; here
@@ -598,8 +599,6 @@ struct DzArgs {
   float clip_lo, clip_hi, beta, alpha, tis_cap;
   int32_t adv_per_row;  // adv holds one A_t per token (else one per trajectory)
   double* row_loss;     // [T]
-  double* loss_accum;   // the caller's total in the call's last chunk, else null
-  uint32_t* done;       // finished-CTA count in the workspace header
   uint32_t* counter;    // the products' work counter, set back here for their next launch
   float* token_stats;
   int32_t* status;
@@ -709,18 +708,15 @@ constexpr int kMaxTilesSmem = 2048;  // V up to 524,288 keeps the row's tile fac
 // partials into its coefficients while the others' first loads are on their way, then
 // p_v = e_v exp(m_j - lse) and dZ_v = Kp p_v (+ cg at v = a), or with the entropy bonus
 // p_v (ca z_v + Ke) (+ cg at v = a), z_v = m_j + ln e_v. Rows that are not trained on become zeros.
-// 16-byte loads and stores. In the call's last chunk the last CTA to finish adds all tokens' loss
-// contributions, in a fixed order, into the caller's total.
+// 16-byte loads and stores.
 //
 // HBM bounds it in a full chunk (2 x 2 B per logit), the chain of trips to memory in a short call: the
-// merge, the rescale, the loss sum and the products' counter were four launches of 7, 14, 8 and 2 us
+// merge, the rescale and the reset of the products' counter were three launches of 7, 14 and 2 us
 // at 500 tokens x 32,000 entries with one CTA and one vector in flight per thread and row; this one
-// takes 20 (serialised, cold caches), the whole call 198 us instead of 208.
+// takes 15 (serialised, cold caches).
 __global__ void __launch_bounds__(kDzThreads, 4) head_dz_kernel(const DzArgs p) {
   __shared__ float fac[kMaxTilesSmem], zoff[kMaxTilesSmem];
   __shared__ RowCoef shared_rc;
-  __shared__ double part_sum[kDzThreads / 32];
-  __shared__ int is_last;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const Chunk ch = chunk_of(p.tok, p.chunk);
   if (blockIdx.x == 0 && tid == 0) *p.counter = 0u;
@@ -807,34 +803,6 @@ __global__ void __launch_bounds__(kDzThreads, 4) head_dz_kernel(const DzArgs p) 
     }
     // the next row's shared_rc is written past this row's second barrier, its fac and zoff past the
     // next row's first: every read of this row's comes before
-  }
-  if (!p.loss_accum) return;
-  // thread 0 wrote this CTA's rows' loss contributions (and earlier launches the others)
-  if (tid == 0) {
-    __threadfence();
-    is_last = atomicAdd(p.done, 1u) == gridDim.x - 1 ? 1 : 0;
-    if (is_last) __threadfence();
-  }
-  __syncthreads();
-  if (!is_last) return;
-  // thread k adds tokens k, k + 256, ... into eight accumulators in turn (eight loads in flight)
-  double acc[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-  int64_t t = tid;
-  for (; t + 7 * kDzThreads < p.tok.T; t += 8 * kDzThreads) {
-#pragma unroll
-    for (int k = 0; k < 8; ++k) acc[k] += __ldcg(p.row_loss + t + k * kDzThreads);
-  }
-#pragma unroll
-  for (int k = 0; k < 8; ++k)
-    if (t + k * kDzThreads < p.tok.T) acc[k] += __ldcg(p.row_loss + t + k * kDzThreads);
-  const double sum = warp_sum(((acc[0] + acc[1]) + (acc[2] + acc[3])) + ((acc[4] + acc[5]) + (acc[6] + acc[7])));
-  if (lane == 0) part_sum[warp] = sum;
-  __syncthreads();
-  if (tid == 0) {
-    double total = 0.0;
-    for (int k = 0; k < kDzThreads / 32; ++k) total += part_sum[k];
-    *p.loss_accum += total;
-    *p.done = 0u;
   }
 }
 
@@ -1330,8 +1298,6 @@ extern "C" rl_status rl_fused_head_loss_fwd_bwd(
     da.tis_cap = rollout_logp ? params->tis_cap : 0.f;
     da.adv_per_row = params->token_level_adv;
     da.row_loss = row_loss;
-    da.loss_accum = c + 1 == n_chunks ? loss_accum : nullptr;
-    da.done = reinterpret_cast<uint32_t*>(wsb + kWsDoneOffset);
     da.counter = reinterpret_cast<uint32_t*>(wsb + kWsHeadCounterOffset);
     da.token_stats = token_stats;
     da.status = status;
@@ -1343,7 +1309,8 @@ extern "C" rl_status rl_fused_head_loss_fwd_bwd(
     if ((c + 1) % L.G == 0 || c + 1 == n_chunks) {
       float* parts = L.parts > 1 ? reinterpret_cast<float*>(wsb + L.off_parts) : nullptr;
       st = head_grad(tok, static_cast<int>(c / L.G), h_rows, dz_base, L.ldz, V, weight, h_group, D, d_hidden,
-                     d_hidden_dtype, d_weight, parts, static_cast<int>(L.parts),
+                     d_hidden_dtype, d_weight, parts, static_cast<int>(L.parts), row_loss,
+                     c + 1 == n_chunks ? loss_accum : nullptr,
                      reinterpret_cast<uint32_t*>(wsb + kWsHeadCounterOffset), status, s);
       if (st != RL_OK) return st;
     }

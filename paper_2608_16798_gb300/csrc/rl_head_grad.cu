@@ -73,11 +73,35 @@ struct GradArgs {
   float* part_sums;      // [parts][Tc x D] with parts > 1 (one chunk per group then)
   void* d_hidden;        // [T x D]
   uint32_t* counter;     // work-item counter (zero at launch)
+  const double* row_loss;  // [T] loss contributions
+  double* loss_accum;    // the caller's total in the call's last launch, else null
   int32_t* status;
 };
 
 // Element type of the stored d_hidden tiles.
 enum HOut { H_F32 = 0, H_BF16 = 1 };
+
+// The tokens' loss contributions added in a fixed order into the caller's total by the four epilogue
+// warps of CTA 0, while its first accumulator fills (a launch of its own took 8 us at 500 tokens, the rescale's last
+// CTA 5).
+// Thread k adds tokens k, k + 128, ... into eight accumulators in turn (eight loads in flight).
+__device__ __forceinline__ void sum_loss(const GradArgs& p) {
+  __shared__ double part[4];
+  const int k = static_cast<int>(threadIdx.x) - 64;
+  double acc[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+  int64_t t = k;
+  for (; t + 7 * 128 < p.tok.T; t += 8 * 128) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) acc[i] += p.row_loss[t + i * 128];
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+    if (t + i * 128 < p.tok.T) acc[i] += p.row_loss[t + i * 128];
+  const double s = warp_sum(((acc[0] + acc[1]) + (acc[2] + acc[3])) + ((acc[4] + acc[5]) + (acc[6] + acc[7])));
+  if ((k & 31) == 0) part[k >> 5] = s;
+  asm volatile("bar.sync 1, 128;" ::: "memory");
+  if (k == 0) *p.loss_accum += (part[0] + part[1]) + (part[2] + part[3]);
+}
 
 template <int HO>
 __global__ void __launch_bounds__(kThreads, 1) head_grad_kernel(
@@ -94,7 +118,11 @@ __global__ void __launch_bounds__(kThreads, 1) head_grad_kernel(
   const uint32_t rank = cluster_ctarank();
   // the group's tokens, its dH tiles (row tiles x n_nt) and the dW tiles' K blocks
   const Chunk grp = group_of(p.tok, p.group);
-  if (grp.count == 0) return;  // the whole grid: nothing to add
+  const bool sums_loss = p.loss_accum != nullptr && blockIdx.x == 0 && warp >= 2;
+  if (grp.count == 0) {  // the whole grid: nothing to multiply
+    if (sums_loss) sum_loss(p);
+    return;
+  }
   const int n_h1 = (grp.count + 2 * BM - 1) / (2 * BM) * p.n_nt;
   const int n_h = n_h1 * p.parts;
   const int nkb_w = (grp.count + BK - 1) / BK;
@@ -260,6 +288,7 @@ __global__ void __launch_bounds__(kThreads, 1) head_grad_kernel(
     uint8_t* my = slabs + (warp - 2) * 2 * SLAB_BYTES;
     const uint32_t tq = tmem + (static_cast<uint32_t>(32 * q) << 16);
     uint32_t buf = 0;
+    if (sums_loss) sum_loss(p);
     for (uint32_t t = 0;; ++t) {
       int item = 0;
       if (lane == 0) item = next_item(t);
@@ -379,8 +408,8 @@ __global__ void __launch_bounds__(256) head_combine_kernel(const GradArgs p) {
 
 rl_status head_grad(const Tokens& tok, int group, int64_t rows, const uint16_t* dz, int64_t ldz, int64_t V,
                     const void* weight, const void* hidden, int64_t D, void* d_hidden, rl_dtype dh_dtype,
-                    float* d_weight, float* part_sums, int parts, uint32_t* counter, int32_t* status,
-                    cudaStream_t s) {
+                    float* d_weight, float* part_sums, int parts, const double* row_loss, double* loss_accum,
+                    uint32_t* counter, int32_t* status, cudaStream_t s) {
   using namespace grad;
   CUtensorMap ah, bh, aw, bw, ow;
   const bool bf16 = dh_dtype == RL_BF16;
@@ -406,6 +435,8 @@ rl_status head_grad(const Tokens& tok, int group, int64_t rows, const uint16_t* 
   a.part_sums = part_sums;
   a.d_hidden = d_hidden;
   a.counter = counter;
+  a.row_loss = row_loss;
+  a.loss_accum = loss_accum;
   a.status = status;
   const int32_t n_h = static_cast<int32_t>((rows + 2 * BM - 1) / (2 * BM)) * a.n_nt * parts;  // at most
 

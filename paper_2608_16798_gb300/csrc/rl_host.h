@@ -47,12 +47,13 @@ struct Tokens;  // rl_head_tokens.cuh
 // d_weight[V x D] += dZ^T H[n x D] (fp32), with dz the bf16 gradient of the logits of the group's
 // tokens ([rows x V] at most, rows ldz elements apart) and hidden their hidden states in the same
 // order. parts > 1 cuts dH's contraction over V into that many items per tile, whose fp32 sums
-// ([parts][Tc x D] at part_sums) a second launch adds. counter: a workspace word for the work-item
-// counter, zero before the launch (head_dz_kernel sets it back).
+// ([parts][Tc x D] at part_sums) a second launch adds. With loss_accum (the call's last launch) the
+// tok.T loss contributions at row_loss are added to it, in a fixed order. counter: a workspace word
+// for the work-item counter, zero before the launch (head_dz_kernel sets it back).
 rl_status head_grad(const Tokens& tok, int group, int64_t rows, const uint16_t* dz, int64_t ldz, int64_t V,
                     const void* weight, const void* hidden, int64_t D, void* d_hidden, rl_dtype dh_dtype,
-                    float* d_weight, float* part_sums, int parts, uint32_t* counter, int32_t* status,
-                    cudaStream_t s);
+                    float* d_weight, float* part_sums, int parts, const double* row_loss, double* loss_accum,
+                    uint32_t* counter, int32_t* status, cudaStream_t s);
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
