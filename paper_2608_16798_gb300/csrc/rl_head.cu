@@ -75,7 +75,7 @@ constexpr int64_t kParts = 2;               // partials per token and vocabulary
 
 enum Mode { STATS = 0, STATS_P = 1 };
 
-// Per-token coefficients of dZ (from head_merge_kernel).
+// Per-token coefficients of dZ (formed by head_dz_kernel).
 struct RowCoef {
   float nlse2;  // -lse * log2(e)
   float Kp;     // dZ_v = Kp p_v (+ cg at v = a), without the entropy term
@@ -605,9 +605,9 @@ struct DzArgs {
 };
 
 // Token r's partials, merged by a warp: lane l takes partials l, l + 32, ... in order, the lanes
-// are combined by shuffles (the same order in both merge kernels, so that the forward-only call and
-// the loss call agree bit for bit). One trip to memory per 32 partials: a thread per token walking
-// them 8 loads at a time took 16 us for 4,096 tokens and 7 us for 500 of 16 partials each.
+// are combined by shuffles (the same order in head_dz_kernel and head_logp_merge_kernel, so that the
+// forward-only call and the loss call agree bit for bit). One trip to memory per 32 partials: a thread
+// per token walking them 8 loads at a time took 16 us for 4,096 tokens, a warp 6.
 __device__ __forceinline__ void merge_partials(const float4* partials, int64_t Tc, int r, int n_part,
                                                SoftmaxPartial& q, float& za) {
   const int lane = threadIdx.x & 31;
