@@ -732,7 +732,7 @@ __global__ void __launch_bounds__((NW + 1) * 32, MINB) rows_kernel(const RowArgs
       const float za = warp_sum(zsum);
       const RowLse rl = row_lse<kSplit>(q);
       const float lnS = rl.lnS, lse = rl.hi;
-      const float H = ENT || sizeof(T) == 4 ? lnS - q.u / q.s : 0.f;  // times 0 without the entropy
+      const float H = lnS - q.u / q.s;  // without the entropy lnS, or NaN for a row that has one
 
       {
         // per-token scalars (every lane computes the same values)
@@ -750,6 +750,8 @@ __global__ void __launch_bounds__((NW + 1) * 32, MINB) rows_kernel(const RowArgs
           kl = ed - d - 1.f;
           dkl = 1.f - ed;
         }
+        // alpha H also without the bonus (alpha = 0): fminf drops the NaN of a ratio, 0 x NaN does not,
+        // and a row with a NaN or +inf logit has to make the loss NaN
         const float ell = -w * surr + p.beta * kl - p.alpha * H;
         const float g = (cut ? 0.f : -w * A * rho) + p.beta * dkl;
         const float cg = c * g, ca0 = c * p.alpha;
@@ -1128,7 +1130,7 @@ __global__ void __launch_bounds__((kF32Warps + 1) * 32, 3) rows_f32_kernel(const
       const float za = warp_sum(zsum);
       const RowLse rl = row_lse<false>(q);
       const float lnS = rl.lnS, lse = rl.hi;
-      const float H = ENT || sizeof(T) == 4 ? lnS - q.u / q.s : 0.f;  // times 0 without the entropy
+      const float H = lnS - q.u / q.s;  // without the entropy lnS, or NaN for a row that has one
 
       {
         // per-token scalars (every lane computes the same values)
@@ -1376,7 +1378,7 @@ __global__ void __launch_bounds__(kSmallWarps * 32, small_ctas<T, NV>(true)) sma
     const SoftmaxPartial q = sr.template fold<ENT>(lane);
     const RowLse rl = row_lse<kSplit>(q);
     const float lnS = rl.lnS, lse = rl.hi;
-    const float H = ENT ? lnS - q.u / q.s : 0.f;
+    const float H = lnS - q.u / q.s;  // without the entropy lnS, or NaN for a row that has one
     // ---- per-token scalars (every lane computes the same values)
     const float old = wd.old;
     const float logp = (za - lse) - rl.lo;
