@@ -259,7 +259,19 @@ __device__ __forceinline__ void fold_block(SoftmaxPartial& ps, const uint4 (&x)[
   if (!(ps.m > -1e38f)) {
     float m0 = vmax(x[0]);
     if (!(m0 > -1e38f)) m0 = all_max();
-    if (!(m0 > -1e38f)) return;
+    if (!(m0 > -1e38f)) {
+      // nothing but -inf, or NaNs, which no maximum sees: they make the sum NaN
+      bool nan = false;
+#pragma unroll
+      for (int k = 0; k < NV; ++k) {
+        float2 q[NP];
+        Vec<T>::pairs(x[k], q);
+#pragma unroll
+        for (int i = 0; i < NP; ++i) nan |= q[i].x != q[i].x || q[i].y != q[i].y;
+      }
+      if (nan) ps.s = __int_as_float(0x7fffffff);
+      return;
+    }
     ps.m = m0;
   }
   // x = (z - m) log2(e) by one fused multiply-add against nm = fl(-m log2(e)); with the

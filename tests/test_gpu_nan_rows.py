@@ -1,6 +1,6 @@
 """Rows whose softmax is undefined (a NaN or +inf logit, every logit at -inf): their loss term and
 gradient are NaN in every form of the loss kernel, whatever outputs are asked for, and the other rows
-keep the bits that they have without them."""
+keep the bits that they have without them. The forward call gives such a row a NaN lse."""
 
 import pytest
 import torch
@@ -47,18 +47,25 @@ def loss(R, z, stats, ent):
     (torch.bfloat16, 12000, 12000), (torch.bfloat16, 32003, 32003), (torch.bfloat16, 151936, 151936),
     (torch.float32, 500, 500), (torch.float32, 2048, 2051), (torch.float32, 32000, 32000),
     (torch.float32, 32000, 32003), (torch.float32, 151936, 151936), (torch.float32, 200001, 200001)])
-@pytest.mark.parametrize("what", ["nan", "inf", "none"])
+@pytest.mark.parametrize("what", ["nan", "inf", "none", "lanes", "all"])
 def test_undefined_rows_make_the_loss_nan(R, dtype, V, ld, what):
+    """lanes: every 32nd 16-byte block of the row, all that some threads hold; all: the whole row."""
     z = logits(dtype, V, ld)
-    _, clean, _ = loss(R, z, False, 0.0)
+    _, clean, lse0 = loss(R, z, False, 0.0)
     if what == "none":
         z[BAD] = float("-inf")
+    elif what == "lanes":
+        z[BAD, torch.arange(V, device="cuda") // (16 // z.element_size()) % 32 == 5] = float("nan")
+    elif what == "all":
+        z[BAD] = float("nan")
     else:
         z[BAD, V // 2] = float(what)
     others = [r for r in range(ROWS) if r != BAD]
     for stats, ent in ((False, 0.0), (True, 0.0), (False, 0.01)):
-        total, g, _ = loss(R, z, stats, ent)
+        total, g, lse = loss(R, z, stats, ent)
         assert total != total, (stats, ent)
+        assert torch.equal(lse[others], lse0[others])
+        assert what == "none" or lse[BAD].isnan()
         assert g[BAD].isnan().any()
         if not stats and not ent:
             assert torch.equal(g[others], clean[others])
