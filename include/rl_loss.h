@@ -127,10 +127,9 @@ size_t rl_workspace_size(int64_t max_rows, int64_t V, int64_t D);
  * chunks of 4,096 tokens; group_tokens <= 4096 gives rl_workspace_size(T, V, D)).
  * The fused head then runs its dH and dW products once per group instead of once
  * per chunk, which reads and writes the fp32 d_weight fewer times, at the cost of
- * ceil(V / 8) * 8 * 2 bytes per token of the group. Any workspace size works: the
- * group is as many whole chunks of trained tokens as the workspace holds, each with its
- * logits gradient and its packed hidden states (4,096 * D * 2 bytes, which this size
- * counts once: the group can be one chunk smaller than asked for). */
+ * (ceil(V / 8) * 8 + D) * 2 bytes per token of the group: its logits gradient and its packed
+ * hidden states. Any workspace size works: the group is as many whole chunks of trained
+ * tokens as the workspace holds. */
 size_t rl_fused_head_workspace_size(int64_t T, int64_t V, int64_t D, int64_t group_tokens);
 
 /* Zero the workspace's 256-byte header: the status word and the finished-block

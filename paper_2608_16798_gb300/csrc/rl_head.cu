@@ -1006,10 +1006,9 @@ static size_t al256(size_t x) { return (x + 255) & ~size_t(255); }
 // parts of dH besides.
 enum Room { kLeast = 0, kPacked = 1, kAll = 2 };
 
-// Workspace of the loss call for up to max_rows tokens. Its smallest form (ws_bytes = 0)
-// keeps the dZ and the packed hidden states of one chunk; a caller that passes more gets as many
-// chunks of both as fit (want_G chunks of dZ, for the size query), so that the two products run
-// once per group of G chunks.
+// Workspace of the loss call for up to max_rows tokens: with room for one chunk's dZ and packed
+// hidden states, for want_G chunks' (the size queries), or, given a workspace of ws_bytes, for as many
+// chunks of both as fit, so that the two products run once per group of G chunks.
 static Layout layout(int64_t max_rows, int64_t V, int64_t D, size_t ws_bytes = 0, int64_t want_G = 0,
                      Room room = kAll) {
   const bool pack = room != kLeast;
@@ -1036,16 +1035,16 @@ static Layout layout(int64_t max_rows, int64_t V, int64_t D, size_t ws_bytes = 0
   L.parts = room == kAll && max_rows <= kChunk ? dh_parts(L.Tc, V, D) : 1;
   L.off_parts = off;
   if (L.parts > 1) off += al(static_cast<size_t>(L.parts * L.Tc * D) * sizeof(float));
+  // the group's chunks: the logits gradient and the packed hidden states of each
   const size_t chunk_dz = static_cast<size_t>(L.Tc * L.ldz) * 2;
   const size_t chunk_h = pack ? al(static_cast<size_t>(L.Tc * D) * 2) : 0;
-  int64_t G = 1;
+  int64_t G = want_G;
   if (ws_bytes > off) G = static_cast<int64_t>((ws_bytes - off) / (chunk_dz + chunk_h));
   L.G = std::max<int64_t>(1, std::min<int64_t>(G, chunks));
   L.off_h = off;
   off += static_cast<size_t>(L.G) * chunk_h;
   L.off_dz = off;
-  const int64_t dz_chunks = std::max<int64_t>(L.G, std::min<int64_t>(want_G, chunks));
-  off += al(static_cast<size_t>(dz_chunks) * chunk_dz);
+  off += al(static_cast<size_t>(L.G) * chunk_dz);
   L.total = off;
   return L;
 }

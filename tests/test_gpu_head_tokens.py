@@ -81,6 +81,24 @@ def test_workspaces_without_packing(R, T, D, V):
     assert np.allclose(a["stats"], b["stats"], rtol=1e-4, atol=1e-5)
 
 
+# trained tokens that make 1, 2, 3 and 4 chunks of the 4 that 16,384 tokens can need
+@pytest.mark.parametrize("n,need", [(4000, 1), (8100, 2), (12200, 3), (16384, 4)])
+@pytest.mark.parametrize("asked", [1, 2, 3, 4])
+def test_groups_are_as_large_as_asked(R, n, need, asked):
+    """The size asked for a group of several chunks gives groups of that many, right also with a second
+    group after a full first one. d W shows how many groups there were: each adds to it once, so on top
+    of other values it is one rounded addition of the call's own d W exactly when one group holds all."""
+    T, D, V = 16384, 64, 300
+    c = case(T, D, V, n, seed=n)
+    size = R.rl_fused_head_workspace_size(T, V, D, asked * 4096)
+    a = run(R, c, size)
+    compare_head(c, a)
+    base = torch.from_numpy(np.random.default_rng(1).normal(0, 64 * np.abs(a["dW"]).max(), (V, D)).astype(np.float32))
+    b = run(R, c, size, d_w=base.cuda())
+    once = (base + torch.from_numpy(a["dW"].astype(np.float32))).numpy().astype(np.float64)
+    assert np.array_equal(b["dW"], once) == (need <= asked)
+
+
 def test_untrained_tokens_do_not_enter(R):
     """NaN hidden states of masked tokens, a bad id and a bad owner (flagged): no trace in d W."""
     c = case(700, 128, 1500, 400, seed=3)
