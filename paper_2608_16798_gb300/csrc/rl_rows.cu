@@ -242,36 +242,26 @@ struct RowMeta {
 template <typename T, bool ENT, int NV, typename Reload>
 __device__ __forceinline__ void fold_block(SoftmaxPartial& ps, const uint4 (&x)[NV], Reload reload) {
   constexpr int NP = Vec<T>::NP;
+  // NaN if any value is: it then becomes the reference and poisons the sums, also where a thread has
+  // nothing but NaNs
   auto vmax = [&](const uint4 w) {
     float2 q[NP];
     Vec<T>::pairs(w, q);
-    float m = fmaxf(q[0].x, q[0].y);
+    float m = max_nan(q[0].x, q[0].y);
 #pragma unroll
-    for (int i = 1; i < NP; ++i) m = fmaxf(m, fmaxf(q[i].x, q[i].y));
+    for (int i = 1; i < NP; ++i) m = max_nan(m, max_nan(q[i].x, q[i].y));
     return m;
   };
   // exact maximum, recomputed from shared memory (the rare paths only)
   auto all_max = [&]() {
     float m = vmax(reload(0));
-    for (int k = 1; k < NV; ++k) m = fmaxf(m, vmax(reload(k)));
+    for (int k = 1; k < NV; ++k) m = max_nan(m, vmax(reload(k)));
     return m;
   };
   if (!(ps.m > -1e38f)) {
     float m0 = vmax(x[0]);
     if (!(m0 > -1e38f)) m0 = all_max();
-    if (!(m0 > -1e38f)) {
-      // nothing but -inf, or NaNs, which no maximum sees: they make the sum NaN
-      bool nan = false;
-#pragma unroll
-      for (int k = 0; k < NV; ++k) {
-        float2 q[NP];
-        Vec<T>::pairs(x[k], q);
-#pragma unroll
-        for (int i = 0; i < NP; ++i) nan |= q[i].x != q[i].x || q[i].y != q[i].y;
-      }
-      if (nan) ps.s = __int_as_float(0x7fffffff);
-      return;
-    }
+    if (m0 <= -1e38f) return;
     ps.m = m0;
   }
   // x = (z - m) log2(e) by one fused multiply-add against nm = fl(-m log2(e)); with the
