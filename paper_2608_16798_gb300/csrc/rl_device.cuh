@@ -248,7 +248,8 @@ struct SoftmaxPartial {
   float m, s, u;
 };
 
-// Merge two partials; a partial with s == 0 (nothing seen) is the identity.
+// Merge two partials; a partial with s == 0 (nothing seen) is the identity. The fused operations are
+// spelled out, so that a merge has the same bits wherever it is compiled.
 __device__ __forceinline__ SoftmaxPartial merge(SoftmaxPartial a, SoftmaxPartial b) {
   if (b.s == 0.f) return a;
   if (a.s == 0.f) return b;
@@ -257,8 +258,8 @@ __device__ __forceinline__ SoftmaxPartial merge(SoftmaxPartial a, SoftmaxPartial
   const float ea = ex2(da * kLog2e), eb = ex2(db * kLog2e);
   SoftmaxPartial r;
   r.m = M;
-  r.s = a.s * ea + b.s * eb;
-  r.u = ea * fmaf(da, a.s, a.u) + eb * fmaf(db, b.s, b.u);
+  r.s = fmaf(a.s, ea, __fmul_rn(b.s, eb));
+  r.u = fmaf(ea, fmaf(da, a.s, a.u), __fmul_rn(eb, fmaf(db, b.s, b.u)));
   return r;
 }
 

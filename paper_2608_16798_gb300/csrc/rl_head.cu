@@ -10,7 +10,7 @@
 //      holds 128 of the tile's tokens). The epilogue reads each tile twice from TMEM: first
 //      its row maximum m_j, then e = exp(z - m_j), which it stores (bf16) in the chunk's
 //      dZ buffer, with m_j per token and tile, and folds into per-row online-softmax
-//      partials: two per vocabulary block (its even and its odd tiles).
+//      partials: two per block of 4,096 entries (its even and its odd tiles).
 //   2. head_dz_kernel       merges each token's partials into lse, entropy and logp (one warp),
 //      evaluates the objective's per-token terms (same readings as the logits path), writes the
 //      token's loss contribution, and rescales the stored e in place into
@@ -26,8 +26,11 @@
 //      are stored at their tokens' places (a short call's in parts of the contraction, which
 //      head_combine_kernel adds), dW added in fp32 by TMA reduce-add, once per group. The last
 //      group's launch also sums the loss.
-// The forward-only call runs head_wide_kernel<STATS> (256 x 512 tiles, no stores; the same two
-// partials per block) and head_logp_merge_kernel.
+// The forward-only call runs head_wide_kernel<STATS> (256 x 512 tiles, no stores; the same
+// partials) and head_logp_merge_kernel.
+// A token's statistics are summed in one order whatever the call's size and workspace: tiles j, j + 2,
+// ... of a block of 16 in turn, then the blocks' partials. Short calls, whose work items are smaller
+// than a block, leave every tile's own partial and the merge takes the first step too.
 // The objective (Sec. 2.3.2, Sec. 3.2.4) is the same as for rl_policy_loss_fwd_bwd; here
 // pi_theta's logits come from the hidden states times the vocabulary projection.
 #include <cuda.h>
@@ -71,7 +74,7 @@ constexpr uint32_t kWBoxRows = kPair ? BN / 2 : BN;  // rows of W per TMA box
 #define RL_HEAD_CHUNK 4096
 #endif
 constexpr int64_t kChunk = RL_HEAD_CHUNK;  // tokens per chunk (tuning knob, compile time)
-constexpr int64_t kParts = 2;               // partials per token and vocabulary block (even, odd tiles)
+constexpr int64_t kParts = 2;               // partials per token and block of 16 tiles (even, odd ones)
 
 enum Mode { STATS = 0, STATS_P = 1 };
 
@@ -91,8 +94,9 @@ struct HeadArgs {
   int32_t chunk;           // which chunk of them
   int32_t D, V, vb_tiles, n_vb, n_nt;  // N tiles per work item (even), items and tiles per row tile
   int32_t ent;
+  int32_t tile_parts;      // partials of every tile instead of two per work item
   const int32_t* token_ids;
-  float4* partials;        // [2 n_vb][Tc] (m, s, u, z_a): a block's even tiles, then its odd tiles
+  float4* partials;        // (m, s, u, z_a): [2 n_vb][Tc], a block's even tiles, then its odd ones, or [n_nt][Tc]
   uint16_t* dz;            // [G Tc x ldz] bf16: e = exp(z - m_j) (STATS_P), the group's chunks in turn
   int64_t ldz;
   float* tmax;             // [Tc x n_nt]: m_j per token and tile (STATS_P)
@@ -243,7 +247,8 @@ __global__ void __launch_bounds__(kThreads, 1) head_kernel(const __grid_constant
       const int r = m0 + rl;  // token within the chunk
       const bool row_ok = r < ch.count;
       const int nt1 = min((vb + 1) * p.vb_tiles, p.n_nt);
-      // running partials of the block's even and odd tiles (the halves of its 256 x 512 tiles)
+      // running partials of the block's even and odd tiles (the halves of its 256 x 512 tiles);
+      // with tile_parts the tiles' own
       SoftmaxPartial ps0{kNegInf, 0.f, 0.f}, ps1{kNegInf, 0.f, 0.f};
       float za = 0.f;
       const int32_t a = row_ok ? p.token_ids[token_of(p.tok, ch, r)] : -1;
@@ -322,10 +327,16 @@ __global__ void __launch_bounds__(kThreads, 1) head_kernel(const __grid_constant
         }
         if (MODE == STATS_P && row_ok) p.tmax[static_cast<int64_t>(r) * p.n_nt + nt] = tm;
         const SoftmaxPartial tile{tm, s0 + s1, u0};
-        if (nt & 1) ps1 = merge(ps1, tile);
-        else ps0 = merge(ps0, tile);
+        if (p.tile_parts) {
+          if (row_ok) p.partials[static_cast<int64_t>(nt) * p.tok.Tc + r] = make_float4(tile.m, tile.s, tile.u, za);
+          za = 0.f;
+        } else if (nt & 1) {
+          ps1 = merge(ps1, tile);
+        } else {
+          ps0 = merge(ps0, tile);
+        }
       }
-      if (ok && row_ok) {
+      if (ok && row_ok && !p.tile_parts) {
         p.partials[static_cast<int64_t>(2 * vb) * p.tok.Tc + r] = make_float4(ps0.m, ps0.s, ps0.u, za);
         p.partials[static_cast<int64_t>(2 * vb + 1) * p.tok.Tc + r] = make_float4(ps1.m, ps1.s, ps1.u, 0.f);
       }
@@ -557,7 +568,12 @@ __global__ void __launch_bounds__(kThreadsW, 1) head_wide_kernel(const __grid_co
           const SoftmaxPartial half =
               epi_half<MODE>(tq + h * BN, j * BN, p.V, a, p.ent, dz_row ? dz_row + j * BN : nullptr, za, tm);
           if (MODE == STATS_P && row_ok) p.tmax[static_cast<int64_t>(r) * p.n_nt + j] = tm;
-          ps = merge(ps, half);
+          if (p.tile_parts) {
+            if (row_ok) p.partials[static_cast<int64_t>(j) * p.tok.Tc + r] = make_float4(half.m, half.s, half.u, za);
+            za = 0.f;
+          } else {
+            ps = merge(ps, half);
+          }
         }
         tc::fence_before_sync();
         __syncwarp();
@@ -566,7 +582,7 @@ __global__ void __launch_bounds__(kThreadsW, 1) head_wide_kernel(const __grid_co
           else mbar_arrive(&acce);
         }
       }
-      if (ok && row_ok)
+      if (ok && row_ok && !p.tile_parts)
         p.partials[static_cast<int64_t>(2 * vb + h) * p.tok.Tc + r] = make_float4(ps.m, ps.s, ps.u, za);
     }
   }
@@ -581,7 +597,8 @@ __global__ void __launch_bounds__(kThreadsW, 1) head_wide_kernel(const __grid_co
 struct DzArgs {
   Tokens tok;
   int32_t chunk;
-  int32_t V, n_nt, n_part, n_traj;  // n_part partials per token (two per vocabulary block)
+  int32_t V, n_nt, n_traj;
+  int32_t n_part, n_tile;           // block partials per token; tile partials, or 0: see merge_partials
   int32_t split;                    // CTAs per row
   int32_t ent;                      // the entropy term is in the gradient
   const float4* partials;
@@ -604,18 +621,43 @@ struct DzArgs {
   int32_t* status;
 };
 
-// Token r's partials, merged by a warp: lane l takes partials l, l + 32, ... in order, the lanes
-// are combined by shuffles (the same order in head_dz_kernel and head_logp_merge_kernel, so that the
-// forward-only call and the loss call agree bit for bit). One trip to memory per 32 partials: a thread
-// per token walking them 8 loads at a time took 16 us for 4,096 tokens, a warp 6.
-__device__ __forceinline__ void merge_partials(const float4* partials, int64_t Tc, int r, int n_part,
+// Token r's partials, merged by a warp: lane l takes the block partials l, l + 32, ... in order, the
+// lanes are combined by shuffles (in head_dz_kernel and in head_logp_merge_kernel: the loss call and
+// the forward-only call give the same bits). Where the statistics pass left every tile's own (n_tile of
+// them, else 0), a block's partial is formed here first, tile by tile as the pass would. One trip to
+// memory per 32 partials, or two: a thread per token walking them 8 loads at a time took 16 us for
+// 4,096 tokens, a warp 6.
+__device__ __forceinline__ void merge_partials(const float4* partials, int64_t Tc, int r, int n_part, int n_tile,
                                                SoftmaxPartial& q, float& za) {
   const int lane = threadIdx.x & 31;
+  const float4 none = make_float4(-__int_as_float(0x7f800000), 0.f, 0.f, 0.f);
+  if (n_tile == 0) {
 #pragma unroll 4
-  for (int b = lane; b < n_part; b += 32) {
-    const float4 w = partials[static_cast<int64_t>(b) * Tc + r];
-    q = merge(q, SoftmaxPartial{w.x, w.y, w.z});
-    za += w.w;  // nonzero in the one partial whose columns hold the sampled id
+    for (int b = lane; b < n_part; b += 32) {
+      const float4 w = partials[static_cast<int64_t>(b) * Tc + r];
+      q = merge(q, SoftmaxPartial{w.x, w.y, w.z});
+      za += w.w;  // nonzero in the one partial whose columns hold the sampled id
+    }
+  } else {
+    for (int b = lane; b < n_part; b += 32) {
+      const int first = (b >> 1) * kMaxVb + (b & 1);
+      SoftmaxPartial blk{none.x, 0.f, 0.f};
+#pragma unroll
+      for (int h = 0; h < kMaxVb; h += 8) {
+        float4 w[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int nt = first + h + 2 * k;
+          w[k] = nt < n_tile ? partials[static_cast<int64_t>(nt) * Tc + r] : none;
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          blk = merge(blk, SoftmaxPartial{w[k].x, w[k].y, w[k].z});
+          za += w[k].w;
+        }
+      }
+      q = merge(q, blk);
+    }
   }
   q = warp_merge<true>(q);
   za = warp_sum(za);
@@ -636,7 +678,7 @@ __device__ __forceinline__ RowCoef row_coef(const DzArgs& p, const Chunk& ch, in
   const float roll = p.rollout_logp ? p.rollout_logp[t] : 0.f;
   SoftmaxPartial q{-__int_as_float(0x7f800000), 0.f, 0.f};
   float za = 0.f;
-  merge_partials(p.partials, p.tok.Tc, r, p.n_part, q, za);
+  merge_partials(p.partials, p.tok.Tc, r, p.n_part, p.n_tile, q, za);
   write = write && (threadIdx.x & 31) == 0;
   RowCoef rc = {};
   rc.a = -1;
@@ -809,7 +851,7 @@ __global__ void __launch_bounds__(kDzThreads, 4) head_dz_kernel(const DzArgs p) 
 struct LogpMergeArgs {
   Tokens tok;
   int32_t chunk;
-  int32_t V, n_part;  // n_part partials per token (two per vocabulary block)
+  int32_t V, n_part, n_tile;  // as in DzArgs
   const float4* partials;
   const int32_t* token_ids;
   float* logp_out;
@@ -827,7 +869,7 @@ __global__ void __launch_bounds__(kMergeThreads) head_logp_merge_kernel(const Lo
   const int64_t t = token_of(p.tok, ch, r);
   SoftmaxPartial q{-__int_as_float(0x7f800000), 0.f, 0.f};
   float za = 0.f;
-  merge_partials(p.partials, p.tok.Tc, r, p.n_part, q, za);
+  merge_partials(p.partials, p.tok.Tc, r, p.n_part, p.n_tile, q, za);
   if (!lead) return;
   const float lnS = logf(q.s);
   const float lse = q.m + lnS;
@@ -962,9 +1004,8 @@ static rl_status make_map(CUtensorMap* m, const void* base, int64_t inner, int64
 // N tiles per work item of the statistics pass. Items are 256 tokens x a block of the vocabulary;
 // blocks of 16 tiles leave few partials, but a short chunk then has fewer items than CTA pairs (500
 // tokens x 32,000 entries: 16 items on 76 pairs, 121 us). The largest of 16, 8, 4 and 2 tiles
-// whose longest pair does at most 3% more tiles than the best of them: full chunks keep 16. A
-// function of the call's token count and vocabulary alone, the same for the loss and the
-// forward-only call, so that their statistics agree bit for bit.
+// whose longest pair does at most 3% more tiles than the best of them: full chunks keep 16. The
+// split changes no token's statistics: see merge_partials.
 static int64_t vb_tiles(int64_t Tc, int64_t n_nt) {
   const int64_t n_m = (Tc + 2 * BM - 1) / (2 * BM);
   auto cost = [&](int64_t vb) { return (n_m * ((n_nt + vb - 1) / vb) + kPairs - 1) / kPairs * vb; };
@@ -995,14 +1036,21 @@ static int dz_split(int64_t Tc, int64_t V) {
 struct Layout {
   int64_t Tc, G, n_nt, n_vb, ldz;  // G chunks per group
   int64_t vb, parts;               // N tiles per work item; parts of dH's contraction
+  int64_t n_part;                  // partials of blocks of 16 tiles (two each)
+  bool tile_parts;                 // the workspace holds every tile's partial instead
   bool pack;                       // the trained tokens are packed
   size_t off_partials, off_tmax, off_idx, off_h, off_parts, off_dz, total;
 };
 
 static size_t al256(size_t x) { return (x + 255) & ~size_t(255); }
 
+// The softmax partials of one chunk.
+static size_t partials_bytes(const Layout& L) {
+  return al256(static_cast<size_t>((L.tile_parts ? L.n_nt : L.n_part) * L.Tc) * sizeof(float4));
+}
+
 // What a workspace has room for: only what every call needs (every token goes through the products,
-// vocabulary blocks of 16 tiles); the packed trained tokens and the finer blocks besides; and the
+// work items of 16 tiles); the packed trained tokens and the tiles' partials besides; and the
 // parts of dH besides.
 enum Room { kLeast = 0, kPacked = 1, kAll = 2 };
 
@@ -1020,14 +1068,14 @@ static Layout layout(int64_t max_rows, int64_t V, int64_t D, size_t ws_bytes = 0
   L.n_nt = n_nt;
   L.vb = pack ? vb_tiles(L.Tc, n_nt) : kMaxVb;
   L.n_vb = (n_nt + L.vb - 1) / L.vb;
+  L.n_part = kParts * ((n_nt + kMaxVb - 1) / kMaxVb);
+  L.tile_parts = L.vb < kMaxVb;
   L.ldz = (V + 7) / 8 * 8;
   auto al = al256;
   size_t off = kWsHeader + al(static_cast<size_t>(std::max<int64_t>(max_rows, 0)) * sizeof(double));
   L.off_partials = off;
-  off += al(static_cast<size_t>(kParts * L.n_vb * L.Tc) * sizeof(float4));
-  // 32 B per token that nothing uses: the sizes asked for, and so what a given workspace has room
-  // for, stay what callers have laid out
-  off += al(static_cast<size_t>(L.Tc) * 32);
+  off += partials_bytes(L);
+  if (!pack) off += al(static_cast<size_t>(L.Tc) * 32);  // unused: what was too small for a call stays too small
   L.off_tmax = off;
   off += al(static_cast<size_t>(L.Tc * n_nt) * sizeof(float));
   L.off_idx = off;  // the number of trained tokens (64 words apart from the list), then the list
@@ -1146,7 +1194,7 @@ size_t head_workspace_bytes_grouped(int64_t max_rows, int64_t V, int64_t D, int6
 // 3,072 and 6,144 are within 2%, 8,192 takes 26.7 ms (73.1), and 32,768 takes 31.5 ms: the
 // hidden states (256 MB) then evict W's tiles from the 129 MB L2.
 static size_t head_logp_workspace_bytes(const head::Layout& L) {
-  return kWsHeader + head::al256(static_cast<size_t>(head::kParts * L.n_vb * L.Tc) * sizeof(float4));
+  return kWsHeader + head::partials_bytes(L);
 }
 
 }  // namespace rl
@@ -1259,6 +1307,7 @@ extern "C" rl_status rl_fused_head_loss_fwd_bwd(
     ha.n_nt = n_nt;
     ha.vb_tiles = static_cast<int>(L.vb);
     ha.n_vb = static_cast<int>(L.n_vb);
+    ha.tile_parts = L.tile_parts ? 1 : 0;
     ha.ent = ent ? 1 : 0;
     ha.token_ids = token_ids;
     ha.partials = partials;
@@ -1274,7 +1323,8 @@ extern "C" rl_status rl_fused_head_loss_fwd_bwd(
     da.chunk = c;
     da.V = static_cast<int>(V);
     da.n_nt = n_nt;
-    da.n_part = ha.n_vb * static_cast<int>(kParts);
+    da.n_part = static_cast<int>(L.n_part);
+    da.n_tile = L.tile_parts ? n_nt : 0;
     da.n_traj = n_traj;
     da.split = dz_split(Tc, V);
     da.ent = params->entropy_coef != 0.f ? 1 : 0;
@@ -1330,7 +1380,7 @@ extern "C" rl_status rl_fused_head_token_logprobs(const void* hidden, const void
   if (T > INT32_MAX || V > INT32_MAX || D > 65536)
     return set_error(RL_ERR_UNSUPPORTED, "rl_fused_head_token_logprobs: T or V above 2^31 - 1, or D above 65536");
   if (!ws) return set_error(RL_ERR_INVALID_ARG, "rl_fused_head_token_logprobs: NULL workspace");
-  // the finer vocabulary blocks where their partials fit, else blocks of 16 tiles
+  // the smaller work items where the tiles' partials fit, else blocks of 16 tiles
   Layout L = layout(T, V, D);
   if (ws_bytes < head_logp_workspace_bytes(L)) L = layout(T, V, D, 0, 0, kLeast);
   if (ws_bytes < head_logp_workspace_bytes(L))
@@ -1366,6 +1416,7 @@ extern "C" rl_status rl_fused_head_token_logprobs(const void* hidden, const void
     ha.n_nt = static_cast<int>(L.n_nt);
     ha.vb_tiles = static_cast<int>(L.vb);
     ha.n_vb = static_cast<int>(L.n_vb);
+    ha.tile_parts = L.tile_parts ? 1 : 0;
     ha.ent = entropy_out ? 1 : 0;
     ha.token_ids = token_ids;
     ha.partials = partials;
@@ -1376,7 +1427,8 @@ extern "C" rl_status rl_fused_head_token_logprobs(const void* hidden, const void
     ma.tok = tok;
     ma.chunk = c;
     ma.V = static_cast<int>(V);
-    ma.n_part = ha.n_vb * static_cast<int>(kParts);
+    ma.n_part = static_cast<int>(L.n_part);
+    ma.n_tile = L.tile_parts ? ha.n_nt : 0;
     ma.partials = partials;
     ma.token_ids = token_ids;
     ma.logp_out = logp_out;
