@@ -884,7 +884,8 @@ __global__ void __launch_bounds__(kMergeThreads) head_logp_merge_kernel(const Lo
 // ------------------------------------------------------------------ trained tokens
 //
 // A token that is not trained on (M_t = 0, c = 0, or a bad id or owner, which is flagged) has no
-// loss and a zero gradient, so it needs none of the three products: head_select_kernel lists the
+// loss and a zero gradient, so it needs none of the three products: head_select_kernel (after
+// head_count_kernel in a call of more than 8,192 tokens) lists the
 // trained tokens in their order (and the others from the list's end), head_gather_kernel packs a
 // chunk's hidden states, and everything after it works on packed rows. On the multi-turn batch
 // (62% trained) that is 38% of the call's flops: 6,000 tokens at D = 4,096 and V = 151,936
@@ -897,45 +898,62 @@ struct SelectArgs {
   const float* coef;
   int32_t* idx;      // [T]
   int32_t* n_dev;    // number of trained tokens
+  int32_t* counts;   // per kSelThreads tokens, from head_count_kernel; null: a short call, without it
   double* row_loss;  // 0 for the others
   float* token_stats;
   int32_t* status;
 };
 
 constexpr int kSelThreads = 1024;
+// CTAs of head_select_kernel up to which it counts by itself.
+constexpr int64_t kSelAlone = 8;
+static int64_t select_blocks(int64_t T) { return (T + kSelThreads - 1) / kSelThreads; }
 
-// One CTA per kSelThreads tokens. Each counts the trained tokens before its own by itself (mask,
-// owner and coefficient of every earlier token: 9 bytes each, from L2), which costs less than a
-// second launch until T is in the millions.
+__device__ __forceinline__ bool is_trained(const SelectArgs& p, int64_t t, bool flag) {
+  if (p.mask[t] == 0) return false;
+  const int32_t i = p.token_traj[t];
+  if (i < 0 || i >= p.n_traj) {
+    if (flag) flag_status(p.status, RL_DEV_BAD_TRAJ);
+    return false;
+  }
+  if (p.coef[i] == 0.f) return false;
+  const int32_t a = p.token_ids[t];
+  if (a < 0 || a >= p.V) {
+    if (flag) flag_status(p.status, RL_DEV_BAD_TOKEN);
+    return false;
+  }
+  return true;
+}
+
+// Trained tokens of each kSelThreads tokens.
+__global__ void __launch_bounds__(kSelThreads) head_count_kernel(const SelectArgs p) {
+  const int64_t t = static_cast<int64_t>(blockIdx.x) * kSelThreads + threadIdx.x;
+  const int n = __syncthreads_count(t < p.T && is_trained(p, t, false));
+  if (threadIdx.x == 0) p.counts[blockIdx.x] = n;
+}
+
+// One CTA per kSelThreads tokens. The trained tokens before its own: the earlier CTAs' counts, or, in a
+// short call, counted here, which spares a launch but reads every earlier token again: 5 us for 4,096
+// tokens, 7 for 8,192, 11 for 16,384, 18 for 32,768 and 386 for 524,288, against 6 (16,384 and
+// 32,768) and 13 us for the two launches.
 __global__ void __launch_bounds__(kSelThreads) head_select_kernel(const SelectArgs p) {
   __shared__ int32_t part[kSelThreads / 32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  auto trained = [&](int64_t t, bool flag) {
-    if (p.mask[t] == 0) return false;
-    const int32_t i = p.token_traj[t];
-    if (i < 0 || i >= p.n_traj) {
-      if (flag) flag_status(p.status, RL_DEV_BAD_TRAJ);
-      return false;
-    }
-    if (p.coef[i] == 0.f) return false;
-    const int32_t a = p.token_ids[t];
-    if (a < 0 || a >= p.V) {
-      if (flag) flag_status(p.status, RL_DEV_BAD_TOKEN);
-      return false;
-    }
-    return true;
-  };
   const int64_t t0 = static_cast<int64_t>(blockIdx.x) * kSelThreads, t = t0 + tid;
   int32_t before = 0;
+  if (p.counts) {
+    for (unsigned b = tid; b < blockIdx.x; b += kSelThreads) before += p.counts[b];
+  } else {
 #pragma unroll 4
-  for (int64_t u = tid; u < t0; u += kSelThreads) before += trained(u, false) ? 1 : 0;
+    for (int64_t u = tid; u < t0; u += kSelThreads) before += is_trained(p, u, false) ? 1 : 0;
+  }
   before = __reduce_add_sync(0xffffffffu, before);
   if (lane == 0) part[warp] = before;
   __syncthreads();
   int32_t base = 0;
   for (int w = 0; w < kSelThreads / 32; ++w) base += part[w];
   __syncthreads();
-  const bool on = t < p.T && trained(t, true);
+  const bool on = t < p.T && is_trained(p, t, true);
   const unsigned ballot = __ballot_sync(0xffffffffu, on);
   if (lane == 0) part[warp] = __popc(ballot);
   __syncthreads();
@@ -1039,7 +1057,7 @@ struct Layout {
   int64_t n_part;                  // partials of blocks of 16 tiles (two each)
   bool tile_parts;                 // the workspace holds every tile's partial instead
   bool pack;                       // the trained tokens are packed
-  size_t off_partials, off_tmax, off_idx, off_h, off_parts, off_dz, total;
+  size_t off_partials, off_tmax, off_idx, off_counts, off_h, off_parts, off_dz, total;
 };
 
 static size_t al256(size_t x) { return (x + 255) & ~size_t(255); }
@@ -1080,6 +1098,8 @@ static Layout layout(int64_t max_rows, int64_t V, int64_t D, size_t ws_bytes = 0
   off += al(static_cast<size_t>(L.Tc * n_nt) * sizeof(float));
   L.off_idx = off;  // the number of trained tokens (64 words apart from the list), then the list
   if (pack) off += 256 + al(static_cast<size_t>(std::max<int64_t>(max_rows, 1)) * sizeof(int32_t));
+  L.off_counts = off;
+  if (pack && select_blocks(max_rows) > kSelAlone) off += al(static_cast<size_t>(select_blocks(max_rows)) * sizeof(int32_t));
   L.parts = room == kAll && max_rows <= kChunk ? dh_parts(L.Tc, V, D) : 1;
   L.off_parts = off;
   if (L.parts > 1) off += al(static_cast<size_t>(L.parts * L.Tc * D) * sizeof(float));
@@ -1268,7 +1288,14 @@ extern "C" rl_status rl_fused_head_loss_fwd_bwd(
     sa.row_loss = row_loss;
     sa.token_stats = token_stats;
     sa.status = status;
-    head_select_kernel<<<static_cast<unsigned>((T + kSelThreads - 1) / kSelThreads), kSelThreads, 0, s>>>(sa);
+    const unsigned blocks = static_cast<unsigned>(select_blocks(T));
+    if (blocks > kSelAlone) {
+      sa.counts = reinterpret_cast<int32_t*>(wsb + L.off_counts);
+      head_count_kernel<<<blocks, kSelThreads, 0, s>>>(sa);
+      e = cudaGetLastError();
+      if (e != cudaSuccess) return cuda_error(e, "head_count_kernel launch");
+    }
+    head_select_kernel<<<blocks, kSelThreads, 0, s>>>(sa);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_error(e, "head_select_kernel launch");
     tok.idx = sa.idx;

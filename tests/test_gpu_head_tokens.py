@@ -81,6 +81,15 @@ def test_workspaces_without_packing(R, T, D, V):
     assert np.allclose(a["stats"], b["stats"], rtol=1e-4, atol=1e-5)
 
 
+# around the largest call that one launch selects in (8,192), and one whose first thousands of tokens
+# are untrained; 70,000: more CTAs than a warp has lanes
+@pytest.mark.parametrize("T,first", [(8192, 0), (8193, 0), (9217, 5000), (70000, 0)])
+def test_selection_of_long_calls(R, T, first):
+    c = make_head_case(T, 64, 130, seed=T, agg=2)
+    c["mask"][:first] = 0
+    compare_head(c, run(R, c))
+
+
 # trained tokens that make 1, 2, 3 and 4 chunks of the 4 that 16,384 tokens can need
 @pytest.mark.parametrize("n,need", [(4000, 1), (8100, 2), (12200, 3), (16384, 4)])
 @pytest.mark.parametrize("asked", [1, 2, 3, 4])
