@@ -652,6 +652,7 @@ __device__ __forceinline__ void merge_partials(const float4* partials, int64_t T
         }
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
+          if (first + h + 2 * k >= n_tile) break;
           blk = merge(blk, SoftmaxPartial{w[k].x, w[k].y, w[k].z});
           za += w[k].w;
         }

@@ -734,7 +734,7 @@ __global__ void __launch_bounds__((NW + 1) * 32, MINB) rows_kernel(const RowArgs
       const float za = warp_sum(zsum);
       const RowLse rl = row_lse<kSplit>(q);
       const float lnS = rl.lnS, lse = rl.hi;
-      const float H = lnS - q.u / q.s;  // without the entropy lnS, or NaN for a row that has one
+      const float H = ENT ? lnS - q.u / q.s : lnS;  // without the entropy: times 0, for its NaN
 
       {
         // per-token scalars (every lane computes the same values)
@@ -752,8 +752,8 @@ __global__ void __launch_bounds__((NW + 1) * 32, MINB) rows_kernel(const RowArgs
           kl = ed - d - 1.f;
           dkl = 1.f - ed;
         }
-        // alpha H also without the bonus (alpha = 0): fminf drops the NaN of a ratio, 0 x NaN does not,
-        // and a row with a NaN or +inf logit has to make the loss NaN
+        // alpha H also without the bonus (alpha = 0): fminf drops the ratio's NaN, but 0 x ln S is NaN for
+        // a row whose softmax is undefined, which has to make the loss NaN
         const float ell = -w * surr + p.beta * kl - p.alpha * H;
         const float g = (cut ? 0.f : -w * A * rho) + p.beta * dkl;
         const float cg = c * g, ca0 = c * p.alpha;
@@ -1132,7 +1132,7 @@ __global__ void __launch_bounds__((kF32Warps + 1) * 32, 3) rows_f32_kernel(const
       const float za = warp_sum(zsum);
       const RowLse rl = row_lse<false>(q);
       const float lnS = rl.lnS, lse = rl.hi;
-      const float H = lnS - q.u / q.s;  // without the entropy lnS, or NaN for a row that has one
+      const float H = lnS - q.u / q.s;  // without the entropy: times 0, for its NaN
 
       {
         // per-token scalars (every lane computes the same values)
@@ -1380,7 +1380,7 @@ __global__ void __launch_bounds__(kSmallWarps * 32, small_ctas<T, NV>(true)) sma
     const SoftmaxPartial q = sr.template fold<ENT>(lane);
     const RowLse rl = row_lse<kSplit>(q);
     const float lnS = rl.lnS, lse = rl.hi;
-    const float H = lnS - q.u / q.s;  // without the entropy lnS, or NaN for a row that has one
+    const float H = ENT ? lnS - q.u / q.s : lnS;  // without the entropy: times 0, for its NaN
     // ---- per-token scalars (every lane computes the same values)
     const float old = wd.old;
     const float logp = (za - lse) - rl.lo;
