@@ -39,6 +39,8 @@
  *     trajectory index outside [0, n_traj), inconsistent offsets, a bounded
  *     wait that ran out) set bits of a status word kept in the workspace;
  *     kernels never trap. Read it with rl_query_status().
+ *   - A workspace is initialised once (rl_workspace_init) and serves one call at a time: calls that
+ *     may overlap on the GPU (other streams) need workspaces of their own.
  *   - The loss returned is the NEGATED objective (the paper maximises the
  *     objective; the library gives a loss to minimise and its gradient).
  *   - Logits rows are dense, row-major, row r starting at element r * ld.
@@ -316,8 +318,9 @@ rl_status rl_fused_head_loss_fwd_bwd(const void* hidden, const void* weight, int
  *   summary_accum      double [5] on the device
  *   ws, ws_bytes       rl_workspace_size(0, 0, 0) bytes suffice (the header: status word, a
  *                      finished-cluster counter and the clusters' totals)
- * One launch of one to five 16-CTA clusters, a fixed assignment of rows to threads and a fixed
- * order of the partial sums, in double precision: deterministic.
+ * One launch of one to five clusters of 16 CTAs (8 where the device has no room for 16), a fixed
+ * assignment of rows to threads and a fixed order of the partial sums, in double precision:
+ * deterministic.
  */
 rl_status rl_token_stats_summary(int64_t rows, const float* token_stats, const uint8_t* mask,
                                  const int32_t* token_traj, int32_t n_traj, const float* coef,

@@ -5,8 +5,8 @@
 // reduction order in double precision: the sums are the same on every run.
 #include <algorithm>
 #include <cstdint>
+#include <map>
 #include <mutex>
-#include <set>
 
 #include "rl_device.cuh"
 #include "rl_host.h"
@@ -21,15 +21,16 @@ namespace rl {
 // CTA totals meet in rank 0's shared memory), and the last cluster to finish adds the clusters'
 // totals in order: the grid depends on the row count alone, so the sums are the same on every run.
 //
-// What bounds it is the FP64 pipe (two lanes per clock and SM: 16 clocks per warp instruction),
-// not memory. So the number of rows and of clipped ones (a flag of 1) are counted in integers, the
-// floats are widened by integer instructions, and three DADD per row remain of ten FP64
-// instructions; and the rows spread over up to 80 SMs instead of 8. The slots that hold a
-// cluster's five totals are spare bytes of the 256-byte workspace header, which every caller has:
-// five of them fit, which with clusters of 16 gives 80 CTAs. Over 1.42 M rows: 487 us with one
-// cluster of 8 and ten FP64 instructions per row, about 32 us now; 131,072 rows: 56 us before.
+// What bounded one cluster of 8 was the FP64 pipe (two lanes per clock and SM: 16 clocks per warp
+// instruction): ten such instructions per row. So the number of rows and of clipped ones (a flag of 1)
+// are counted in integers, the floats are widened by integer instructions, and three DADD per row remain;
+// and the rows spread over up to 80 SMs. The slots that hold a cluster's five totals are spare bytes of
+// the 256-byte workspace header, which every caller has: five of them fit, which with clusters of 16
+// gives 80 CTAs. 1.42 M rows: 487 -> 30 us, 131,072 rows: 56 -> 17. What bounds it now is latency (the
+// three dependent trips, four scalar loads of each 20-byte row, the cluster's launch and barriers): sums in
+// 64-bit integers, without any FP64 per row, took as long.
 constexpr int kSumThreads = 1024;
-constexpr int kSumCluster = 16;
+constexpr int kSumCluster = 16;  // 8 where the device has no room for one of 16
 constexpr int kSumUnroll = 4;
 constexpr int kSumSlots = 5;
 static_assert(kWsSummaryOffset + kSumSlots * 5 * sizeof(double) <= kWsHeader, "summary slots fit the header");
@@ -45,7 +46,7 @@ __global__ void __launch_bounds__(kSumThreads)
   __shared__ double part[kSumThreads / 32][5];
   __shared__ double cta_total[kSumCluster][5];  // used in rank 0
   const uint32_t rank = cluster_ctarank();
-  const unsigned cid = blockIdx.x / kSumCluster, ncl = gridDim.x / kSumCluster;
+  const unsigned C = cluster_nctarank(), cid = blockIdx.x / C, ncl = gridDim.x / C;
   const int64_t G = static_cast<int64_t>(gridDim.x) * kSumThreads;
   double acc[3] = {0.0, 0.0, 0.0};  // H, KL, rho
   double clip = 0.0;                // flags other than 0 and 1
@@ -110,7 +111,7 @@ __global__ void __launch_bounds__(kSumThreads)
   if (rank != 0 || warp != 0) return;
   if (lane < 5) {
     double sum = 0.0;
-    for (int k = 0; k < kSumCluster; ++k) sum += cta_total[k][lane];
+    for (unsigned k = 0; k < C; ++k) sum += cta_total[k][lane];
     if (ncl == 1) {
       out[lane] += sum;
       return;
@@ -151,32 +152,43 @@ extern "C" rl_status rl_token_stats_summary(int64_t rows, const float* token_sta
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return cuda_error(e, "cudaGetDevice");
-  static std::mutex mu;
-  static std::set<int> ready;  // devices on which clusters of 16 are allowed for this kernel
-  {
-    std::lock_guard<std::mutex> lock(mu);
-    if (!ready.count(dev)) {
-      e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-      if (e != cudaSuccess) return cuda_error(e, "cudaFuncSetAttribute(stats_summary_kernel)");
-      ready.insert(dev);
-    }
-  }
-  // a cluster per 8,192 rows up to the five that have a slot: below that a second cluster's
-  // trip through the slots costs more than the rows it takes over
-  // (a workspace whose slots are not on 8-byte boundaries has one cluster, which needs none)
-  const int64_t clusters =
-      reinterpret_cast<uintptr_t>(ws) % 8 != 0 ? 1 : std::min<int64_t>(kSumSlots, (rows + 8191) / 8192);
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = kSumCluster;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
-  cfg.gridDim = dim3(static_cast<unsigned>(clusters * kSumCluster));
+  cfg.gridDim = dim3(kSumCluster);
   cfg.blockDim = dim3(kSumThreads);
   cfg.stream = s;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  static std::mutex mu;
+  static std::map<int, unsigned> width;  // by device: CTAs of a cluster
+  unsigned C = 0;
+  {
+    std::lock_guard<std::mutex> lock(mu);
+    auto it = width.find(dev);
+    if (it == width.end()) {
+      // clusters of 16 are not portable: a partition of a GPU may have no 16 SMs in one GPC
+      int fit = 0;
+      e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&fit, kern, &cfg);
+      if (e != cudaSuccess) {
+        (void)cudaGetLastError();
+        fit = 0;
+      }
+      it = width.emplace(dev, fit > 0 ? kSumCluster : kSumCluster / 2).first;
+    }
+    C = it->second;
+  }
+  // a cluster per 8,192 rows up to the five that have a slot: below that a second cluster's
+  // trip through the slots costs more than the rows it takes over
+  // (a workspace whose slots are not on 8-byte boundaries has one cluster, which needs none)
+  const int64_t clusters =
+      reinterpret_cast<uintptr_t>(ws) % 8 != 0 ? 1 : std::min<int64_t>(kSumSlots, (rows + 8191) / 8192);
+  attr[0].val.clusterDim.x = C;
+  cfg.gridDim = dim3(static_cast<unsigned>(clusters) * C);
   char* wsb = static_cast<char*>(ws);
   e = cudaLaunchKernelEx(&cfg, kern, rows, token_stats, mask, token_traj, n_traj, coef, summary_accum,
                          reinterpret_cast<double*>(wsb + kWsSummaryOffset),
