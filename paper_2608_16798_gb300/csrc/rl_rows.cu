@@ -32,7 +32,6 @@
 // header) sums the partials in a fixed order into the caller's total, so the
 // loss is bit-reproducible without a second launch.
 #include <algorithm>
-#include <cmath>
 #include <cstdint>
 #include <map>
 #include <mutex>
@@ -192,7 +191,7 @@ __device__ __forceinline__ void raise_max(SoftmaxPartial& ps, float vm) {
 
 // Shared-memory stages per CTA (tuning knob). The consumer warps per CTA, the 16-byte vectors
 // of the slice each consumer thread holds in registers, the CTAs per SM and the slice size that
-// picks the cluster width are chosen per path on the host (loss_shape).
+// picks the cluster width are chosen per row length on the host (kPicksBf16, kPicksF32).
 #ifndef RL_STAGES
 #define RL_STAGES 2
 #endif
@@ -1843,72 +1842,67 @@ static rl_status launch_f32(const RowArgs& args, const Plan& plan, cudaStream_t 
   return launch_clusters(rows_f32_kernel<ENT>, (kF32Warps + 1) * 32, args, plan, s, n_clusters_out);
 }
 
-// Shapes of the loss kernel: consumer warps, 16-byte vectors each of their threads holds, CTAs per
-// SM, tau, the time a CTA takes per row (us; and tau_c, what each CTA of the cluster adds), and the
-// most bytes of rows (MB) that should be resident at once.
-//
-// tau is a chain of waits (the slice, the exchange, the merges) and depends little on how full the
-// slice is, so up to a point what counts is how many bytes of rows are resident: clusters of the shape
-// that fit on the GPU x bytes of a row. Past that point (10 MB with several CTAs per SM, 11 to 15
-// with one) reads and writes of more rows at once slow the memory down: 16,384 bf16 entries, clusters of
-// one with 10 vectors (10.0 MB) 5,609 GB/s and 9.7 MB on shape 5 6,348, but 14.6 MB (V = 32,000, shape 1)
-// 5,360. Measured over every shape and width at 19 vocabularies from 4,160 to 262,144 entries
-// (bf16, all rows trained, 0.8 GB of logits, GB/s read and written): the choice below is
-// within 5% of the fastest at each; against one shape for all (8 x 10 at 2 per SM, slices of 20 to
-// 40 KB): V = 4,160 1,682 -> 4,956, 8,192 3,156 -> 5,525, 25,600 4,614 -> 5,830, 65,536 5,301 ->
-// 6,308, 151,936 5,625 -> 6,357, 262,144 4,729 -> 6,441 (with the shorter merges of bf16 rows).
-// From 29,728 to 34,215 entries one CTA of 16 warps per row: 8,192 packed rows of 32,003 entries, 62%
-// trained, 155 us against 163 with clusters of two of 8 warps.
+// Shapes of rows_kernel: consumer warps, 16-byte vectors each of their threads holds, CTAs per SM.
 struct Shape {
   int warps, hold, per_sm;
-  double tau, tau_c, most, most_wide;  // most: clusters of up to 3; most_wide: wider ones
 };
-constexpr Shape kShapes[] = {
-    {8, 10, 2, 2.45, 0.07, 10.4, 10.4}, {7, 9, 3, 3.00, 0.07, 10.4, 10.4}, {8, 6, 3, 2.55, 0.10, 10.4, 10.4},
-    {4, 10, 4, 2.60, 0.09, 10.4, 10.4}, {4, 5, 5, 2.52, 0.05, 10.4, 10.4}, {16, 10, 1, 2.75, 0.09, 11.0, 11.0},
-    {19, 11, 1, 3.40, 0.10, 12.6, 14.8},
-};
-constexpr int kNumShapes = sizeof(kShapes) / sizeof(kShapes[0]);
+constexpr Shape kShapes[] = {{8, 10, 2}, {8, 6, 3}, {4, 10, 4}, {4, 5, 5}, {16, 10, 1}, {19, 11, 1}};
 
-// Clusters of C CTAs resident at once with 1 to 4 CTAs per SM (152 SMs in GPCs of different sizes:
-// cudaOccupancyMaxActiveClusters), for choosing a shape before anything is launched.
-constexpr int kResident[4][16] = {
-    {152, 76, 46, 36, 28, 23, 15, 15, 15, 13, 8, 8, 7, 7, 7, 7},
-    {304, 152, 97, 74, 58, 46, 38, 36, 30, 28, 23, 23, 19, 14, 14, 14},
-    {456, 228, 148, 110, 87, 74, 59, 51, 46, 43, 36, 36, 28, 26, 26, 21},
-    {608, 304, 194, 148, 117, 97, 81, 74, 61, 58, 51, 46, 40, 35, 33, 33},
+// The shape and the cluster width for rows of up to V entries (above the entry before). The time a CTA
+// takes per row, 2.5 to 4 us, is a chain of waits (the slice, the exchange, the merges) that depends
+// little on how full its slice is, so what counts is how many bytes of rows are resident, up to 10 to 15
+// MB, past which reads and writes of more rows at once slow the memory down: which of the shapes comes
+// closest changes with every slice that a cluster more or less brings, by no simple law. So the lines are
+// where the measurements cross, or where a row outgrows its slices. Measured: every shape at its three
+// narrowest widths, 146 vocabularies of 4,104 to 819,200 bf16 entries and 39 of 129,032 to 409,600 fp32
+// ones (0.8 GB of logits), all rows trained without and with the entropy, and 62% of them trained in
+// spans; a crossing that one of the three loses by more than 2% is left out. In the mean of the three
+// the choice is 0.8% from the fastest on average and 7% at most (fp32: 0.1% and 2%). GB/s read and
+// written, all rows trained without the entropy, against one shape for all (8 x 10 at 2 CTAs per SM,
+// slices of 20 to 40 KB): V = 4,160 4,810 (1,682), 8,192 5,560 (3,156), 25,600 5,880 (4,614), 32,000 6,190
+// (5,503), 65,536 6,110 (5,301), 128,256 6,180 (5,077), 151,936 6,220 (5,625), 262,144 5,490 (4,729). The
+// number of rows does not enter: a row's results do not depend on the size of its microbatch (bf16 rows
+// with a leading dimension that is no multiple of 8 are cut where memory blocks end, so the order of
+// their sums depends on r ld mod 8).
+struct Pick {
+  int32_t V;
+  int8_t shape, C;
+};
+constexpr Pick kPicksBf16[] = {
+    {5120, 3, 1}, {8816, 2, 1}, {12288, 1, 1}, {19320, 0, 1}, {22800, 1, 2}, {26800, 2, 3}, {29720, 0, 2},
+    {36552, 4, 1}, {41440, 5, 1}, {44440, 2, 5}, {47624, 1, 4}, {59768, 2, 6}, {68608, 0, 4},
+    {78848, 4, 2}, {82888, 5, 2}, {102400, 2, 10}, {108536, 2, 11}, {122880, 0, 6}, {133120, 2, 13},
+    {143360, 0, 7}, {163840, 4, 4}, {184320, 0, 9}, {204800, 5, 4}, {256000, 5, 5}, {307200, 5, 6},
+    {368640, 4, 9}, {409600, 4, 10}, {460800, 5, 9}, {512000, 5, 10}, {655360, 4, 16}, {768000, 5, 15},
+    {819200, 5, 16},
+};
+constexpr Pick kPicksF32[] = {
+    {153600, 5, 6}, {184320, 4, 9}, {197488, 4, 10}, {204800, 5, 8}, {230400, 5, 9}, {256000, 5, 10},
+    {286720, 4, 14}, {327680, 4, 16}, {343992, 5, 14}, {384000, 5, 15}, {409600, 5, 16},
 };
 
-// The shape (from `first` on) and cluster width with the highest estimate of the rate in TB/s: the
-// resident bytes over tau, against the memory's rate below and above the shape's `most` (combined in
-// the fourth power: near the knee both count). The number of rows does not enter: a row's results are
-// the same in any microbatch.
-static int pick_shape(int64_t V, int es, Plan* plan, int first) {
-  int best = -1;
-  double best_rate = 0.0;
-  for (int k = first; k < kNumShapes; ++k) {
-    const Shape& sh = kShapes[k];
-    const int64_t cap = static_cast<int64_t>(sh.warps) * 32 * sh.hold * 16;
-    int tried = 0;
-    for (int C = 1; C <= 16 && tried < 3; ++C) {
-      const Plan pl = cut(V, es, C);
-      if (pl.slice * es > std::min(cap, kMaxSliceBytes)) continue;
-      ++tried;
-      const double clusters = sh.per_sm <= 4 ? kResident[sh.per_sm - 1][C - 1] : kResident[3][C - 1] * sh.per_sm / 4.0;
-      const double resident = clusters * static_cast<double>(V) * es / 1e6;  // MB
-      const double chain = 2.0 * resident / (sh.tau + sh.tau_c * C);
-      // one CTA per row and SM: the fewest streams at once, and no exchange through the cluster
-      const double alone = C == 1 && sh.per_sm == 1 ? 7.2 : 6.5;
-      const double memory = resident <= (C <= 3 ? sh.most : sh.most_wide) ? alone : 5.4;
-      const double rate = 1.0 / std::pow(std::pow(1.0 / chain, 4) + std::pow(1.0 / memory, 4), 0.25);
-      if (rate > best_rate) {
-        best = k;
-        best_rate = rate;
-        *plan = pl;
-      }
+// A CTA's slice of a row fits the registers that its shape holds it in, and a stage.
+constexpr bool fits(const Pick& p, int es) {
+  const int64_t epv = 16 / es, bytes = ((p.V + p.C - 1) / p.C + epv - 1) / epv * 16;
+  return bytes <= static_cast<int64_t>(kShapes[p.shape].warps) * 32 * kShapes[p.shape].hold * 16 &&
+         bytes <= kMaxSliceBytes;
+}
+template <int N>
+constexpr bool all_fit(const Pick (&t)[N], int es) {
+  for (int k = 0; k < N; ++k)
+    if (!fits(t[k], es) || (k > 0 && t[k].V <= t[k - 1].V)) return false;
+  return static_cast<int64_t>(t[N - 1].V) * es == 16 * kMaxSliceBytes;
+}
+static_assert(all_fit(kPicksBf16, 2) && all_fit(kPicksF32, 4), "every row up to the largest has a shape that holds it");
+
+template <int N>
+static int pick_shape(const Pick (&t)[N], int64_t V, int es, Plan* plan) {
+  for (const Pick& p : t)
+    if (V <= p.V) {
+      *plan = cut(V, es, p.C);
+      return p.shape;
     }
-  }
-  return best;
+  return -1;
 }
 
 // Launches a short-row kernel: as many CTAs as fit on the GPU at once, at most one warp per row.
@@ -1968,34 +1962,31 @@ static rl_status dispatch_loss(bool ent, RowArgs args, int64_t V, cudaStream_t s
   Plan plan = {};
   if constexpr (sizeof(T) == 4) {
     // fp32: slices of at most 30 KB on 3 CTAs per SM (another cut would change the order of the sums
-    // and with it the last bits), wider rows on the two widest shapes
+    // and with it the last bits), wider rows by kPicksF32
     const bool shift = args.ld % 4 != 0;
     if (make_plan(V, 4, &plan, 30 * 1024) && plan.slice * 4 <= kF32Hold * kF32Warps * 32 * 16) {
       if (!shift) return ent ? run(plan, launch_f32<true>) : run(plan, launch_f32<false>);
       return ent ? run(plan, launch_rows<T, 7, true, 9, 3, true>) : run(plan, launch_rows<T, 7, false, 9, 3, true>);
     }
-    const int k = pick_shape(V, 4, &plan, 5);
-    if (k < 0) return set_error(RL_ERR_UNSUPPORTED, "rl_policy_loss_fwd_bwd: row too large");
-    if (k == 5) {
-      if (shift) return ent ? run(plan, launch_rows<T, 16, true, 10, 1, true>) : run(plan, launch_rows<T, 16, false, 10, 1, true>);
-      return ent ? run(plan, launch_rows<T, 16, true, 10, 1>) : run(plan, launch_rows<T, 16, false, 10, 1>);
+#define RL_RUN(K, SHIFT) \
+  (ent ? run(plan, launch_rows<T, kShapes[K].warps, true, kShapes[K].hold, kShapes[K].per_sm, SHIFT>) \
+       : run(plan, launch_rows<T, kShapes[K].warps, false, kShapes[K].hold, kShapes[K].per_sm, SHIFT>))
+    switch (pick_shape(kPicksF32, V, 4, &plan)) {
+      case 4: return shift ? RL_RUN(4, true) : RL_RUN(4, false);
+      case 5: return shift ? RL_RUN(5, true) : RL_RUN(5, false);
     }
-    if (shift) return ent ? run(plan, launch_rows<T, 19, true, 11, 1, true>) : run(plan, launch_rows<T, 19, false, 11, 1, true>);
-    return ent ? run(plan, launch_rows<T, 19, true, 11, 1>) : run(plan, launch_rows<T, 19, false, 11, 1>);
   } else {
-#define RL_RUN(NW, H, B) (ent ? run(plan, launch_rows<T, NW, true, H, B>) : run(plan, launch_rows<T, NW, false, H, B>))
-    switch (pick_shape(V, 2, &plan, 0)) {
-      case 0: return RL_RUN(8, 10, 2);
-      case 1: return RL_RUN(7, 9, 3);
-      case 2: return RL_RUN(8, 6, 3);
-      case 3: return RL_RUN(4, 10, 4);
-      case 4: return RL_RUN(4, 5, 5);
-      case 5: return RL_RUN(16, 10, 1);
-      case 6: return RL_RUN(19, 11, 1);
+    switch (pick_shape(kPicksBf16, V, 2, &plan)) {
+      case 0: return RL_RUN(0, false);
+      case 1: return RL_RUN(1, false);
+      case 2: return RL_RUN(2, false);
+      case 3: return RL_RUN(3, false);
+      case 4: return RL_RUN(4, false);
+      case 5: return RL_RUN(5, false);
     }
 #undef RL_RUN
-    return set_error(RL_ERR_UNSUPPORTED, "rl_policy_loss_fwd_bwd: row too large");
   }
+  return set_error(RL_ERR_UNSUPPORTED, "rl_policy_loss_fwd_bwd: row too large");
 }
 
 constexpr int kFwdWarps = 8;
