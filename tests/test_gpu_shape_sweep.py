@@ -1,8 +1,8 @@
 """A seeded sweep of loss-call shapes against the float64 oracle (needs a GB300).
 
 Vocabulary sizes are drawn log-uniformly up to the largest rows the loss kernels accept
-(819,200 bf16, 409,600 fp32 entries), so the sweep crosses every cluster width the launcher
-picks (1 to 16 CTAs per row) and both sides of the 8 KB limit of the warp-per-row kernel;
+(819,200 bf16, 409,600 fp32 entries), so the sweep crosses many of the cluster widths and shapes the
+launcher picks (test_gpu_loss_shapes.py: all) and both sides of the 8 KB limit of the warp-per-row kernel;
 leading dimensions are padded by 0-8 elements (16-byte aligned or not), rows are taken anywhere
 in a workload's packed stream (its masks and owners), and the objective's optional terms
 (entropy bonus, k3 KL, TIS) and the three aggregation modes are drawn too. The row count keeps
@@ -15,15 +15,16 @@ import numpy as np
 import pytest
 import torch
 
+from loss_shapes import pick
 from parity_cases import compare, make_case, run_loss
 from paper_2608_16798_gb300 import workloads as W
 
 
 def _draw(n=40, seed=2026):
     """Cases 0-13: vocabularies log-uniform up to 8,192, mostly with rows on 16-byte boundaries
-    (the warp-per-row kernel where a row fits in 8 KB; one-CTA clusters otherwise); cases 14-39: a cluster width C drawn from 1-16 and a
-    vocabulary within that width's range (C x 40 KB of bf16 or C x 30 KB of fp32 per row), C = 16
-    up to the largest rows accepted."""
+    (the warp-per-row kernel where a row fits in 8 KB; one-CTA clusters otherwise); cases 14-39: a
+    number C drawn from 1-16 and a vocabulary of (C - 1) to C times 40 KB of bf16 or 30 KB of fp32 per row,
+    for C = 16 up to the largest rows accepted."""
     rng = np.random.default_rng(seed)
     cases = []
     for k in range(n):
@@ -32,13 +33,13 @@ def _draw(n=40, seed=2026):
         if k < 14:
             V = int(np.exp(rng.uniform(0.0, np.log(8192))))
         else:
-            span = 7680 if fp32 else 20480  # elements per CTA slice at the loss kernel's target
+            span = 7680 if fp32 else 20480
             C = int(rng.integers(1, 17))
             hi = (409_600 if fp32 else 819_200) if C == 16 else C * span
             V = int(rng.integers((C - 1) * span + 1, hi + 1))
         rows = int(max(1, min(48, 8_000_000 // V)))
         epv = 4 if fp32 else 8  # elements per 16 bytes
-        if k < 14 and rng.random() < 0.7:  # rows on 16-byte boundaries: the warp-per-row kernel
+        if k < 14 and rng.random() < 0.7:  # rows on 16-byte boundaries
             ld_pad = (-V) % epv + epv * int(rng.integers(0, 2))
         else:
             ld_pad = int(rng.integers(0, 9))
@@ -66,22 +67,15 @@ def R():
 
 
 def test_sweep_spans_the_kernel_shapes():
-    """The draw covers short rows and every cluster width the launcher can pick (no GPU needed)."""
-    widths = set()
-    short = 0
-    for _, name, V, ld_pad, *_ in CASES:
-        es = 4 if name == "edge" else 2
-        if V * es <= 8192 and ((V + ld_pad) * es) % 16 == 0:
-            short += 1
-            continue
-        target = 30 * 1024 if es == 4 else 40 * 1024
-        for C in range(1, 17):
-            per = -(-V // C)
-            slice_b = -(-per // (16 // es)) * 16
-            if slice_b <= target or (C == 16 and slice_b <= 100 * 1024):
-                widths.add(C)
-                break
-    assert short >= 5 and len(widths) >= 8, (short, sorted(widths))
+    """The draw covers short rows on and off the 16-byte boundaries, most cluster widths and most
+    shapes that the launcher picks (no GPU needed); the rest of them: test_gpu_loss_shapes.py."""
+    picks = [(name, pick("f32" if name == "edge" else "bf16", V), (V + ld_pad) * (4 if name == "edge" else 2) % 16 == 0)
+             for _, name, V, ld_pad, *_ in CASES]
+    short = [aligned for _, (kind, _), aligned in picks if kind == "warp"]
+    widths = {C for _, (kind, C), _ in picks if kind != "warp"}
+    shapes = {(name == "edge", kind) for name, (kind, _), _ in picks}
+    assert sum(short) >= 5 and len(short) > sum(short) and len(widths) >= 8 and len(shapes) >= 7, \
+        (short, sorted(widths), shapes)
 
 
 @pytest.mark.gpu
