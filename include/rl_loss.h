@@ -120,8 +120,8 @@ const char* rl_last_error_message(void);
  * (min(max_rows, 4096) * ceil(V / 8) * 8 * 2 bytes: 1.24 GB at V = 151,936);
  * others are the packed hidden states of one chunk and, for few tokens, partial
  * sums of d_hidden. A smaller workspace, without room for the last two, is
- * accepted by rl_fused_head_loss_fwd_bwd down to what the others take; every
- * token then goes through the products. */
+ * accepted by rl_fused_head_loss_fwd_bwd down to what the others take; without
+ * room for the packed hidden states every token goes through the products. */
 size_t rl_workspace_size(int64_t max_rows, int64_t V, int64_t D);
 
 /* Workspace bytes with which rl_fused_head_loss_fwd_bwd on up to T tokens keeps the
@@ -232,6 +232,9 @@ rl_status rl_token_logprobs(const void* logits, rl_dtype dtype, int64_t rows, in
  * Every other row gets an exactly-zero gradient row and contributes nothing.
  * Logits at -inf have probability 0 (and a zero gradient); a NaN logit makes its own row's
  * loss term, statistics and gradient NaN (so the loss is NaN) and leaves the other rows alone.
+ * A row's results do not depend on the other rows or on their number: the same bits in any
+ * microbatch. Only where it starts counts, for bf16 rows whose ld is no multiple of 8: they are summed
+ * by the 16-byte blocks of memory they cover, so their last bits depend on r ld mod 8.
  *
  *   logits        [rows x ld] of `dtype`, base 16-byte aligned
  *   rows, V, ld   rows >= 0, 1 <= V <= ld; V at most 819,200 (bf16) or 409,600 (fp32), as
@@ -285,16 +288,19 @@ rl_status rl_policy_loss_fwd_bwd(const void* logits, rl_dtype dtype, int64_t row
  *                 4,096 tokens, or of a group of several chunks when ws_bytes allows
  *                 (rl_fused_head_workspace_size), consumed by the dH and dW products
  * Tokens that are not trained on (M_t = 0, c = 0, a bad id or owner) enter none of the
- * products, whatever their hidden states hold. The others are packed and processed in chunks
+ * products, whatever their hidden states hold (but with a workspace below rl_workspace_size that
+ * has no room for packing they go through them with a zero gradient, and a NaN or infinite
+ * hidden state of theirs makes d_weight NaN). The others are packed and processed in chunks
  * of at most 4,096: per chunk, one tensor-core pass forms the logits tile by tile, folds them
  * into softmax partials and keeps exp(z - tile max) in bf16 with the tile maxima; a per-token
  * merge evaluates the objective; an in-place rescale turns the kept values into the logits'
  * gradient. After the last chunk of each group (each chunk, with the smallest workspace), two
  * tensor-core products give the group's dH and add its dW (fp32, one addition per element and
- * group, in chunk order: deterministic). The groups follow ws_bytes, and the blocks of the
- * vocabulary and the parts of dH's contraction follow T, so the rounding of d_weight and
- * d_hidden (not their values up to rounding) depends on both; calls with the same T and
- * ws_bytes give the same bits. The logits of all T tokens are never held at once.
+ * group, in chunk order: deterministic). The groups follow ws_bytes and the parts of dH's
+ * contraction follow T, so the rounding of d_weight and d_hidden (not their values up to
+ * rounding) depends on both; calls with the same T and ws_bytes give the same bits. A token's
+ * statistics depend on neither, and are the bits of rl_fused_head_token_logprobs. The logits of all T
+ * tokens are never held at once.
  */
 rl_status rl_fused_head_loss_fwd_bwd(const void* hidden, const void* weight, int64_t T, int64_t D, int64_t V,
                                      const int32_t* token_ids, const uint8_t* mask, const int32_t* token_traj,
@@ -468,11 +474,12 @@ rl_status rl_sequence_is_weights(int32_t n_traj, int64_t n_tokens, const int32_t
  *   entropy_out  float [T] or NULL (entropy work is skipped when NULL)
  *   lse_out      float [T] or NULL
  *   ws, ws_bytes workspace; rl_workspace_size(T, V, D) bytes always suffice (the
- *                call uses the status word and softmax partials after it: two of 16 bytes per
- *                token and vocabulary block, at least 32 * ceil(V / 4096) * min(T, 4096) bytes;
- *                more allow smaller blocks, which few tokens need to fill the GPU)
+ *                call uses the status word and softmax partials after it,
+ *                at least 32 * ceil(V / 4096) * min(T, 4096) bytes; with more, few tokens
+ *                are spread over the GPU in smaller work items)
  * One tensor-core pass per chunk of 4,096 tokens, then a per-token merge of the
- * vocabulary blocks' partials in fixed order (deterministic).
+ * partials in an order that depends on V alone: a token's results are the same bits in
+ * any call.
  */
 rl_status rl_fused_head_token_logprobs(const void* hidden, const void* weight, int64_t T, int64_t D, int64_t V,
                                        const int32_t* token_ids, float* logp_out, float* entropy_out,

@@ -18,8 +18,9 @@
 // the even CTA's barrier and the MMA's commits are multicast to both). Sharing A between two
 // MMAs moves a quarter fewer operand bytes through shared memory and L2 per flop than 256 x
 // 256 tiles, which is what lets the MMAs run close to their peak rate. The epilogue drains
-// TMEM 32 columns at a time into a swizzled shared-memory slab and hands it to the TMA: a
-// tiled store into d_hidden (bf16 or fp32) or a tiled reduce-add into the fp32 d_weight.
+// TMEM 32 columns at a time: a dW tile into a swizzled shared-memory slab, which the TMA adds to the
+// fp32 d_weight (a tiled reduce-add); a dH tile from the registers to its tokens' rows of d_hidden (bf16
+// or fp32), or to a part's sums.
 //
 // Work items are dH tiles (each the whole contraction over V: long) followed by dW tiles
 // (contraction over the n tokens: short), handed out by a counter in global memory as pairs
@@ -82,8 +83,8 @@ struct GradArgs {
 enum HOut { H_F32 = 0, H_BF16 = 1 };
 
 // The tokens' loss contributions added in a fixed order into the caller's total by the four epilogue
-// warps of CTA 0, while its first accumulator fills (a launch of its own took 8 us at 500 tokens, the rescale's last
-// CTA 5).
+// warps of CTA 0, while its first accumulator fills (at 500 tokens a launch of its own took 8 us, the
+// rescale's last CTA 5).
 // Thread k adds tokens k, k + 128, ... into eight accumulators in turn (eight loads in flight).
 __device__ __forceinline__ void sum_loss(const GradArgs& p) {
   __shared__ double part[4];
