@@ -238,29 +238,30 @@ struct RowMeta {
 // fresh partial, the first vector's maximum; when the exponentials sum above 1e30
 // (a value far above the reference) everything is redone against the exact
 // maximum. Values at or below -1e38 count as -inf.
-template <typename T, bool ENT, int NV, typename Reload>
+template <typename T, bool ENT, int NV, bool NAN_REF = true, typename Reload>
 __device__ __forceinline__ void fold_block(SoftmaxPartial& ps, const uint4 (&x)[NV], Reload reload) {
   constexpr int NP = Vec<T>::NP;
-  // NaN if any value is: it then becomes the reference and poisons the sums, also where a thread has
-  // nothing but NaNs
+  // NAN_REF: NaN if any value is, so that a thread that has nothing but NaNs (and -inf) takes one as its
+  // reference, which poisons the sums; else the largest of the others
+  auto larger = [](float a, float b) { return NAN_REF ? max_nan(a, b) : fmaxf(a, b); };
   auto vmax = [&](const uint4 w) {
     float2 q[NP];
     Vec<T>::pairs(w, q);
-    float m = max_nan(q[0].x, q[0].y);
+    float m = larger(q[0].x, q[0].y);
 #pragma unroll
-    for (int i = 1; i < NP; ++i) m = max_nan(m, max_nan(q[i].x, q[i].y));
+    for (int i = 1; i < NP; ++i) m = larger(m, larger(q[i].x, q[i].y));
     return m;
   };
   // exact maximum, recomputed from shared memory (the rare paths only)
   auto all_max = [&]() {
     float m = vmax(reload(0));
-    for (int k = 1; k < NV; ++k) m = max_nan(m, vmax(reload(k)));
+    for (int k = 1; k < NV; ++k) m = larger(m, vmax(reload(k)));
     return m;
   };
   if (!(ps.m > -1e38f)) {
     float m0 = vmax(x[0]);
     if (!(m0 > -1e38f)) m0 = all_max();
-    if (m0 <= -1e38f) return;
+    if (NAN_REF ? m0 <= -1e38f : !(m0 > -1e38f)) return;
     ps.m = m0;
   }
   // x = (z - m) log2(e) by one fused multiply-add against nm = fl(-m log2(e)); with the
@@ -1294,14 +1295,25 @@ struct SmallRow {
   __device__ __forceinline__ SoftmaxPartial fold(int lane) {
     SoftmaxPartial ps{RL_NEG_INF, 0.f, 0.f};
     fold_part<ENT>(ps, lane);
-    return finish<ENT>(ps);
+    return finish<ENT>(ps, ps.s == 0.f, lane);
   }
   template <bool ENT>
   __device__ __forceinline__ void fold_part(SoftmaxPartial& ps, int lane) {
-    fold_block<T, ENT>(ps, x, [&](int k) { return block(k, lane); });
+    fold_block<T, ENT, NV, false>(ps, x, [&](int k) { return block(k, lane); });
   }
+  // A lane that had seen nothing after some part (`none`) had only -inf or NaNs there, which no maximum
+  // sees: looked for here, where the row's words are no longer held (kept as references, as the cluster
+  // kernels do, they cost 5 to 7% of the forward call at 4,096 and 5,000 entries).
   template <bool ENT>
-  __device__ __forceinline__ SoftmaxPartial finish(SoftmaxPartial ps) {
+  __device__ __forceinline__ SoftmaxPartial finish(SoftmaxPartial ps, bool none, int lane) {
+    if (none) {
+      for (int j = lane; j < span.vecs; j += 32) {
+        float2 q[Vec<T>::NP];
+        Vec<T>::pairs(reinterpret_cast<const uint4*>(row + span.head)[j], q);
+        for (int i = 0; i < Vec<T>::NP; ++i)
+          if (q[i].x != q[i].x || q[i].y != q[i].y) ps.s = __int_as_float(0x7fffffff);
+      }
+    }
     if (edge >= 0 && ez != RL_NEG_INF) {
       raise_max<ENT>(ps, ez);
       accumulate<ENT>(ps, ez, -ps.m * kLog2e);
@@ -1509,13 +1521,15 @@ __global__ void __launch_bounds__(kSmallWarps * 32, small_ctas<T, NV>(false)) sm
     next = r + all_warps < p.rows ? p.token_ids[r + all_warps] : 0;
     SoftmaxPartial ps{RL_NEG_INF, 0.f, 0.f};
     sr.template fold_part<ENT>(ps, lane);
+    bool none = ps.s == 0.f;
     if (NV == 16) {
       for (int first = 32 * NV; first < sr.span.vecs; first += 32 * NV) {
         sr.load(lane, first);
         sr.template fold_part<ENT>(ps, lane);
+        none = none || ps.s == 0.f;
       }
     }
-    const SoftmaxPartial q = sr.template finish<ENT>(ps);
+    const SoftmaxPartial q = sr.template finish<ENT>(ps, none, lane);
     if (lane == 0) {
       const float lnS = logf(q.s);
       const float lse = q.m + lnS;
