@@ -1567,8 +1567,9 @@ struct ChunkInfo {
   int32_t last;   // the row's last chunk: 1, or 2 if the sampled token is out of range
 };
 
-template <typename T, int NW, bool ENT>
-__global__ void __launch_bounds__((NW + 1) * 32, 2) stream_logprobs_kernel(const StreamArgs p) {
+// MINB: CTAs per SM the register budget is sized for (2 leaves 64 to 72 registers, 3 CTAs).
+template <typename T, int NW, bool ENT, int MINB>
+__global__ void __launch_bounds__((NW + 1) * 32, MINB) stream_logprobs_kernel(const StreamArgs p) {
   constexpr int EPV = Vec<T>::N;
   constexpr int NS = FwdCfg<ENT>::kStages;
   constexpr int NC = NW * 32;
@@ -2005,6 +2006,31 @@ static rl_status dispatch_loss(bool ent, RowArgs args, int64_t V, cudaStream_t s
 
 constexpr int kFwdWarps = 8;
 
+// CTAs of a streaming kernel that fit on the GPU at once.
+static rl_status stream_grid(void (*kern)(StreamArgs), size_t smem, int* grid) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return cuda_error(e, "cudaGetDevice");
+  rl_status st = configure(reinterpret_cast<const void*>(kern), dev, smem);
+  if (st != RL_OK) return st;
+  static std::mutex mu;
+  static std::map<std::pair<const void*, int>, int> cache;
+  std::lock_guard<std::mutex> lock(mu);
+  auto key = std::make_pair(reinterpret_cast<const void*>(kern), dev);
+  auto it = cache.find(key);
+  if (it == cache.end()) {
+    int per_sm = 0, sms = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, (kFwdWarps + 1) * 32, smem);
+    if (e != cudaSuccess) return cuda_error(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
+    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return cuda_error(e, "cudaDeviceGetAttribute");
+    if (per_sm <= 0) return set_error(RL_ERR_UNSUPPORTED, "stream kernel does not fit on an SM");
+    it = cache.emplace(key, per_sm * sms).first;
+  }
+  *grid = it->second;
+  return RL_OK;
+}
+
 template <typename T, bool ENT>
 static rl_status launch_stream(StreamArgs args, cudaStream_t s) {
   const int64_t row_bytes = args.V * static_cast<int64_t>(sizeof(T));
@@ -2015,39 +2041,31 @@ static rl_status launch_stream(StreamArgs args, cudaStream_t s) {
       default: return launch_small(small_logprobs_kernel<T, ENT, 16>, args, s);
     }
   }
-  auto kern = stream_logprobs_kernel<T, kFwdWarps, ENT>;
   args.chunk = FwdCfg<ENT>::kChunkKB * 1024 / 16;
   // the chunk, then the row's two partial blocks, to a multiple of 128 bytes
   args.buf_elems = (static_cast<int64_t>(args.chunk) * 16 + 128) / static_cast<int64_t>(sizeof(T));
   const size_t smem = static_cast<size_t>(FwdCfg<ENT>::kStages) * args.buf_elems * sizeof(T);
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return cuda_error(e, "cudaGetDevice");
-  rl_status st = configure(reinterpret_cast<const void*>(kern), dev, smem);
-  if (st != RL_OK) return st;
-  static std::mutex mu;
-  static std::map<std::pair<const void*, int>, int> grid_cache;
+  auto kern = stream_logprobs_kernel<T, kFwdWarps, ENT, 2>;
   int grid = 0;
-  {
-    std::lock_guard<std::mutex> lock(mu);
-    auto key = std::make_pair(reinterpret_cast<const void*>(kern), dev);
-    auto it = grid_cache.find(key);
-    if (it != grid_cache.end()) {
-      grid = it->second;
-    } else {
-      int per_sm = 0, sms = 0;
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, (kFwdWarps + 1) * 32, smem);
-      if (e != cudaSuccess) return cuda_error(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
-      e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-      if (e != cudaSuccess) return cuda_error(e, "cudaDeviceGetAttribute");
-      if (per_sm <= 0) return set_error(RL_ERR_UNSUPPORTED, "stream kernel does not fit on an SM");
-      grid = per_sm * sms;
-      grid_cache[key] = grid;
+  rl_status st = stream_grid(kern, smem, &grid);
+  if (st != RL_OK) return st;
+  if constexpr (sizeof(T) == 4) {
+    // fp32 rows are long, and few of them may fill their last round of the grid badly: with 4 CTAs per SM
+    // where that takes fewer places. 0.8 GB of rows: 1,316 rows of 151,936 entries 116 us on 3 CTAs per SM
+    // (1,368 places) and 125 on 4 (1,824), 999 of 200,064 126 and 118, 500 of 400,000 147 and 117.
+    auto kern4 = stream_logprobs_kernel<T, kFwdWarps, ENT, 4>;
+    int grid4 = 0;
+    st = stream_grid(kern4, smem, &grid4);
+    if (st != RL_OK) return st;
+    auto places = [&](int64_t g) { return (args.rows + g - 1) / g * g; };
+    if (places(grid4) < places(grid)) {
+      kern = kern4;
+      grid = grid4;
     }
   }
   const unsigned blocks = static_cast<unsigned>(std::min<int64_t>(grid, args.rows));
   kern<<<blocks, (kFwdWarps + 1) * 32, smem, s>>>(args);
-  e = cudaGetLastError();
+  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_error(e, "stream_logprobs_kernel launch");
   return RL_OK;
 }
