@@ -621,37 +621,37 @@ struct DzArgs {
   int32_t* status;
 };
 
-// Token r's partials, merged by a warp: lane l takes the block partials l, l + 32, ... in order, the
-// lanes are combined by shuffles (in head_dz_kernel and in head_logp_merge_kernel: the loss call and
-// the forward-only call give the same bits). Where the statistics pass left every tile's own (n_tile of
-// them, else 0), a block's partial is formed here first, tile by tile as the pass would. One trip to
-// memory per 32 partials, or two: a thread per token walking them 8 loads at a time took 16 us for
-// 4,096 tokens, a warp 6.
-__device__ __forceinline__ void merge_partials(const float4* partials, int64_t Tc, int r, int n_part, int n_tile,
+// A token's partials (`stride` apart), merged by a warp: lane l takes the block partials l, l + 32, ... in
+// order, the lanes are combined by shuffles (in head_dz_kernel and in head_logp_merge_kernel: the loss
+// call and the forward-only call give the same bits). Where the statistics pass left every tile's own
+// (n_tile of them, else 0), a block's partial is formed here first, tile by tile as the pass would, with
+// LOADS of them in flight. A thread per token walking them 8 loads at a time took 16 us for 4,096 tokens,
+// a warp 6.
+template <int LOADS>
+__device__ __forceinline__ void merge_partials(const float4* partials, int64_t stride, int n_part, int n_tile,
                                                SoftmaxPartial& q, float& za) {
   const int lane = threadIdx.x & 31;
-  const float4 none = make_float4(-__int_as_float(0x7f800000), 0.f, 0.f, 0.f);
   if (n_tile == 0) {
 #pragma unroll 4
     for (int b = lane; b < n_part; b += 32) {
-      const float4 w = partials[static_cast<int64_t>(b) * Tc + r];
+      const float4 w = partials[b * stride];
       q = merge(q, SoftmaxPartial{w.x, w.y, w.z});
       za += w.w;  // nonzero in the one partial whose columns hold the sampled id
     }
   } else {
     for (int b = lane; b < n_part; b += 32) {
       const int first = (b >> 1) * kMaxVb + (b & 1);
-      SoftmaxPartial blk{none.x, 0.f, 0.f};
+      SoftmaxPartial blk{-__int_as_float(0x7f800000), 0.f, 0.f};
 #pragma unroll
-      for (int h = 0; h < kMaxVb; h += 8) {
-        float4 w[4];
+      for (int h = 0; h < kMaxVb; h += 2 * LOADS) {
+        float4 w[LOADS];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 0; k < LOADS; ++k) {
           const int nt = first + h + 2 * k;
-          w[k] = nt < n_tile ? partials[static_cast<int64_t>(nt) * Tc + r] : none;
+          if (nt < n_tile) w[k] = partials[nt * stride];
         }
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 0; k < LOADS; ++k) {
           if (first + h + 2 * k >= n_tile) break;
           blk = merge(blk, SoftmaxPartial{w[k].x, w[k].y, w[k].z});
           za += w[k].w;
@@ -670,7 +670,8 @@ constexpr int kMergeRows = kMergeThreads / 32;
 // Row r's coefficients, by one warp (the same in every lane): the vocabulary blocks' partials merged
 // in a fixed order and the per-token objective terms. With `write` lane 0 also writes the token's
 // loss contribution and statistics. The words that need only the token are loaded together.
-__device__ __forceinline__ RowCoef row_coef(const DzArgs& p, const Chunk& ch, int r, bool write) {
+__device__ __forceinline__ RowCoef row_coef(const DzArgs& p, const Chunk& ch, int r, const float4* partials, int64_t stride,
+                                            bool write) {
   const int64_t t = token_of(p.tok, ch, r);
   const uint8_t m = p.mask[t];
   const int32_t i = p.token_traj[t], a = p.token_ids[t];
@@ -679,7 +680,7 @@ __device__ __forceinline__ RowCoef row_coef(const DzArgs& p, const Chunk& ch, in
   const float roll = p.rollout_logp ? p.rollout_logp[t] : 0.f;
   SoftmaxPartial q{-__int_as_float(0x7f800000), 0.f, 0.f};
   float za = 0.f;
-  merge_partials(p.partials, p.tok.Tc, r, p.n_part, p.n_tile, q, za);
+  merge_partials<4>(partials, stride, p.n_part, p.n_tile, q, za);
   write = write && (threadIdx.x & 31) == 0;
   RowCoef rc = {};
   rc.a = -1;
@@ -745,6 +746,7 @@ __device__ __forceinline__ RowCoef row_coef(const DzArgs& p, const Chunk& ch, in
 
 constexpr int kDzThreads = 256;
 constexpr int kDzLoads = 4;          // vectors in flight per thread
+constexpr int kTilesStaged = 640;    // tile partials of a row staged in shared memory: V up to 163,840
 constexpr int kMaxTilesSmem = 2048;  // V up to 524,288 keeps the row's tile factors in shared memory
 
 // p.split CTAs per token row of the chunk (grid-stride): the CTA's first warp merges the row's
@@ -760,6 +762,7 @@ constexpr int kMaxTilesSmem = 2048;  // V up to 524,288 keeps the row's tile fac
 __global__ void __launch_bounds__(kDzThreads, 4) head_dz_kernel(const DzArgs p) {
   __shared__ float fac[kMaxTilesSmem], zoff[kMaxTilesSmem];
   __shared__ RowCoef shared_rc;
+  __shared__ float4 tiles[kTilesStaged];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const Chunk ch = chunk_of(p.tok, p.chunk);
   if (blockIdx.x == 0 && tid == 0) *p.counter = 0u;
@@ -788,8 +791,14 @@ __global__ void __launch_bounds__(kDzThreads, 4) head_dz_kernel(const DzArgs p) 
     };
     load(k_lo + tid);
     float m = j_lo + tid < j_hi ? p.tmax[static_cast<int64_t>(r) * p.n_nt + j_lo + tid] : 0.f;
+    // many tile partials (V above 16,384) come in one trip of the whole CTA
+    const bool staged = p.n_tile > 64 && p.n_tile <= kTilesStaged;
+    if (staged) {
+      for (int t = tid; t < p.n_tile; t += kDzThreads) tiles[t] = p.partials[static_cast<int64_t>(t) * p.tok.Tc + r];
+      __syncthreads();
+    }
     if (warp == 0) {
-      const RowCoef c = row_coef(p, ch, r, part == 0);
+      const RowCoef c = row_coef(p, ch, r, staged ? tiles : p.partials + r, staged ? 1 : p.tok.Tc, part == 0);
       if (lane == 0) shared_rc = c;
     }
     __syncthreads();
@@ -844,8 +853,8 @@ __global__ void __launch_bounds__(kDzThreads, 4) head_dz_kernel(const DzArgs p) 
       if (v == rc.a) x += rc.cg;
       row[v] = f32_to_bf16(x);
     }
-    // the next row's shared_rc is written past this row's second barrier, its fac and zoff past the
-    // next row's first: every read of this row's comes before
+    // the next row's shared_rc and tiles are written past this row's last barrier, its fac and zoff past
+    // the next row's first: every read of this row's comes before
   }
 }
 
@@ -870,7 +879,7 @@ __global__ void __launch_bounds__(kMergeThreads) head_logp_merge_kernel(const Lo
   const int64_t t = token_of(p.tok, ch, r);
   SoftmaxPartial q{-__int_as_float(0x7f800000), 0.f, 0.f};
   float za = 0.f;
-  merge_partials(p.partials, p.tok.Tc, r, p.n_part, p.n_tile, q, za);
+  merge_partials<8>(p.partials + r, p.tok.Tc, p.n_part, p.n_tile, q, za);
   if (!lead) return;
   const float lnS = logf(q.s);
   const float lse = q.m + lnS;
