@@ -94,7 +94,6 @@ struct HeadArgs {
   int32_t chunk;           // which chunk of them
   int32_t D, V, vb_tiles, n_vb, n_nt;  // N tiles per work item (even), items and tiles per row tile
   int32_t ent;
-  int32_t tile_parts;      // partials of every tile instead of two per work item
   const int32_t* token_ids;
   float4* partials;        // (m, s, u, z_a): [2 n_vb][Tc], a block's even tiles, then its odd ones, or [n_nt][Tc]
   uint16_t* dz;            // [G Tc x ldz] bf16: e = exp(z - m_j) (STATS_P), the group's chunks in turn
@@ -111,7 +110,7 @@ struct HeadArgs {
 // CTAs, and each CTA's epilogue drains its own 128 TMEM lanes (all 256 columns) and tells the
 // even CTA's MMA thread when an accumulator is free. Per pair this halves the W operand each SM
 // fetches and stages per MMA.
-template <int MODE, bool PAIR>
+template <int MODE, bool PAIR, bool TILE_PARTS>
 __global__ void __launch_bounds__(kThreads, 1) head_kernel(const __grid_constant__ CUtensorMap tmH,
                                                            const __grid_constant__ CUtensorMap tmW,
                                                            const HeadArgs p) {
@@ -248,7 +247,7 @@ __global__ void __launch_bounds__(kThreads, 1) head_kernel(const __grid_constant
       const bool row_ok = r < ch.count;
       const int nt1 = min((vb + 1) * p.vb_tiles, p.n_nt);
       // running partials of the block's even and odd tiles (the halves of its 256 x 512 tiles);
-      // with tile_parts the tiles' own
+      // with TILE_PARTS the tiles' own go out
       SoftmaxPartial ps0{kNegInf, 0.f, 0.f}, ps1{kNegInf, 0.f, 0.f};
       float za = 0.f;
       const int32_t a = row_ok ? p.token_ids[token_of(p.tok, ch, r)] : -1;
@@ -327,7 +326,7 @@ __global__ void __launch_bounds__(kThreads, 1) head_kernel(const __grid_constant
         }
         if (MODE == STATS_P && row_ok) p.tmax[static_cast<int64_t>(r) * p.n_nt + nt] = tm;
         const SoftmaxPartial tile{tm, s0 + s1, u0};
-        if (p.tile_parts) {
+        if (TILE_PARTS) {
           if (row_ok) p.partials[static_cast<int64_t>(nt) * p.tok.Tc + r] = make_float4(tile.m, tile.s, tile.u, za);
           za = 0.f;
         } else if (nt & 1) {
@@ -336,7 +335,7 @@ __global__ void __launch_bounds__(kThreads, 1) head_kernel(const __grid_constant
           ps0 = merge(ps0, tile);
         }
       }
-      if (ok && row_ok && !p.tile_parts) {
+      if (ok && row_ok && !TILE_PARTS) {
         p.partials[static_cast<int64_t>(2 * vb) * p.tok.Tc + r] = make_float4(ps0.m, ps0.s, ps0.u, za);
         p.partials[static_cast<int64_t>(2 * vb + 1) * p.tok.Tc + r] = make_float4(ps1.m, ps1.s, ps1.u, 0.f);
       }
@@ -437,7 +436,7 @@ __device__ __forceinline__ SoftmaxPartial epi_half(uint32_t tacc, int n0, int V,
 // warps 6-9 its second 256, each group with its own running partial (two per vocabulary block)
 constexpr int kThreadsW = 320;
 
-template <int MODE>
+template <int MODE, bool TILE_PARTS>
 __global__ void __launch_bounds__(kThreadsW, 1) head_wide_kernel(const __grid_constant__ CUtensorMap tmH,
                                                                 const __grid_constant__ CUtensorMap tmW,
                                                                 const HeadArgs p) {
@@ -568,7 +567,7 @@ __global__ void __launch_bounds__(kThreadsW, 1) head_wide_kernel(const __grid_co
           const SoftmaxPartial half =
               epi_half<MODE>(tq + h * BN, j * BN, p.V, a, p.ent, dz_row ? dz_row + j * BN : nullptr, za, tm);
           if (MODE == STATS_P && row_ok) p.tmax[static_cast<int64_t>(r) * p.n_nt + j] = tm;
-          if (p.tile_parts) {
+          if (TILE_PARTS) {
             if (row_ok) p.partials[static_cast<int64_t>(j) * p.tok.Tc + r] = make_float4(half.m, half.s, half.u, za);
             za = 0.f;
           } else {
@@ -582,7 +581,7 @@ __global__ void __launch_bounds__(kThreadsW, 1) head_wide_kernel(const __grid_co
           else mbar_arrive(&acce);
         }
       }
-      if (ok && row_ok && !p.tile_parts)
+      if (ok && row_ok && !TILE_PARTS)
         p.partials[static_cast<int64_t>(2 * vb + h) * p.tok.Tc + r] = make_float4(ps.m, ps.s, ps.u, za);
     }
   }
@@ -791,8 +790,8 @@ __global__ void __launch_bounds__(kDzThreads, 4) head_dz_kernel(const DzArgs p) 
     };
     load(k_lo + tid);
     float m = j_lo + tid < j_hi ? p.tmax[static_cast<int64_t>(r) * p.n_nt + j_lo + tid] : 0.f;
-    // many tile partials (V above 16,384) come in one trip of the whole CTA
-    const bool staged = p.n_tile > 64 && p.n_tile <= kTilesStaged;
+    // a short call's tile partials come in one trip of the whole CTA
+    const bool staged = p.n_tile != 0 && p.n_tile <= kTilesStaged;
     if (staged) {
       for (int t = tid; t < p.n_tile; t += kDzThreads) tiles[t] = p.partials[static_cast<int64_t>(t) * p.tok.Tc + r];
       __syncthreads();
@@ -1148,10 +1147,13 @@ static Layout layout_in(int64_t T, int64_t V, int64_t D, size_t ws_bytes) {
 #define RL_HEAD_WIDE 1
 #endif
 
-template <int MODE>
-static rl_status launch_head(const CUtensorMap& mh, const CUtensorMap& mw, const HeadArgs& a, cudaStream_t s) {
+template <int MODE, bool TILE_PARTS>
+static rl_status launch_head_form(const CUtensorMap& mh, const CUtensorMap& mw, const HeadArgs& a, cudaStream_t s) {
   constexpr bool kWide = ((RL_HEAD_WIDE >> MODE) & 1) != 0;
-  auto kern = kWide ? head_wide_kernel<MODE> : head_kernel<MODE, kPair>;
+  auto kern = [] {
+    if constexpr (kWide) return head_wide_kernel<MODE, TILE_PARTS>;
+    else return head_kernel<MODE, kPair, TILE_PARTS>;
+  }();
   constexpr size_t smem = kWide ? kSmemW : (kPair ? kSmem2 : kSmem);
   int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -1203,6 +1205,12 @@ static rl_status launch_head(const CUtensorMap& mh, const CUtensorMap& mw, const
     if (e != cudaSuccess) return cuda_error(e, "head_kernel launch");
   }
   return RL_OK;
+}
+
+template <int MODE>
+static rl_status launch_head(const CUtensorMap& mh, const CUtensorMap& mw, const HeadArgs& a, bool tile_parts,
+                             cudaStream_t s) {
+  return tile_parts ? launch_head_form<MODE, true>(mh, mw, a, s) : launch_head_form<MODE, false>(mh, mw, a, s);
 }
 
 }  // namespace head
@@ -1344,7 +1352,6 @@ extern "C" rl_status rl_fused_head_loss_fwd_bwd(
     ha.n_nt = n_nt;
     ha.vb_tiles = static_cast<int>(L.vb);
     ha.n_vb = static_cast<int>(L.n_vb);
-    ha.tile_parts = L.tile_parts ? 1 : 0;
     ha.ent = ent ? 1 : 0;
     ha.token_ids = token_ids;
     ha.partials = partials;
@@ -1352,7 +1359,7 @@ extern "C" rl_status rl_fused_head_loss_fwd_bwd(
     ha.ldz = L.ldz;
     ha.tmax = tmax;
     ha.status = status;
-    st = launch_head<STATS_P>(mh, mw, ha, s);
+    st = launch_head<STATS_P>(mh, mw, ha, L.tile_parts, s);
     if (st != RL_OK) return st;
 
     DzArgs da = {};
@@ -1453,12 +1460,11 @@ extern "C" rl_status rl_fused_head_token_logprobs(const void* hidden, const void
     ha.n_nt = static_cast<int>(L.n_nt);
     ha.vb_tiles = static_cast<int>(L.vb);
     ha.n_vb = static_cast<int>(L.n_vb);
-    ha.tile_parts = L.tile_parts ? 1 : 0;
     ha.ent = entropy_out ? 1 : 0;
     ha.token_ids = token_ids;
     ha.partials = partials;
     ha.status = status;
-    st = launch_head<STATS>(mh, mw, ha, s);
+    st = launch_head<STATS>(mh, mw, ha, L.tile_parts, s);
     if (st != RL_OK) return st;
     LogpMergeArgs ma = {};
     ma.tok = tok;
