@@ -868,11 +868,12 @@ __global__ void __launch_bounds__((NW + 1) * 32, MINB) rows_kernel(const RowArgs
 // fp32 rows of up to 129,024 entries whose leading dimension is a multiple of four keep a kernel of
 // their own: the same split as rows_kernel's fp32 form and the same bits (the order of the sums is
 // part of the fp32 path's results, see merge_lanes), with a row's words held by each consumer and its
-// places worked out there. A stage is released only once the row's exchange has arrived: copies
-// issued earlier compete with the gradient's stores. On the edge batch (32,768 rows of 32,000 entries, 38%
-// of them zero-filled; HBM's floor 999 us) that takes 1,066 us, an early release 1,102 to 1,147 us (1,067
-// where a register spill happened to hold the consumers back), and rows_kernel on the same shape,
-// whose producer works out more per row before it may issue the next copies, 1,136 us either way.
+// places worked out there. A stage is released only once the row's exchange has arrived. On the edge
+// batch (32,768 rows of 32,000 entries, 38% of them zero-filled; HBM's floor 1,008 us) that takes 1,066 us, an
+// early release 1,102 to 1,147 us, and rows_kernel on the same shape 1,136 us either way. How the compiler
+// allots the consumers' registers moves this kernel by 5%, by V in either direction (a build without its
+// 4 bytes of spills 1,140 us there, but 6% faster at 80,000 entries); why is not known. Fewer clusters than
+// fit, a release after the gradient's stores: slower.
 // Slices of at most 30 KB (clusters of 5 at V = 32,000), 7 consumer warps of up to 9
 // vectors, 3 CTAs per SM: 4.15 ms per 131,072 rows against 4.35 with clusters of 4 at 2 per SM.
 constexpr int kF32Warps = 7, kF32Hold = 9;
