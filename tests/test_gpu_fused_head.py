@@ -138,30 +138,31 @@ def test_fused_head_parity(R, T, D, V, agg, ent, tis):
 
 @pytest.mark.parametrize("group_tokens", [0, 6000, 3 * 4096])
 def test_fused_head_three_chunks_bf16_grad(R, group_tokens):
-    """More than 8,192 tokens, bf16 d_hidden. With the smallest workspace each chunk of 4,096 is
-    its own group and dW is added three times; with room for two chunks (6,000 tokens round up
-    to two) the groups are two chunks and a ragged last one; with room for three the group
-    holds them all and dW is added once."""
-    c = make_head_case(8192 + 77, 128, 1100, seed=5, agg=2)
+    """More than 8,192 tokens, all trained on, bf16 d_hidden: three chunks. With the smallest
+    workspace each is its own group and dW is added three times; with room for two chunks (6,000
+    tokens round up to two) the groups are two chunks and a ragged last one; with room for three
+    the group holds them all and dW is added once."""
+    c = make_head_case(8192 + 77, 128, 1100, seed=5, agg=2, masked=0.0)
     out = run_head(R, c, dh_dtype=torch.bfloat16, group_tokens=group_tokens)
     compare_head(c, out, dh_bf16=True)
 
 
 @pytest.mark.parametrize("group_tokens", [0, 32768])
 def test_fused_head_ten_chunks(R, group_tokens):
-    """More than 32,768 tokens: ten chunks, each its own group (the smallest workspace: dW
-    added ten times), or a full group of eight and a ragged second group of two (dH stored in
-    fp32 over 32,768 tokens, the second group's dW added onto the first's)."""
-    c = make_head_case(32768 + 4096 + 50, 64, 600, seed=11, agg=0, ent=True)
+    """More than 32,768 tokens, all trained on: ten chunks, each its own group (the smallest
+    workspace: dW added ten times), or a full group of eight and a ragged second group of two (dH
+    stored in fp32 over 32,768 tokens, the second group's dW added onto the first's)."""
+    c = make_head_case(32768 + 4096 + 50, 64, 600, seed=11, agg=0, ent=True, masked=0.0)
     out = run_head(R, c, group_tokens=group_tokens)
     compare_head(c, out)
 
 
 def test_fused_head_deterministic_and_workspace_independent(R):
-    """Two calls give the same bits (dH's split halves and dW's per-chunk additions land in a
-    fixed order); the smallest and a grouped workspace give the same loss and statistics bit
-    for bit (the products group their sums differently, so those are held to the oracle)."""
-    c = make_head_case(4096 + 300, 128, 2000, seed=8, agg=0)
+    """Two calls give the same bits (dW's per-chunk additions land in a fixed order); the
+    smallest workspace (two groups of one chunk) and a grouped one (one of two) give the same loss and
+    statistics bit for bit (the products group their sums differently, so those are held to the
+    oracle)."""
+    c = make_head_case(4096 + 300, 128, 2000, seed=8, agg=0, masked=0.0)
     a = run_head(R, c)
     b = run_head(R, c)
     g = run_head(R, c, group_tokens=8192)

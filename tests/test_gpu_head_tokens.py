@@ -67,11 +67,11 @@ def test_trained_token_counts(R, T, D, V, n, dh):
         assert out["loss"] == 0 and not out["dH"].any() and not out["dW"].any() and not out["stats"].any()
 
 
-@pytest.mark.parametrize("T,D,V", [(500, 128, 9000), (4200, 64, 520)])
-def test_workspaces_without_packing(R, T, D, V):
+@pytest.mark.parametrize("T,D,V,n", [(500, 128, 9000, 300), (4200, 64, 520, 4150)])
+def test_workspaces_without_packing(R, T, D, V, n):
     """The least workspace that is accepted takes every token through the products; one byte less is
-    refused; room for several packed chunks puts them in one group."""
-    c = case(T, D, V, T * 3 // 5, seed=T, ent=True)
+    refused; room for several packed chunks (4,150 trained tokens are two) puts them in one group."""
+    c = case(T, D, V, n, seed=T, ent=True)
     a = run(R, c, least_bytes(T, V))
     compare_head(c, a)
     with pytest.raises(R.RLError):
